@@ -1,19 +1,23 @@
 // Polarized Raman tail in float64 (Sec. II.G, Eqs. 7-8).
 //
-//   mean   per component of alpha(t) (or chi(t)), one CTA per component
-//   prep   x [9][T] channel-major, mean removed if asked
-//   corr   C_pq(tau) = sum_t x_p(t) x_q(t + tau), all 81 ordered pairs; one
-//          thread owns one pair and four consecutive lags and walks t in order
-//          (direct sums, used while 81 T M is small), or for long series
-//   fft    the symmetrised sums S_pq(tau) through the Fourier transform: the
-//          nine channels, zero-padded to N >= T + M (a power of two, so the
-//          circular correlation equals the linear one for tau <= M), are
-//          transformed (radix-2 Stockham, float64), the real cross spectra
-//          Re(conj(X_p) X_q) of the 45 pairs p <= q are transformed back two
-//          per complex transform, and S_pq(tau) = (1/N) IDFT[...](tau)
-//   cos    L_pq(nu_k) = dt [S_pq(0) + 2 sum_tau S_pq(tau) cos(pi k tau / M)],
-//          S_pq = (C_pq + C_qp) / (2 (T - tau)); one CTA per frequency, one
-//          warp per group of pairs
+//   sums   partial column sums of alpha(t) (or chi(t)), a fixed grid
+//   direct route (short series):
+//     prep   x [9][T] channel-major, mean removed if asked
+//     corr   C_pq(tau) = sum_t x_p(t) x_q(t + tau), all 81 ordered pairs; one
+//            thread owns one pair and four consecutive lags and walks t in order
+//     lags   S_pq(tau) = (C_pq + C_qp) / (2 (T - tau)), sequence-major
+//   Fourier route (rule at raman_uses_fft): segments of L = N/2 >= M samples,
+//   N a power of two, as in the spectrum tail (X_b, F_b defined there):
+//     prep   two channels per complex value, [5 packs][T], mean removed if asked
+//     fft    5 x (number of segments) transforms of length N
+//     (T = 1e5, M = 2000, tensor and 181-angle map: 6136 -> 844 us a call;
+//     before, one 2^17-point transform per channel and 23 back, and 4240 us of
+//     cosine sums that divided and took a 64-bit remainder in every term)
+//     cross  for the 45 pairs p <= q, sum over the segments b of
+//            conj(X_p) F_q + conj(X_q) F_p
+//     ifft   23 transforms, two pairs each; the real sequences are S_pq(tau)
+//   cos    L_pq(nu_k) = dt [S_pq(0) + 2 sum_tau S_pq(tau) cos(pi k tau / M)]
+//          (spectrum.cu)
 //   polar  spec_o(nu_k) = sum_pq w_p w_q L_pq(nu_k), w = vec(n_o eps_o^T) (Eq. 7)
 //   porto  the same for Z(XX)Z-bar / Z(XY)Z-bar of a crystal turned by theta
 // Every sum runs in a fixed order, so results do not depend on the launch.
@@ -23,39 +27,80 @@
 #include <utility>
 
 #include "engine.h"
+#include "fft.cuh"
 
 namespace tnep {
 
 namespace {
 
-constexpr double kCmPerInvFs = 1.0 / 2.99792458e-5;
 constexpr int kLagsPerThread = 4;
-// 81 T (M + 1) above which the correlations go through the Fourier transform
-constexpr double kFftAbove = 1.0e9;
 constexpr int kCorrThreads = 128;
+constexpr int kSumThreads = 288, kMaxSumBlocks = 128;  // 288 = 9 x 32: a thread keeps its column
+constexpr int kPacks = 5;
 
-__global__ void __launch_bounds__(1024) k_rmean(const double* __restrict__ s, int T, int subtract_mean,
-                                                double* __restrict__ mean) {
-  __shared__ double red[1024];
-  const int c = blockIdx.x;
-  double acc = 0.0;
-  if (subtract_mean)
-    for (int t = threadIdx.x; t < T; t += blockDim.x) acc += s[(size_t)t * 9 + c];
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = blockDim.x >> 1; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) mean[c] = red[0] / (double)T;
+// The direct sums cost 81 T (M + 1) multiply-adds of FP64 issue (2e7: 35 us and
+// more, one serial chain per lag), the Fourier route about a dozen launches.
+// Its error is uniform over the lags while S(tau) divides by T - tau, so lags
+// beyond T / 2 keep the direct sums until these cost milliseconds.
+bool raman_uses_fft(int T, int M) {
+  const double terms = 81.0 * (double)T * (double)(M + 1);
+  return terms > 1.0e9 || (terms > 2.0e7 && M <= T / 2);
 }
 
-__global__ void k_rprep(const double* __restrict__ s, int T, const double* __restrict__ mean,
-                        double* __restrict__ x) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 9LL * T) return;
-  const int t = (int)(i / 9), c = (int)(i % 9);
-  x[(size_t)c * T + t] = s[i] - mean[c];
+// Partial column sums of s [T][9], part[block][9].
+__global__ void __launch_bounds__(kSumThreads) k_rsum(const double* __restrict__ s, long long n,
+                                                      double* __restrict__ part) {
+  __shared__ double red[kSumThreads];
+  double acc = 0.0;
+  for (long long i = (long long)blockIdx.x * kSumThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kSumThreads)
+    acc += s[i];
+  red[threadIdx.x] = acc;
+  __syncthreads();
+  if (threadIdx.x < 72) {
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v += red[((threadIdx.x / 9) * 4 + k) * 9 + threadIdx.x % 9];
+    acc = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < 72) red[threadIdx.x] = acc;
+  __syncthreads();
+  if (threadIdx.x < 9) {
+    double v = 0.0;
+#pragma unroll
+    for (int h = 0; h < 8; ++h) v += red[h * 9 + threadIdx.x];
+    part[blockIdx.x * 9 + threadIdx.x] = v;
+  }
+}
+
+// PACK: z [pack][T], channels (0, 1) (2, 3) (4, 5) (6, 7) (8, -); else x [9][T].
+template <bool PACK>
+__global__ void __launch_bounds__(256) k_rprep(const double* __restrict__ s, int T, const double* __restrict__ part,
+                                               int n_part, int subtract_mean, double* __restrict__ out) {
+  __shared__ double mean[9];
+  const int lane = threadIdx.x & 31;
+  for (int c = threadIdx.x >> 5; c < 9; c += 8) {
+    double v = 0.0;
+    for (int b = lane; b < n_part; b += 32) v += part[b * 9 + c];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) mean[c] = subtract_mean ? v / (double)T : 0.0;
+  }
+  __syncthreads();
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= T) return;
+  double x[10];
+#pragma unroll
+  for (int c = 0; c < 9; ++c) x[c] = s[(size_t)t * 9 + c] - mean[c];
+  x[9] = 0.0;
+  if constexpr (PACK) {
+    double2* z = reinterpret_cast<double2*>(out) + t;
+#pragma unroll
+    for (int k = 0; k < kPacks; ++k) z[(size_t)k * T] = make_double2(x[2 * k], x[2 * k + 1]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 9; ++c) out[(size_t)c * T + t] = x[c];
+  }
 }
 
 // grid (lag tiles, 81 pairs); thread: lags tau0..tau0+3 of pair (p, q).
@@ -88,82 +133,141 @@ __global__ void __launch_bounds__(kCorrThreads) k_rcorr(const double* __restrict
     if (tau0 + j <= M) C[((size_t)(tau0 + j)) * 81 + pair] = acc[j];
 }
 
-// ---- Fourier route (float64 complex as double2) ----
-
-// Channel c of the mean-removed series, zero-padded to N, as complex.
-__global__ void k_fft_load(const double* __restrict__ x, int T, int N, double2* __restrict__ z) {
-  const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= 9LL * N) return;
-  const int c = (int)(g / N), t = (int)(g % N);
-  z[g] = make_double2(t < T ? x[(size_t)c * T + t] : 0.0, 0.0);
-}
-
-// Cross spectra of the 45 pairs p <= q, two per complex array:
-// z_w[f] = Re(conj(X_p) X_q)[f] + i Re(conj(X_p') X_q')[f].
-__global__ void k_fft_cross(const double2* __restrict__ X, int N, double2* __restrict__ z) {
-  const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= 23LL * N) return;
-  const int w = (int)(g / N), f = (int)(g % N);
-  double re[2] = {0.0, 0.0};
-  for (int h = 0; h < 2; ++h) {
-    const int u = 2 * w + h;
-    if (u >= 45) break;
-    int p = 0, rem = u;
-    while (rem >= 9 - p) { rem -= 9 - p; ++p; }
-    const int q = p + rem;
-    const double2 xp = X[(size_t)p * N + f], xq = X[(size_t)q * N + f];
-    re[h] = xp.x * xq.x + xp.y * xq.y;
-  }
-  z[g] = make_double2(re[0], re[1]);
-}
-
-// C[tau][81] (both p q and q p) = S_pq(tau): the inverse transform carries
-// no 1/N, so divide by N here.
-__global__ void k_fft_store(const double2* __restrict__ z, int N, int M, double* __restrict__ C) {
+// lags [45][M + 1] from the ordered pairs' sums C [M + 1][81].
+__global__ void k_rlags(const double* __restrict__ C, int T, int M, double* __restrict__ lags) {
   const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= 45LL * (M + 1)) return;
   const int u = (int)(g / (M + 1)), tau = (int)(g % (M + 1));
   int p = 0, rem = u;
   while (rem >= 9 - p) { rem -= 9 - p; ++p; }
   const int q = p + rem;
-  const double2 v = z[(size_t)(u >> 1) * N + tau];
-  const double sv = ((u & 1) ? v.y : v.x) / (double)N;
-  C[(size_t)tau * 81 + p * 9 + q] = sv;
-  C[(size_t)tau * 81 + q * 9 + p] = sv;
+  const double* c = C + (size_t)tau * 81;
+  lags[g] = 0.5 * (c[p * 9 + q] + c[q * 9 + p]) / (double)(T - tau);
 }
 
-__global__ void k_rcostab(int M, double* tab) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m < 2 * M) tab[m] = cospi((double)m / (double)M);
+// ---- Fourier route ----
+
+// Segment b of pack k (transform k nb + b): its L = N/2 samples, then zeros.
+struct LoadSegment {
+  const double2* z;
+  int T, nb, logN;
+  __device__ __forceinline__ double2 operator()(int f, unsigned i) const {
+    const int k = f / nb, b = f - k * nb;
+    const long long t = ((long long)b << (logN - 1)) + i;
+    if (i >= (1u << (logN - 1)) || t >= T) return make_double2(0.0, 0.0);
+    return __ldg(z + (size_t)k * T + t);
+  }
+};
+
+// First pair (p, p) of row p among the 45.
+__host__ __device__ constexpr int pair_row(int p) { return p * 9 - p * (p - 1) / 2; }
+
+// Rows of G: 0 = {0, 3}, 1 = {1, 2}, 2 = {4, 5, 6, 7, 8}: 15 pairs each, so that
+// the sums, the 9 transforms of this and of the next segment stay in registers.
+template <int G>
+__host__ __device__ constexpr bool has_row(int p) {
+  return G == 0 ? (p == 0 || p == 3) : (G == 1 ? (p == 1 || p == 2) : p >= 4);
 }
 
-// One CTA (8 warps) per frequency k; warp w handles the unique pairs
-// u = w, w + 8, ... of the 45 (p <= q).
-__global__ void __launch_bounds__(256) k_rcos(const double* __restrict__ C, const double* __restrict__ tab, int T,
-                                              int M, double dt, double* __restrict__ freq, double* __restrict__ L) {
-  const int k = blockIdx.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int u = warp; u < 45; u += 8) {
-    int p = 0, rem = u;
-    while (rem >= 9 - p) { rem -= 9 - p; ++p; }
-    const int q = p + rem;
-    double acc = 0.0;
-    for (int tau = 1 + lane; tau <= M; tau += 32) {
-      const double* c = C + (size_t)tau * 81;
-      const double s = 0.5 * (c[p * 9 + q] + c[q * 9 + p]) / (double)(T - tau);
-      acc = fma(s, tab[(long long)k * tau % (2LL * M)], acc);
+// part[chunk][45][N/2 + 1]: the pairs' spectra over segments [b0, b1), four
+// times the sums of the header.
+template <int G>
+__device__ __forceinline__ void cross_rows(const double2* __restrict__ z, int logN, int nb, int b0, int b1, unsigned f,
+                                           double2* __restrict__ part) {
+  constexpr int C0 = G == 2 ? 4 : (G == 1 ? 1 : 0);  // channels below are not read
+  const unsigned N = 1u << logN, half = N >> 1, g = (N - f) & (N - 1);
+  const double sgn = (f & 1u) ? -1.0 : 1.0;
+  auto load = [&](int b, double2* x) {
+#pragma unroll
+    for (int k = C0 / 2; k < kPacks; ++k) {
+      double2 u = make_double2(0.0, 0.0), v = u;
+      if (b < nb) {
+        const size_t o = ((size_t)k * nb + b) << logN;
+        u = z[o + f];
+        v = z[o + g];
+      }
+      x[2 * k] = make_double2(u.x + v.x, u.y - v.y);
+      if (k < kPacks - 1) x[2 * k + 1] = make_double2(u.y + v.y, v.x - u.x);
+    }
+  };
+  double2 x[9], nx[9], w[9];
+  double2 acc[45];
+#pragma unroll
+  for (int u = 0; u < 45; ++u) acc[u] = make_double2(0.0, 0.0);
+  load(b0, x);
+  for (int b = b0; b < b1; ++b) {
+    load(b + 1, nx);
+#pragma unroll
+    for (int c = C0; c < 9; ++c) w[c] = make_double2(fma(sgn, nx[c].x, x[c].x), fma(sgn, nx[c].y, x[c].y));
+#pragma unroll
+    for (int p = 0; p < 9; ++p) {
+      if (!has_row<G>(p)) continue;
+#pragma unroll
+      for (int q = p; q < 9; ++q) {
+        double2& a = acc[pair_row(p) + q - p];
+        a.x = fma(x[p].x, w[q].x, fma(x[p].y, w[q].y, a.x));
+        a.y = fma(x[p].x, w[q].y, fma(-x[p].y, w[q].x, a.y));
+        if (q != p) {
+          a.x = fma(x[q].x, w[p].x, fma(x[q].y, w[p].y, a.x));
+          a.y = fma(x[q].x, w[p].y, fma(-x[q].y, w[p].x, a.y));
+        }
+      }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) {
-      const double s0 = 0.5 * (C[p * 9 + q] + C[q * 9 + p]) / (double)T;
-      const double v = dt * (s0 + 2.0 * acc);
-      L[(size_t)k * 81 + p * 9 + q] = v;
-      L[(size_t)k * 81 + q * 9 + p] = v;
+    for (int c = C0; c < 9; ++c) x[c] = nx[c];
+  }
+#pragma unroll
+  for (int p = 0; p < 9; ++p) {
+    if (!has_row<G>(p)) continue;
+#pragma unroll
+    for (int q = p; q < 9; ++q) {
+      const int u = pair_row(p) + q - p;
+      part[(size_t)u * (half + 1) + f] = q == p ? fft::add(acc[u], acc[u]) : acc[u];
     }
   }
-  if (threadIdx.x == 0) freq[k] = (double)k / (2.0 * M * dt) * kCmPerInvFs;
 }
+
+// grid (frequency tiles, 3 row groups, chunks of segments).  FP64-bound: 8
+// multiply-adds per pair, frequency and segment.
+__global__ void __launch_bounds__(128) k_rcross(const double2* __restrict__ z, int logN, int nb, int per_chunk,
+                                                double2* __restrict__ part) {
+  const unsigned half = 1u << (logN - 1);
+  const unsigned f = blockIdx.x * blockDim.x + threadIdx.x;
+  if (f > half) return;
+  const int b0 = blockIdx.z * per_chunk, b1 = min(nb, b0 + per_chunk);
+  double2* dst = part + (size_t)blockIdx.z * 45 * (half + 1);
+  if (blockIdx.y == 0) cross_rows<0>(z, logN, nb, b0, b1, f, dst);
+  else if (blockIdx.y == 1) cross_rows<1>(z, logN, nb, b0, b1, f, dst);
+  else cross_rows<2>(z, logN, nb, b0, b1, f, dst);
+}
+
+// Pairs 2f and 2f + 1 (spectra of real sequences) as one complex spectrum,
+// the chunks summed in order.
+struct LoadCross {
+  const double2* part;
+  int chunks, logN;
+  __device__ __forceinline__ double2 operator()(int f, unsigned i) const {
+    const unsigned N = 1u << logN, half = N >> 1, g = i <= half ? i : N - i;
+    double2 u = make_double2(0.0, 0.0), v = u;
+    for (int c = 0; c < chunks; ++c) {
+      const double2* s = part + ((size_t)c * 45 + 2 * f) * (half + 1) + g;
+      u = fft::add(u, s[0]);
+      if (2 * f + 1 < 45) v = fft::add(v, s[half + 1]);
+    }
+    return i <= half ? make_double2(u.x - v.y, u.y + v.x) : make_double2(u.x + v.y, v.x - u.y);
+  }
+};
+struct StoreLags {
+  double* lags;  // [45][M + 1]
+  int T, M;
+  double scale;  // 1 / (8 N)
+  __device__ __forceinline__ void operator()(int f, unsigned i, double2 v) const {
+    if (i > (unsigned)M) return;
+    const double s = scale / (double)(T - (int)i);
+    lags[(size_t)(2 * f) * (M + 1) + i] = v.x * s;
+    if (2 * f + 1 < 45) lags[(size_t)(2 * f + 1) * (M + 1) + i] = v.y * s;
+  }
+};
 
 __device__ __forceinline__ double contract(const double* __restrict__ Lk, const double w[9]) {
   double acc = 0.0;
@@ -244,49 +348,65 @@ tnep_status tnep_raman_tensor(const double* series, int T, double dt_fs, int max
   if (M < 1 || M >= T) return fail(TNEP_ERR_INVALID, "max_lag must be in [1, T)");
   if (!have_device()) return fail(TNEP_ERR_NO_DEVICE, "no CUDA device");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const size_t nS = (size_t)T * 9, nX = (size_t)T * 9, nC = (size_t)(M + 1) * 81, nT = 2 * (size_t)M;
-  const size_t nF = (size_t)(M + 1), nL = (size_t)(M + 1) * 81;
-  // direct time-origin sums while they are cheap, the Fourier route beyond
-  const bool use_fft = 81.0 * (double)T * (double)(M + 1) > kFftAbove;
-  int N = 2;
-  while (N < T + M) N <<= 1;
-  const size_t nZ = use_fft ? (size_t)2 * 23 * N + (size_t)N / 2 : 0;  // double2: two work arrays + twiddles
-  double* d = nullptr;
-  TNEP_CUDA(dev_malloc_async((void**)&d, sizeof(double) * (nS + nX + nC + nT + nF + nL + 16 + 2 * nZ), st));
-  // the FFT work area (double2) first, where the allocation's alignment holds
-  double2* zwork = reinterpret_cast<double2*>(d);
-  double* d_s = d + 2 * nZ;
-  double* d_x = d_s + nS;
-  double* d_c = d_x + nX;
-  double* d_tab = d_c + nC;
-  double* d_f = d_tab + nT;
-  double* d_l = d_f + nF;
-  double* d_mean = d_l + nL;
-  cudaError_t e = cudaMemcpyAsync(d_s, series, sizeof(double) * nS, cudaMemcpyDefault, st);
+  const bool use_fft = raman_uses_fft(T, M);
+  const int logN = fft::log2_at_least(2LL * M);
+  const int nb = (int)(((long long)T + (1ll << (logN - 1)) - 1) >> (logN - 1));
+  const unsigned half = 1u << (logN - 1);
+  // chunks of segments: enough (frequency, row group, chunk) threads to fill the chip
+  int chunks = (int)std::min<long long>(nb, std::max<long long>(1, (1ll << 15) >> (logN - 1)));
+  const int per_chunk = (nb + chunks - 1) / chunks;
+  chunks = (nb + per_chunk - 1) / per_chunk;
+  const int n_part = (int)std::min<long long>(kMaxSumBlocks, (9LL * T + 4 * kSumThreads - 1) / (4 * kSumThreads));
+  size_t at = 0;
+  auto place = [&](size_t bytes) {
+    const size_t o = at;
+    at += (bytes + 255) & ~size_t(255);
+    return o;
+  };
+  const size_t nF = (size_t)(M + 1), nL = (size_t)(M + 1) * 81, nZ = (size_t)std::max(kPacks * nb, 23) << logN;
+  const size_t o_s = place(sizeof(double) * 9 * (size_t)T), o_part = place(sizeof(double) * 9 * n_part);
+  const size_t o_x = place(sizeof(double) * (use_fft ? 2 * kPacks : 9) * (size_t)T);
+  const size_t o_a = place(use_fft ? sizeof(double2) * nZ : sizeof(double) * nL);
+  const size_t o_b = place(use_fft ? sizeof(double2) * nZ : 0);
+  const size_t o_tw = place(use_fft ? sizeof(double2) * fft::table_size(logN) : 0);
+  const size_t o_cross = place(use_fft ? sizeof(double2) * 45 * chunks * (size_t)(half + 1) : 0);
+  const size_t o_lags = place(sizeof(double) * 45 * nF), o_f = place(sizeof(double) * nF);
+  const size_t o_l = place(sizeof(double) * nL), o_cos = place(cosine_work_bytes(M, 45));
+  char* d = nullptr;
+  TNEP_CUDA(dev_malloc_async((void**)&d, at, st));
+  auto dbl = [&](size_t o) { return reinterpret_cast<double*>(d + o); };
+  double *d_s = dbl(o_s), *d_part = dbl(o_part), *d_x = dbl(o_x), *d_lags = dbl(o_lags), *d_f = dbl(o_f), *d_l = dbl(o_l);
+  cudaError_t e = cudaMemcpyAsync(d_s, series, sizeof(double) * 9 * (size_t)T, cudaMemcpyDefault, st);
   if (e == cudaSuccess) {
-    k_rmean<<<9, 1024, 0, st>>>(d_s, T, subtract_mean, d_mean);
-    k_rprep<<<blocks_for(9LL * T, 256), 256, 0, st>>>(d_s, T, d_mean, d_x);
+    k_rsum<<<n_part, kSumThreads, 0, st>>>(d_s, 9LL * T, d_part);
+    count_launches(3);
     if (!use_fft) {
+      double* d_c = dbl(o_a);
+      k_rprep<false><<<blocks_for(T, 256), 256, 0, st>>>(d_s, T, d_part, n_part, subtract_mean, d_x);
       const int tiles = (M + 1 + kCorrThreads * kLagsPerThread - 1) / (kCorrThreads * kLagsPerThread);
       k_rcorr<<<dim3(tiles, 81), kCorrThreads, 0, st>>>(d_x, T, M, d_c);
+      k_rlags<<<blocks_for(45LL * (M + 1), 256), 256, 0, st>>>(d_c, T, M, d_lags);
       count_launches(1);
+      e = cudaGetLastError();
     } else {
-      double2* za = zwork;
-      double2* zb = za + (size_t)23 * N;
-      double2* tw = zb + (size_t)23 * N;
-      launch_fft_twiddles(N, tw, st);
-      k_fft_load<<<blocks_for(9LL * N, 256), 256, 0, st>>>(d_x, T, N, za);
-      launch_fft(&za, &zb, tw, N, 9, 0, st);
-      k_fft_cross<<<blocks_for(23LL * N, 256), 256, 0, st>>>(za, N, zb);
-      std::swap(za, zb);
-      launch_fft(&za, &zb, tw, N, 23, 1, st);
-      k_fft_store<<<blocks_for(45LL * (M + 1), 256), 256, 0, st>>>(za, N, M, d_c);
-      count_launches(3);
+      double2 *za = reinterpret_cast<double2*>(d + o_a), *zb = reinterpret_cast<double2*>(d + o_b);
+      double2* tw = reinterpret_cast<double2*>(d + o_tw);
+      double2 *zx = reinterpret_cast<double2*>(d_x), *cross = reinterpret_cast<double2*>(d + o_cross);
+      k_rprep<true><<<blocks_for(T, 256), 256, 0, st>>>(d_s, T, d_part, n_part, subtract_mean, d_x);
+      e = launch_fft_table(logN, tw, st);
+      double2* fin = fft::last_source(logN) == 0 ? zb : za;
+      if (e == cudaSuccess)
+        e = fft::transform<false>(LoadSegment{zx, T, nb, logN}, fft::StorePlain{fin, logN}, za, zb, tw, logN,
+                                  kPacks * nb, st);
+      if (e == cudaSuccess) {
+        k_rcross<<<dim3((half + 1 + 127) / 128, 3, chunks), 128, 0, st>>>(fin, logN, nb, per_chunk, cross);
+        e = fft::transform<true>(LoadCross{cross, chunks, logN},
+                                 StoreLags{d_lags, T, M, 1.0 / (8.0 * (double)(1ll << logN))}, za, zb, tw, logN,
+                                 23, st);
+      }
     }
-    k_rcostab<<<blocks_for(2LL * M, 256), 256, 0, st>>>(M, d_tab);
-    k_rcos<<<M + 1, 256, 0, st>>>(d_c, d_tab, T, M, dt_fs, d_f, d_l);
-    count_launches(4);
-    e = cudaGetLastError();
+    if (e == cudaSuccess)
+      e = launch_cosine(d_lags, M, 45, CosineOut{1, 0, dt_fs, d_f, d_l}, nullptr, d + o_cos, st);
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(freq_cm1, d_f, sizeof(double) * nF, cudaMemcpyDefault, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(L, d_l, sizeof(double) * nL, cudaMemcpyDefault, st);

@@ -15,8 +15,10 @@
 namespace {
 
 constexpr int kNoallocMaxT = TNEP_NOALLOC_MAX_T;
-// signal [T][9] + acf [M+1] + cosine table [2M], with M < T
-constexpr size_t kNoallocWords = (size_t)kNoallocMaxT * 9 + (size_t)kNoallocMaxT + 2 * (size_t)kNoallocMaxT;
+// acf [M+1], then the direct route's work area: column sums, cosine table [2M]
+// and signal [T][9], with M < T (each part rounded up to 256 bytes)
+constexpr size_t kNoallocAcf = (size_t)kNoallocMaxT;
+constexpr size_t kNoallocWords = kNoallocAcf + 2 * (size_t)kNoallocMaxT + (size_t)kNoallocMaxT * 9 + 2048;
 
 static __device__ __align__(256) double g_spectrum_scratch[kNoallocWords];
 
@@ -88,8 +90,8 @@ extern "C" tnep_status tnep_spectrum_noalloc(const double* series, int T, int C,
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   // Every scratch element the kernels read is written earlier in the same
   // call, so nothing left by the previous call needs clearing.
-  cudaError_t e = tnep::launch_spectrum(series, T, C, dt_fs, kind, M, subtract_mean, scratch, freq_cm1, spec,
-                                        acf_out, st);
+  cudaError_t e = tnep::launch_spectrum(series, T, C, dt_fs, kind, M, subtract_mean, false, false,
+                                        scratch + kNoallocAcf, freq_cm1, spec, acf_out ? acf_out : scratch, st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return noalloc_fail(TNEP_ERR_CUDA, cudaGetErrorString(e));

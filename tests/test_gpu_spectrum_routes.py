@@ -1,0 +1,92 @@
+"""Both routes of the spectrum and polarized Raman tails at the edges of their
+rules, against the plain float64 definition.
+
+Reference: time-origin averages by numpy's FFT of the zero-padded series and
+the cosine transform by numpy's real FFT of the even extension.  Tolerance: a
+float64 transform of length N is accurate to a few eps log2(N) of the root
+sum of squares, about 1e-15 of the correlation at lag 0; divided by T - tau >=
+T / 2 and summed over M lags this stays below 1e-12 of the largest value
+(omega^2 weights are relative to the same maximum)."""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+REL = 1e-12
+
+
+@pytest.fixture(scope="module")
+def tn():
+    from paper_2312_05233_gb300 import tnep
+    return tnep
+
+
+def series(T, C, seed):
+    rng = np.random.default_rng(seed)
+    t = np.arange(T)[:, None]
+    return (rng.standard_normal((1, C)) + 0.1 * np.cos(0.05 * t + rng.uniform(0, 6, (1, C)))
+            + 0.05 * rng.standard_normal((T, C)))
+
+
+def correlate(x, y, M):
+    N = 1 << (len(x) + M).bit_length()
+    return np.fft.irfft(np.conj(np.fft.rfft(x, N)) * np.fft.rfft(y, N), N)[:M + 1] / (len(x) - np.arange(M + 1))
+
+
+def cosine(c, dt):
+    return dt * np.fft.rfft(np.concatenate([c[:-1], 2 * c[-1:], c[1:-1][::-1]])).real
+
+
+def close(got, ref):
+    np.testing.assert_allclose(got, ref, rtol=0, atol=REL * np.abs(ref).max())
+
+
+# (T, M): direct below 2e7 terms, segments of 2^7 .. 2^16 samples above, M at,
+# below and above a segment's length, lags beyond T / 2, one segment, and the
+# cosine transform on both sides of its rule (M = 4000)
+SIZES = [(2, 1), (3, 2), (37, 18), (400, 399), (5000, 2500), (60000, 128), (60000, 129), (60001, 127), (30000, 1024),
+         (30000, 1023), (30000, 1025), (40000, 3999), (40000, 4000), (40000, 4001), (16384, 8192), (100000, 33000),
+         (20000, 12000), (70000, 60000)]
+
+
+@pytest.mark.parametrize("T,M", SIZES)
+@pytest.mark.parametrize("kind", ["ir", "iso", "aniso"])
+def test_spectrum_routes(tn, T, M, kind):
+    code = {"ir": tn.TNEP_SPECTRUM_IR, "iso": tn.TNEP_SPECTRUM_RAMAN_ISO, "aniso": tn.TNEP_SPECTRUM_RAMAN_ANISO}[kind]
+    s = series(T, 3 if kind == "ir" else 9, T + M)
+    x = s
+    if kind != "ir":
+        g = (s[:, 0] + s[:, 4] + s[:, 8])[:, None] / 3
+        x = g if kind == "iso" else s - g * np.eye(3).reshape(1, 9)
+    x = x - x.mean(0)
+    w = x.shape[1]
+    pairs = [(c, (c % 3) * 3 + c // 3) for c in range(9)] if kind == "aniso" else [(c, c) for c in range(w)]
+    acf = sum(correlate(x[:, p], x[:, q], M) for p, q in pairs) / (3 if kind == "ir" else 1)
+    ref = cosine(acf, 0.5)
+    nu = np.arange(M + 1) / (2 * M * 0.5)
+    if kind == "ir":
+        ref = ref * (2 * np.pi * nu) ** 2
+    f, S, a = tn.tnep_spectrum(s, 0.5, code, M, want_acf=True)
+    if M <= T // 2:
+        close(a, acf)
+        close(S, ref)
+    else:  # few terms per lag at the end: the reference itself is good to eps T / (T - tau)
+        np.testing.assert_allclose(a, acf, rtol=0, atol=REL * T / (T - M) * np.abs(acf).max())
+        np.testing.assert_allclose(S, ref, rtol=0, atol=REL * T / (T - M) * np.abs(ref).max())
+    np.testing.assert_allclose(f, nu / 2.99792458e-5, rtol=1e-14)
+
+
+@pytest.mark.parametrize("T,M", [(2, 1), (50, 49), (300, 150), (4000, 128), (4001, 129), (9000, 700), (3000, 1500),
+                                 (20000, 256), (6000, 4096), (30000, 2048)])
+def test_raman_tensor_routes(tn, T, M):
+    s = series(T, 9, T * 3 + M)
+    x = s - s.mean(0)
+    f, L = tn.tnep_raman_tensor(s, 2.0, M)
+    slack = 1.0 if M <= T // 2 else T / (T - M)
+    ref = np.zeros((M + 1, 9, 9))
+    for p in range(9):
+        for q in range(p, 9):
+            c = 0.5 * (correlate(x[:, p], x[:, q], M) + correlate(x[:, q], x[:, p], M))
+            ref[:, p, q] = ref[:, q, p] = cosine(c, 2.0)
+    np.testing.assert_allclose(L, ref, rtol=0, atol=slack * REL * np.abs(ref).max())
+    np.testing.assert_allclose(f, np.arange(M + 1) / (2 * M * 2.0) / 2.99792458e-5, rtol=1e-14)
