@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -18,6 +19,10 @@
 #include "engine.h"
 
 using namespace tnep;
+
+namespace {
+std::atomic<int> g_contexts{0};
+}
 
 extern "C" {
 
@@ -46,6 +51,7 @@ tnep_status tnep_create(const tnep_model_desc* models, int n_models, int n_types
   TNEP_CUDA(cudaSetDevice(device));
   tnep_ctx* c = new (std::nothrow) tnep_ctx();
   if (!c) return fail(TNEP_ERR_OOM, "host allocation failed");
+  g_contexts.fetch_add(1);
   c->device = device;
   c->n_types = n_types;
   c->rc_R = cutoffs[0];
@@ -133,6 +139,7 @@ void tnep_destroy(tnep_ctx* c) {
   if (c->ev_fused) cudaEventDestroy(c->ev_fused);
   if (c->ev_reduced) cudaEventDestroy(c->ev_reduced);
   delete c;
+  if (g_contexts.fetch_sub(1) == 1) trim_pools();
 }
 
 int tnep_output_dim(const tnep_ctx* c, int model) {

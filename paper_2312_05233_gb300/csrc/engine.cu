@@ -21,6 +21,33 @@ std::atomic<long long> g_allocs{0};
 long long g_fault_at = 0;  // 0 = no injected failure
 std::once_flag g_fault_once;
 
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mutex;
+cudaMemPool_t g_pools[kMaxDevices] = {nullptr};
+
+// The library's pool of device `dev`, made on first use; null when the device
+// has none (the caller then takes the runtime's).
+cudaMemPool_t pool_of(int dev) {
+  if (dev < 0 || dev >= kMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  if (!g_pools[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    unsigned long long keep = tnep::kPoolKeepBytes;
+    if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
+    g_pools[dev] = p;
+  }
+  return g_pools[dev];
+}
+
 // True if this allocation is the one TNEP_FAULT=oom@N asks to fail.
 bool injected_oom() {
   std::call_once(g_fault_once, [] {
@@ -38,13 +65,29 @@ namespace tnep {
 cudaError_t dev_malloc(void** p, size_t bytes) {
   *p = nullptr;
   if (injected_oom()) return cudaErrorMemoryAllocation;
-  return cudaMalloc(p, bytes);
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {  // give back what the pools keep and try once more
+    cudaGetLastError();
+    trim_pools();
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
 }
 
 cudaError_t dev_malloc_async(void** p, size_t bytes, cudaStream_t st) {
   *p = nullptr;
   if (injected_oom()) return cudaErrorMemoryAllocation;
-  return cudaMallocAsync(p, bytes, st);
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const cudaMemPool_t pool = pool_of(dev);
+  return pool ? cudaMallocFromPoolAsync(p, bytes, pool, st) : cudaMallocAsync(p, bytes, st);
+}
+
+void trim_pools() {
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  for (cudaMemPool_t p : g_pools)
+    if (p && cudaMemPoolTrimTo(p, 0) != cudaSuccess) cudaGetLastError();
 }
 
 cudaError_t host_alloc(void** p, size_t bytes) {

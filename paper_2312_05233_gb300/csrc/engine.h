@@ -37,7 +37,14 @@ tnep_status cuda_fail(cudaError_t e, const char* what);
 // allocated and the device is not touched), so callers can check that every
 // entry point returns TNEP_ERR_OOM and that the context stays usable.
 cudaError_t dev_malloc(void** p, size_t bytes);
+// Stream-ordered scratch of one call, from a pool of this library per device
+// that keeps up to kPoolKeepBytes between calls (the runtime's default pool
+// gives everything back at each synchronisation, and mapping it again cost
+// about 200 us a call); freed with cudaFreeAsync.  The pool is trimmed when an
+// allocation does not fit and when the last context goes.
+constexpr size_t kPoolKeepBytes = size_t(256) << 20;
 cudaError_t dev_malloc_async(void** p, size_t bytes, cudaStream_t st);
+void trim_pools();
 cudaError_t host_alloc(void** p, size_t bytes);
 long long alloc_count();
 
