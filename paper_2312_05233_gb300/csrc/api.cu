@@ -230,7 +230,6 @@ tnep_status tnep_eval(tnep_ctx* c, int n_frames, int n_atoms, const float* pos, 
   if (n_atoms >= kMaxBatchAtoms) return fail(TNEP_ERR_INVALID, "a frame must hold fewer than 2^29 atoms");
   fb = std::max(1, std::min(fb, (kMaxBatchAtoms - 1) / std::max(n_atoms, 1)));
   const bool pos_dev = is_device_ptr(pos);
-  const bool box_dev = box && is_device_ptr(box);
   const bool out_dev = is_device_ptr(out);
   const int* d_types = nullptr;
   TNEP_TRY(stage_in(types, (size_t)n_atoms, c->ws.types_stage, &d_types, st));
@@ -240,9 +239,13 @@ tnep_status tnep_eval(tnep_ctx* c, int n_frames, int n_atoms, const float* pos, 
     for (int a = 0; a < n_atoms; ++a)
       if (types[a] < 0 || types[a] >= c->n_types) return fail(TNEP_ERR_INVALID, "type index out of range");
   const float* d_box_all = nullptr;
-  if (box) TNEP_TRY(stage_in(box, (size_t)3 * n_frames, c->ws.box_stage, &d_box_all, st));
+  if (box) {
+    if (c->skin > 0.f) TNEP_TRY(stage_in(box, (size_t)3 * n_frames, c->ws.box_stage, &d_box_all, st));
+    else TNEP_TRY(stage_box(c->ws, box, n_frames, &d_box_all));
+  }
   if (!out_dev) TNEP_CUDA(c->h_out.ensure((size_t)n_frames * Ctot));
   std::vector<int> offs(fb + 1);
+  const cudaStream_t red = n_frames > fb ? c->red_stream : nullptr;
   // Verlet-skin reuse needs one box for the whole pass and n_atoms > 0; any
   // violation found on the device (displacement above skin / 2, changed box,
   // box too small for the enlarged cutoff) redoes the call with fresh lists
@@ -278,21 +281,21 @@ tnep_status tnep_eval(tnep_ctx* c, int n_frames, int n_atoms, const float* pos, 
         TNEP_TRY(build_lists(c, c->ws, st, nf, offs.data(), d_pos, d_box, d_types, n_atoms));
       if (!pos_dev && n_atoms > 0) TNEP_CUDA(cudaEventRecord(c->ev_consumed[b & 1], st));
       TNEP_CUDA(cudaEventRecord(ev[1], st));
-      // the pass's per-frame sums and their copy-out run on the side stream,
-      // overlapping the next pass's cell lists and neighbour build
-      TNEP_TRY(run_models(c, c->ws, st, nf, nf * n_atoms, ev[2], nullptr, c->red_stream));
+      // with several passes, a pass's per-frame sums and their copy-out run on
+      // the side stream, overlapping the next pass's cell lists and neighbour build
+      TNEP_TRY(run_models(c, c->ws, st, nf, nf * n_atoms, ev[2], nullptr, red));
       // scatter results: model m block [n_frames][C_m]
       size_t src_off = 0, dst_base = 0;
       for (const auto& m : c->models) {
         double* dst = out_dev ? out : c->h_out.p;
         TNEP_TRY(copy_out(dst + dst_base + (size_t)f0 * m.C, c->ws.out.p + src_off, (size_t)nf * m.C,
-                          c->red_stream));
+                          red ? red : st));
         src_off += (size_t)nf * m.C;
         dst_base += (size_t)n_frames * m.C;
       }
-      TNEP_CUDA(cudaEventRecord(c->ev_reduced, c->red_stream));
+      if (red) TNEP_CUDA(cudaEventRecord(c->ev_reduced, red));
     }
-    TNEP_CUDA(cudaStreamWaitEvent(st, c->ev_reduced, 0));
+    if (red) TNEP_CUDA(cudaStreamWaitEvent(st, c->ev_reduced, 0));
     if (use_skin) {
       TNEP_CUDA(cudaMemcpyAsync(c->skin_ws.h_status.p, c->skin_ws.d_status, sizeof(DevStatus),
                                 cudaMemcpyDeviceToHost, st));
@@ -347,7 +350,7 @@ tnep_status tnep_eval_batch(tnep_ctx* c, int n_structs, const int* atom_offsets,
   const float* d_box = nullptr;
   TNEP_TRY(stage_in(pos, (size_t)N * 3, c->ws.pos_stage[0], &d_pos, st));
   TNEP_TRY(stage_in(types, (size_t)N, c->ws.types_stage, &d_types, st));
-  if (box) TNEP_TRY(stage_in(box, (size_t)n_structs * 3, c->ws.box_stage, &d_box, st));
+  if (box) TNEP_TRY(stage_box(c->ws, box, n_structs, &d_box));
   const int Ctot = total_C(c);
   for (int attempt = 0; attempt < 4; ++attempt) {
     TNEP_TRY(reset_status(c->ws, st));
@@ -410,7 +413,7 @@ tnep_status tnep_neighbors(tnep_ctx* c, int n_structs, const int* atom_offsets, 
   const float* d_pos = nullptr;
   const float* d_box = nullptr;
   TNEP_TRY(stage_in(pos, (size_t)N * 3, c->ws.pos_stage[0], &d_pos, st));
-  if (box) TNEP_TRY(stage_in(box, (size_t)n_structs * 3, c->ws.box_stage, &d_box, st));
+  if (box) TNEP_TRY(stage_box(c->ws, box, n_structs, &d_box));
   DevBuf<int> zeros;
   TNEP_CUDA(zeros.ensure(1));
   TNEP_CUDA(cudaMemsetAsync(zeros.p, 0, sizeof(int), st));
@@ -481,7 +484,7 @@ tnep_status tnep_eval_population(tnep_ctx* c, int model, int n_pop, const float*
   const double* d_target = nullptr;
   TNEP_TRY(stage_in(pos, (size_t)N * 3, c->ws.pos_stage[0], &d_pos, st));
   TNEP_TRY(stage_in(types, (size_t)N, c->ws.types_stage, &d_types, st));
-  if (box) TNEP_TRY(stage_in(box, (size_t)n_structs * 3, c->ws.box_stage, &d_box, st));
+  if (box) TNEP_TRY(stage_box(c->ws, box, n_structs, &d_box));
   TNEP_TRY(stage_in(target, (size_t)n_structs * m.C, c->pop_target, &d_target, st));
   for (int attempt = 0; attempt < 4; ++attempt) {
     TNEP_TRY(reset_status(c->ws, st));
@@ -504,7 +507,7 @@ tnep_status tnep_eval_population(tnep_ctx* c, int model, int n_pop, const float*
     TNEP_TRY(pass_events(c, 0, &ev));
     TNEP_CUDA(launch_fused(m.variant, m.d.rank, f, n_pop, c->block_atoms, m.d.mlp_precision, st));
     TNEP_CUDA(cudaEventRecord(ev[2], st));
-    TNEP_CUDA(w.partial.ensure((size_t)n_pop * n_structs * reduce_chunks(w.max_atoms) * m.C));
+    TNEP_CUDA(w.partial.ensure((size_t)n_pop * n_structs * reduce_chunks(w.max_atoms) * 9));
     TNEP_CUDA(launch_reduce(n_structs, n_pop, w.offsets.p, w.max_atoms, w.per_atom.p, pa_pop, w.atom_stride, m.C,
                             w.partial.p, w.out.p, (size_t)n_structs * m.C, st));
     TNEP_CUDA(launch_rmse(n_pop, n_structs, m.C, w.out.p, d_target, c->pop_rmse.p, st));

@@ -214,7 +214,7 @@ tnep_status ensure_batch(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, cons
   for (int s = 0; s < S; ++s) mx = std::max(mx, h_offsets[s + 1] - h_offsets[s]);
   w.max_atoms = mx;
   w.atom_stride = stride;
-  w.cells_cap = 2 * N + 8 * S;
+  w.cells_cap = 2 * N + 9 * S;  // small structures take a private range of 2 n + 9
   w.cap_R = cap_R;
   w.cap_A = cap_A;
   TNEP_CUDA(w.offsets.ensure(S + 1));
@@ -238,7 +238,44 @@ tnep_status ensure_batch(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, cons
   TNEP_CUDA(w.nbr_tmp.ensure((size_t)stride * w.cap_R));
   TNEP_CUDA(w.nbr_A.ensure((size_t)stride * w.cap_A));
   TNEP_CUDA(w.seg_R.ensure((size_t)stride * c->n_types));
-  TNEP_CUDA(cudaMemcpyAsync(w.offsets.p, h_offsets, sizeof(int) * (S + 1), cudaMemcpyHostToDevice, st));
+  if (!w.ev_pin) TNEP_CUDA(cudaEventCreateWithFlags(&w.ev_pin, cudaEventDisableTiming));
+  // A trajectory's later passes have a prefix of the first one's offsets,
+  // which its kernels may still be reading.
+  if (w.h_offsets.n < (size_t)S + 1 || !std::equal(h_offsets, h_offsets + S + 1, w.h_offsets.p)) {
+    TNEP_TRY(pin_wait(w));
+    TNEP_CUDA(w.h_offsets.ensure(S + 1));
+    std::copy(h_offsets, h_offsets + S + 1, w.h_offsets.p);
+  }
+  return TNEP_OK;
+}
+
+tnep_status pin_wait(Workspace& w) {
+  if (!w.pin_read) return TNEP_OK;
+  TNEP_CUDA(cudaEventSynchronize(w.ev_pin));
+  w.pin_read = false;
+  return TNEP_OK;
+}
+
+tnep_status pin_mark(Workspace& w, cudaStream_t st) {
+  w.pin_read = true;
+  TNEP_CUDA(cudaEventRecord(w.ev_pin, st));
+  return TNEP_OK;
+}
+
+tnep_status stage_box(Workspace& w, const float* box, int n, const float** dev) {
+  *dev = box;
+  if (!box || is_device_ptr(box)) return TNEP_OK;
+  TNEP_TRY(pin_wait(w));
+  TNEP_CUDA(w.h_box.ensure((size_t)3 * n));
+  std::copy(box, box + (size_t)3 * n, w.h_box.p);
+  *dev = w.h_box.p;
+  return TNEP_OK;
+}
+
+// Offsets on the device for the kernels of a batch whose preparation does not
+// copy them itself.
+tnep_status copy_offsets(Workspace& w, cudaStream_t st, int S) {
+  TNEP_CUDA(cudaMemcpyAsync(w.offsets.p, w.h_offsets.p, sizeof(int) * (S + 1), cudaMemcpyHostToDevice, st));
   return TNEP_OK;
 }
 
@@ -247,12 +284,18 @@ tnep_status build_lists(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, const
   const float rc_R = spec ? spec->rc_R : c->rc_R, rc_A = spec ? spec->rc_A : c->rc_A;
   TNEP_TRY(ensure_batch(c, w, st, S, h_offsets, spec ? spec->cap_R : c->cap_R, spec ? spec->cap_A : c->cap_A));
   const int N = h_offsets[S];
-  TNEP_CUDA(cudaMemsetAsync(w.cell_count.p, 0, sizeof(int) * (w.cells_cap + 1), st));
-  TNEP_CUDA(cudaMemsetAsync(w.struct_flags.p, 0, sizeof(int) * S, st));
+  if (w.max_atoms > kSmallStruct) {
+    TNEP_TRY(copy_offsets(w, st, S));
+    TNEP_CUDA(cudaMemsetAsync(w.cell_count.p, 0, sizeof(int) * (w.cells_cap + 1), st));
+    TNEP_CUDA(cudaMemsetAsync(w.struct_flags.p, 0, sizeof(int) * S, st));
+  }
   NbrArgs a{};
   a.n_structs = S;
   a.n_atoms = N;
+  a.max_struct = w.max_atoms;
   a.offsets = w.offsets.p;
+  a.src_offsets = w.h_offsets.p;
+  a.offsets_out = w.offsets.p;
   a.pos = d_pos;
   a.box = d_box;
   a.types = d_types;
@@ -290,6 +333,7 @@ tnep_status build_lists(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, const
   a.cells_cap = w.cells_cap;
   a.status = w.d_status;
   TNEP_CUDA(launch_neighbor_pipeline(a, st));
+  TNEP_TRY(pin_mark(w, st));
   return TNEP_OK;
 }
 
@@ -305,6 +349,7 @@ tnep_status skin_lists(tnep_ctx* c, Workspace& w, Workspace& sw, cudaStream_t st
   std::vector<int> offs(nf + 1);
   for (int k = 0; k <= nf; ++k) offs[k] = k * N;
   TNEP_TRY(ensure_batch(c, w, st, nf, offs.data(), c->cap_R, c->cap_A));
+  TNEP_TRY(copy_offsets(w, st, nf));
   SkinArgs a{};
   a.nf = nf;
   a.N = N;
@@ -339,6 +384,7 @@ tnep_status skin_lists(tnep_ctx* c, Workspace& w, Workspace& sw, cudaStream_t st
   a.status = w.d_status;
   w.two_ended = 0;  // the compacted lists are front-packed per type
   TNEP_CUDA(launch_skin_compact(a, st));
+  TNEP_TRY(pin_mark(w, st));
   return TNEP_OK;
 }
 
@@ -474,20 +520,20 @@ tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N,
     for (size_t k = 0; k < c->models.size(); ++k)
       TNEP_CUDA(launch_zero_ghosts(N, w.sorted_orig.p, ghost, w.per_atom.p + k * per_model, w.atom_stride,
                                    c->models[k].C, st));
-  TNEP_CUDA(w.partial.ensure((size_t)std::max(S, 1) * reduce_chunks(w.max_atoms) * 9));
+  TNEP_CUDA(w.partial.ensure((size_t)std::max(S, 1) * reduce_chunks(w.max_atoms) * 9 * c->models.size()));
   cudaStream_t rs = st;
   if (red_st) {
     TNEP_CUDA(cudaEventRecord(c->ev_fused, st));
     TNEP_CUDA(cudaStreamWaitEvent(red_st, c->ev_fused, 0));
     rs = red_st;
   }
+  std::vector<ReduceModel> rm;
   size_t off = 0;
   for (size_t k = 0; k < c->models.size(); ++k) {
-    const Model& m = c->models[k];
-    TNEP_CUDA(launch_reduce(S, 1, offsets, w.max_atoms, w.per_atom.p + k * per_model, 0, w.atom_stride, m.C,
-                            w.partial.p, w.out.p + off, 0, rs));
-    off += (size_t)S * m.C;
+    rm.push_back({w.per_atom.p + k * per_model, w.out.p + off, c->models[k].C});
+    off += (size_t)S * c->models[k].C;
   }
+  TNEP_CUDA(launch_reduce_models(S, (int)rm.size(), rm.data(), offsets, w.max_atoms, w.atom_stride, w.partial.p, rs));
   return TNEP_OK;
 }
 

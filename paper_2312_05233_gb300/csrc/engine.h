@@ -121,6 +121,13 @@ struct Workspace {
   DevBuf<int> types_stage;
   DevStatus* d_status = nullptr;  // device status word of this workspace
   PinBuf<DevStatus> h_status;     // pinned host copy
+  // Structure offsets and boxes of the last batch in pinned memory, read by its
+  // kernels (no copy is enqueued for a few bytes).  ev_pin is recorded after
+  // the last kernel that reads them; pin_wait waits for it before they change.
+  PinBuf<int> h_offsets;
+  PinBuf<float> h_box;
+  cudaEvent_t ev_pin = nullptr;
+  bool pin_read = false;
   int atom_stride = 0;
   int cells_cap = 0;
   int cap_R = 0, cap_A = 0;  // caps the lists were built with
@@ -136,6 +143,11 @@ struct Workspace {
     if (d_status) cudaFree(d_status);
     d_status = nullptr;
     h_status.release();
+    h_offsets.release();
+    h_box.release();
+    if (ev_pin) cudaEventDestroy(ev_pin);
+    ev_pin = nullptr;
+    pin_read = false;
   }
 };
 
@@ -201,6 +213,11 @@ struct ListSpec {
   float rc_R, rc_A;
   int cap_R, cap_A;
 };
+// Waits until no kernel reads the workspace's pinned offsets and boxes.
+tnep_status pin_wait(Workspace& w);
+// The boxes [n] for the kernels of one call: the caller's device memory, or a
+// copy in the workspace's pinned memory.
+tnep_status stage_box(Workspace& w, const float* box, int n, const float** dev);
 tnep_status ensure_batch(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, const int* h_offsets, int cap_R,
                          int cap_A);
 tnep_status build_lists(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, const int* h_offsets, const float* d_pos,

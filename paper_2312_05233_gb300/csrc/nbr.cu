@@ -25,13 +25,16 @@ namespace tnep {
 
 namespace {
 
+constexpr int kSmallThreads = 256;
+
 __device__ __forceinline__ void raise_error(DevStatus* st, int code, int s) {
   if (atomicCAS(&st->error, 0, code) == 0) st->bad_struct = s;
 }
 
-__global__ void k_plan(NbrArgs a) {
-  const int s = blockIdx.x;
-  const int a0 = a.offsets[s], a1 = a.offsets[s + 1];
+// Box checks, bounding box of open axes and cell grid of structure s (atoms
+// [a0, a1)), by one CTA; the result (cells in G.nc, G.cell_offset = 0) is valid
+// in thread 0, the others return false.
+__device__ bool plan_structure(const NbrArgs& a, int s, int a0, int a1, StructGrid& G, StructBox& B) {
   const int n = a1 - a0;
   float L[3];
   for (int d = 0; d < 3; ++d) L[d] = a.box ? a.box[3 * s + d] : 0.0f;
@@ -57,13 +60,11 @@ __global__ void k_plan(NbrArgs a) {
   if (lane == 0)
     for (int d = 0; d < 3; ++d) { smn[d][w] = mn[d]; smx[d][w] = mx[d]; }
   __syncthreads();
-  if (threadIdx.x != 0) return;
+  if (threadIdx.x != 0) return false;
   for (int d = 0; d < 3; ++d) {
     mn[d] = smn[d][0]; mx[d] = smx[d][0];
     for (int k = 1; k < nw; ++k) { mn[d] = fminf(mn[d], smn[d][k]); mx[d] = fmaxf(mx[d], smx[d][k]); }
   }
-  StructGrid G;
-  StructBox B;
   const float edge_min = a.rc_R / (float)a.cell_div * (1.0f + 1e-5f);
   // x_div thins the cells along x (cell_div = 1 only)
   const float edge_min_x = a.cell_div == 1 ? edge_min / (float)a.x_div : edge_min;
@@ -109,9 +110,17 @@ __global__ void k_plan(NbrArgs a) {
     B.invL[d] = G.invL[d];
   }
   G.cell_offset = 0;
+  return true;
+}
+
+__global__ void k_plan(NbrArgs a) {
+  const int s = blockIdx.x;
+  StructGrid G;
+  StructBox B;
+  if (!plan_structure(a, s, a.offsets[s], a.offsets[s + 1], G, B)) return;
   a.grids[s] = G;
   a.boxes[s] = B;
-  a.struct_cells[s] = nc[0] * nc[1] * nc[2];
+  a.struct_cells[s] = G.nc[0] * G.nc[1] * G.nc[2];
 }
 
 // Exclusive scan of in[0..n) into out[0..n], out[n] = total, one CTA of 1024.
@@ -181,6 +190,12 @@ __device__ __forceinline__ int cell_coord(float x, const StructGrid& G, int d) {
   return min(max(c, 0), G.nc[d] - 1);
 }
 
+// A coordinate lies outside [0, L) on a periodic axis.
+__device__ __forceinline__ bool outside_box(float x0, float x1, float x2, const StructGrid& G) {
+  return (G.L[0] > 0.0f && !(x0 >= 0.0f && x0 < G.L[0])) || (G.L[1] > 0.0f && !(x1 >= 0.0f && x1 < G.L[1])) ||
+         (G.L[2] > 0.0f && !(x2 >= 0.0f && x2 < G.L[2]));
+}
+
 __global__ void k_bin(NbrArgs a) {
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= a.n_atoms) return;
@@ -197,10 +212,7 @@ __global__ void k_bin(NbrArgs a) {
   const int c0 = cell_coord(x0, G, 0);
   const int c1 = cell_coord(x1, G, 1);
   const int c2 = cell_coord(x2, G, 2);
-  const bool outside = (G.L[0] > 0.0f && !(x0 >= 0.0f && x0 < G.L[0])) ||
-                       (G.L[1] > 0.0f && !(x1 >= 0.0f && x1 < G.L[1])) ||
-                       (G.L[2] > 0.0f && !(x2 >= 0.0f && x2 < G.L[2]));
-  if (outside) atomicOr(&a.struct_flags[s], 1);
+  if (outside_box(x0, x1, x2, G)) atomicOr(&a.struct_flags[s], 1);
   const int cell = G.cell_offset + (c2 * G.nc[1] + c1) * G.nc[0] + c0;
   if (cell >= a.cells_cap) {  // unreachable: cells per structure <= 2n + 8
     raise_error(a.status, TNEP_ERR_INVALID, s);
@@ -248,6 +260,110 @@ __global__ void k_cell_sort(NbrArgs a, int* sorted_cell) {
     a.pos4[dst] = make_float4(a.pos[3 * (size_t)id], a.pos[3 * (size_t)id + 1], a.pos[3 * (size_t)id + 2],
                               __int_as_float(t));
   }
+  }
+}
+
+// The whole of plan, bin, scan, scatter and sort for structures of at most
+// kSmallStruct atoms, one CTA each: a structure's cells and cell-ordered atoms
+// need nothing from the others (its atoms occupy [offsets[s], offsets[s + 1]) in
+// both orders, its cells a private range of 2 n + 9 entries), so the six
+// launches of the general pipeline, each a few microseconds of latency, and
+// its two single-CTA scans fall away.  Bound by latency.  With the sums
+// of all models in one launch and the boxes and offsets read from pinned
+// memory, a call on a GB300 went from 286 to 235 us (one frame of 64 water
+// molecules) and from 333 to 284 us (61 open clusters).  Atom order, grids and positions are those of the
+// general pipeline.
+// Dynamic shared memory: 4 n + 9 ints (counts / starts of up to 2 n + 8 cells,
+// then per atom its cell and slot, and the atoms by cell), n = max_struct.
+__global__ void __launch_bounds__(kSmallThreads) k_prep_small(NbrArgs a, int* __restrict__ sorted_cell) {
+  extern __shared__ int sm_prep[];
+  __shared__ StructGrid Gs;
+  __shared__ int flag, carry, warp_sums[32];
+  const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
+  const int a0 = a.src_offsets[s], a1 = a.src_offsets[s + 1], n = a1 - a0;
+  {
+    StructGrid G;
+    StructBox B;
+    if (plan_structure(a, s, a0, a1, G, B)) {
+      G.cell_offset = 2 * a0 + 9 * s;
+      // the plan keeps to 2 n + 8 cells; an absurd box (infinite edges) may not
+      const int most = 2 * n + 8;
+      if (G.nc[0] < 1 || G.nc[1] < 1 || G.nc[2] < 1 || G.nc[0] > most || G.nc[1] > most || G.nc[2] > most ||
+          (long long)G.nc[0] * G.nc[1] * G.nc[2] > most) {
+        raise_error(a.status, TNEP_ERR_INVALID, s);
+        G.nc[0] = G.nc[1] = G.nc[2] = 1;
+      }
+      Gs = G;
+      a.grids[s] = G;
+      a.boxes[s] = B;
+      a.offsets_out[s] = a0;
+      if (s == a.n_structs - 1) a.offsets_out[a.n_structs] = a1;
+      flag = 0;
+      carry = 0;
+    }
+  }
+  __syncthreads();
+  const StructGrid G = Gs;
+  const int ncell = G.nc[0] * G.nc[1] * G.nc[2];
+  int* cnt = sm_prep;               // ncell + 1
+  int* where = cnt + 2 * n + 9;     // cell << 12 | slot
+  int* ids = where + n;
+  for (int c = tid; c <= ncell; c += blockDim.x) cnt[c] = 0;
+  __syncthreads();
+  bool out = false;
+  for (int l = tid; l < n; l += blockDim.x) {
+    const float* p = a.pos + 3 * (size_t)(a0 + l);
+    const float x0 = p[0], x1 = p[1], x2 = p[2];
+    out |= outside_box(x0, x1, x2, G);
+    const int cell = (cell_coord(x2, G, 2) * G.nc[1] + cell_coord(x1, G, 1)) * G.nc[0] + cell_coord(x0, G, 0);
+    where[l] = (cell << 12) | atomicAdd(&cnt[cell], 1);
+  }
+  if (out) flag = 1;
+  __syncthreads();
+  // exclusive scan of the counts in place, and the cell starts
+  int* starts = a.cell_start + G.cell_offset;
+  for (int base = 0; base <= ncell; base += blockDim.x) {
+    const int c = base + tid;
+    const int v = c < ncell ? cnt[c] : 0;
+    int incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (lane == 31) warp_sums[w] = incl;
+    __syncthreads();
+    int before = carry;
+    for (int k = 0; k < w; ++k) before += warp_sums[k];
+    if (c <= ncell) {
+      cnt[c] = before + incl - v;
+      starts[c] = a0 + before + incl - v;
+    }
+    __syncthreads();
+    if (tid == blockDim.x - 1) carry = before + incl;
+    __syncthreads();
+  }
+  if (tid == 0) a.struct_flags[s] = flag;
+  for (int l = tid; l < n; l += blockDim.x) ids[cnt[where[l] >> 12] + (where[l] & 4095)] = l;
+  __syncthreads();
+  // order every cell's atoms by input index
+  for (int e = tid; e < n; e += blockDim.x) {
+    const int l = ids[e], cell = where[l] >> 12;
+    const int b = cnt[cell], m = cnt[cell + 1];
+    int rank = 0;
+    for (int f = b; f < m; ++f) rank += ids[f] < l;
+    const int dst = a0 + b + rank, id = a0 + l;
+    a.sorted_orig[dst] = id;
+    a.orig_sorted[id] = dst;
+    a.sorted_struct[dst] = s;
+    sorted_cell[dst] = G.cell_offset + cell;
+    int t = a.types[id % a.types_period];
+    if (t < 0 || t >= a.n_types) {
+      raise_error(a.status, TNEP_ERR_INVALID, s);
+      t = 0;
+    }
+    a.pos4[dst] = make_float4(a.pos[3 * (size_t)id], a.pos[3 * (size_t)id + 1], a.pos[3 * (size_t)id + 2],
+                              __int_as_float(t));
   }
 }
 
@@ -666,17 +782,26 @@ __global__ void k_export(int n, const int* sorted_orig, const int* nbr_R, const 
 cudaError_t launch_neighbor_pipeline(const NbrArgs& a, cudaStream_t st) {
   const int S = a.n_structs, N = a.n_atoms;
   if (S <= 0) return cudaSuccess;
-  count_launches(N > 0 ? 7 : 3);
-  k_plan<<<S, 256, 0, st>>>(a);
-  k_scan_structs<<<1, 1024, 0, st>>>(a);
-  // The number of cells in use is known only on the device; the cell scan
-  // and the per-cell sort read it from struct_cells[S].
-  if (N > 0) k_bin<<<(N + 255) / 256, 256, 0, st>>>(a);
-  k_scan_cells<<<1, 1024, 0, st>>>(a);
-  if (N > 0) {
+  if (a.max_struct <= kSmallStruct) {
+    const int smem = (int)sizeof(int) * (4 * a.max_struct + 9);
+    const cudaError_t e = cudaFuncSetAttribute(k_prep_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)sizeof(int) * (4 * kSmallStruct + 9));
+    if (e != cudaSuccess) return e;
+    count_launches(N > 0 ? 2 : 1);
+    k_prep_small<<<S, kSmallThreads, smem, st>>>(a, a.atom_slot);
+  } else {
+    count_launches(7);
+    k_plan<<<S, 256, 0, st>>>(a);
+    k_scan_structs<<<1, 1024, 0, st>>>(a);
+    // The number of cells in use is known only on the device; the cell scan
+    // and the per-cell sort read it from struct_cells[S].
+    k_bin<<<(N + 255) / 256, 256, 0, st>>>(a);
+    k_scan_cells<<<1, 1024, 0, st>>>(a);
     k_scatter<<<(N + 255) / 256, 256, 0, st>>>(a);
     // sorted_cell reuses atom_slot (dead after the scatter)
     k_cell_sort<<<1216, 256, 0, st>>>(a, a.atom_slot);
+  }
+  if (N > 0) {
     const float rc2R = a.rc_R * a.rc_R, rc2A = a.rc_A * a.rc_A;
     if (a.two_ended)
       k_build<true><<<(N + 127) / 128, 128, 0, st>>>(a, a.atom_slot, rc2R, rc2A);

@@ -306,7 +306,7 @@ tnep_status create_pop(tnep_population* p, const float* params0, const float* po
   }
   const size_t pa = (size_t)m.C * p->ws.atom_stride * p->n_pop;
   TNEP_CUDA(p->ws.per_atom.ensure(pa));
-  TNEP_CUDA(p->ws.partial.ensure((size_t)p->n_pop * S * reduce_chunks(p->ws.max_atoms) * m.C));
+  TNEP_CUDA(p->ws.partial.ensure((size_t)p->n_pop * S * reduce_chunks(p->ws.max_atoms) * 9));
   TNEP_CUDA(p->d_params.ensure((size_t)p->n_pop * m.lay.words));
   TNEP_CUDA(p->h_params.ensure((size_t)p->n_pop * m.lay.words));
   TNEP_CUDA(p->d_target.ensure((size_t)S * m.C));

@@ -51,10 +51,16 @@ __host__ __device__ __forceinline__ size_t nbr_index(int i, int k, int cap) {
 }
 
 // Arguments of the neighbour-list pipeline.
+// Structures up to this size are prepared by one CTA each (nbr.cu): a cell's
+// atom slot takes 12 bits, and 64 KB of shared memory hold the counts.
+constexpr int kSmallStruct = 4095;
 struct NbrArgs {
   int n_structs;
   int n_atoms;
+  int max_struct;           // largest structure
   const int* offsets;       // [S+1] device
+  const int* src_offsets;   // [S+1] pinned host copy (small structures: read by the device)
+  int* offsets_out;         // device array the small-structure kernel copies them to
   const float* pos;         // [N][3] input order, device
   const float* box;         // [S][3] device or null
   const int* types;         // input types, device
@@ -261,12 +267,21 @@ size_t fused_smem_bytes(int variant, const ModelLayout& lay, int block, int tcm)
 cudaError_t launch_fused(int variant, int rank, const FusedArgs& a, int n_pop, int block, int tcm, cudaStream_t st);
 
 // Per-structure FP64 reduction of per-atom contributions.  `max_atoms` is
-// the largest structure; `partial` holds n_pop * n_structs * reduce_chunks(max_atoms) * C doubles.
+// the largest structure; `partial` holds n_pop * n_structs * reduce_chunks(max_atoms) * 9 doubles.
 constexpr int kReduceChunk = 2048;
 inline int reduce_chunks(int max_atoms) { return max_atoms > 0 ? (max_atoms + kReduceChunk - 1) / kReduceChunk : 1; }
 cudaError_t launch_reduce(int n_structs, int n_pop, const int* offsets, int max_atoms, const float* per_atom,
                           size_t per_atom_stride, int atom_stride, int C, double* partial, double* out,
                           size_t out_pop_stride, cudaStream_t st);
+// The same for several models over the same structures in one launch:
+// partial holds n_models * n_structs * reduce_chunks(max_atoms) * 9 doubles.
+struct ReduceModel {
+  const float* per_atom;
+  double* out;
+  int C;
+};
+cudaError_t launch_reduce_models(int n_structs, int n_models, const ReduceModel* models, const int* offsets,
+                                 int max_atoms, int atom_stride, double* partial, cudaStream_t st);
 
 // Gathers per-atom contributions back to input order: out[g][c] = pa[c][orig_sorted[g]].
 cudaError_t launch_gather_per_atom(int n_atoms, const int* orig_sorted, const float* per_atom,
