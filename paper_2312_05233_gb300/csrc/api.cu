@@ -100,6 +100,9 @@ tnep_status tnep_create(const tnep_model_desc* models, int n_models, int n_types
     e = dev_malloc(reinterpret_cast<void**>(&m.d_packed), sizeof(float) * m.lay.words);
     if (e == cudaSuccess)
       e = cudaMemcpy(m.d_packed, packed.data(), sizeof(float) * m.lay.words, cudaMemcpyHostToDevice);
+    const std::vector<float> w0t = pack_w0t(m, packed.data());
+    if (e == cudaSuccess) e = dev_malloc(reinterpret_cast<void**>(&m.d_w0t), sizeof(float) * w0t.size());
+    if (e == cudaSuccess) e = cudaMemcpy(m.d_w0t, w0t.data(), sizeof(float) * w0t.size(), cudaMemcpyHostToDevice);
     c->models.push_back(std::move(m));
     if (e != cudaSuccess) return bail(cuda_fail(e, "model upload"));
     if (fused_smem_bytes(c->models.back().variant, c->models.back().lay, kFusedBlockMax,
@@ -118,6 +121,8 @@ void tnep_destroy(tnep_ctx* c) {
   if (c->red_stream) cudaStreamSynchronize(c->red_stream);
   for (auto& m : c->models)
     if (m.d_packed) cudaFree(m.d_packed);
+  for (auto& m : c->models)
+    if (m.d_w0t) cudaFree(m.d_w0t);
   c->ws.release();
   c->skin_ws.release();
   c->pop_params.release();
@@ -278,7 +283,7 @@ tnep_status tnep_eval(tnep_ctx* c, int n_frames, int n_atoms, const float* pos, 
       if (use_skin)
         TNEP_TRY(skin_lists(c, c->ws, c->skin_ws, st, nf, n_atoms, d_pos, d_box, d_types));
       else
-        TNEP_TRY(build_lists(c, c->ws, st, nf, offs.data(), d_pos, d_box, d_types, n_atoms));
+        TNEP_TRY(build_lists(c, c->ws, st, nf, offs.data(), d_pos, d_box, d_types, n_atoms, nullptr, nf * n_atoms));
       if (!pos_dev && n_atoms > 0) TNEP_CUDA(cudaEventRecord(c->ev_consumed[b & 1], st));
       TNEP_CUDA(cudaEventRecord(ev[1], st));
       // with several passes, a pass's per-frame sums and their copy-out run on
@@ -357,7 +362,7 @@ tnep_status tnep_eval_batch(tnep_ctx* c, int n_structs, const int* atom_offsets,
     cudaEvent_t* ev = nullptr;
     TNEP_TRY(pass_events(c, 0, &ev));
     TNEP_CUDA(cudaEventRecord(ev[0], st));
-    TNEP_TRY(build_lists(c, c->ws, st, n_structs, atom_offsets, d_pos, d_box, d_types, std::max(N, 1)));
+    TNEP_TRY(build_lists(c, c->ws, st, n_structs, atom_offsets, d_pos, d_box, d_types, std::max(N, 1), nullptr, N));
     TNEP_CUDA(cudaEventRecord(ev[1], st));
     TNEP_TRY(run_models(c, c->ws, st, n_structs, N, ev[2]));
     bool regrow = false;

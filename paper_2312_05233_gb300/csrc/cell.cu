@@ -271,7 +271,7 @@ tnep_status tnep_eval_batch_cell(tnep_ctx* c, int n_structs, const int* atom_off
     const int Ctot = total_C(c);
     for (int attempt = 0; attempt < 4; ++attempt) {
       TNEP_TRY(reset_status(w, st));
-      TNEP_TRY(build_lists(c, w, st, n_structs, eoff.data(), d_epos.p, d_ebox.p, d_etypes.p, std::max(Ne, 1)));
+      TNEP_TRY(build_lists(c, w, st, n_structs, eoff.data(), d_epos.p, d_ebox.p, d_etypes.p, std::max(Ne, 1), nullptr, N));
       TNEP_TRY(run_models(c, w, st, n_structs, Ne, nullptr, d_ghost.p));
       regrow = false;
       TNEP_TRY(finish(c, w, st, &regrow));

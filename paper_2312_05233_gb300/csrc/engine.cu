@@ -178,6 +178,17 @@ void pack_params(const Model& m, int T, const float* flat, const float* scaler, 
   for (int d = 0; d < m.D; ++d) out[L.off_scaler + d] = scaler[d];
 }
 
+std::vector<float> pack_w0t(const Model& m, const float* packed) {
+  const ModelLayout& L = m.lay;
+  const int Hp = round_up(L.H, 32);
+  std::vector<float> t((size_t)L.nets * L.Dp * Hp, 0.f);
+  for (int net = 0; net < L.nets; ++net)
+    for (int h = 0; h < L.H; ++h)
+      for (int d = 0; d < L.Dp; ++d)
+        t[(((size_t)net * (L.Dp / 4) + d / 4) * Hp + h) * 4 + d % 4] = packed[L.off_W0 + (net * L.H + h) * L.Dp + d];
+  return t;
+}
+
 size_t expected_params(const tnep_model_desc& d, int T) {
   const int D = (d.n_max_R + 1) + (d.n_max_A + 1) * (d.l_max + (d.use_4body ? 1 : 0));
   const int nets = d.per_type_nn ? T : 1;
@@ -234,10 +245,6 @@ tnep_status ensure_batch(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, cons
   TNEP_CUDA(w.cnt_A.ensure(stride));
   TNEP_CUDA(w.cell_count.ensure(w.cells_cap + 1));
   TNEP_CUDA(w.cell_start.ensure(w.cells_cap + 1));
-  TNEP_CUDA(w.nbr_R.ensure((size_t)stride * w.cap_R));
-  TNEP_CUDA(w.nbr_tmp.ensure((size_t)stride * w.cap_R));
-  TNEP_CUDA(w.nbr_A.ensure((size_t)stride * w.cap_A));
-  TNEP_CUDA(w.seg_R.ensure((size_t)stride * c->n_types));
   if (!w.ev_pin) TNEP_CUDA(cudaEventCreateWithFlags(&w.ev_pin, cudaEventDisableTiming));
   // A trajectory's later passes have a prefix of the first one's offsets,
   // which its kernels may still be reading.
@@ -272,6 +279,16 @@ tnep_status stage_box(Workspace& w, const float* box, int n, const float** dev) 
   return TNEP_OK;
 }
 
+// Neighbour lists of the batch (not needed where one warp per atom keeps them
+// in shared memory).
+tnep_status ensure_lists(tnep_ctx* c, Workspace& w) {
+  TNEP_CUDA(w.nbr_R.ensure((size_t)w.atom_stride * w.cap_R));
+  TNEP_CUDA(w.nbr_tmp.ensure((size_t)w.atom_stride * w.cap_R));
+  TNEP_CUDA(w.nbr_A.ensure((size_t)w.atom_stride * w.cap_A));
+  TNEP_CUDA(w.seg_R.ensure((size_t)w.atom_stride * c->n_types));
+  return TNEP_OK;
+}
+
 // Offsets on the device for the kernels of a batch whose preparation does not
 // copy them itself.
 tnep_status copy_offsets(Workspace& w, cudaStream_t st, int S) {
@@ -280,10 +297,14 @@ tnep_status copy_offsets(Workspace& w, cudaStream_t st, int S) {
 }
 
 tnep_status build_lists(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, const int* h_offsets, const float* d_pos,
-                        const float* d_box, const int* d_types, int types_period, const ListSpec* spec) {
+                        const float* d_box, const int* d_types, int types_period, const ListSpec* spec,
+                        int wide_atoms) {
   const float rc_R = spec ? spec->rc_R : c->rc_R, rc_A = spec ? spec->rc_A : c->rc_A;
   TNEP_TRY(ensure_batch(c, w, st, S, h_offsets, spec ? spec->cap_R : c->cap_R, spec ? spec->cap_A : c->cap_A));
   const int N = h_offsets[S];
+  w.wide = wide_atoms > 0 && wide_atoms <= kWideAtoms && !spec &&
+           wide_smem_bytes(c->n_types, w.cap_R, w.cap_A) <= kWideMaxSmem;
+  if (!w.wide) TNEP_TRY(ensure_lists(c, w));
   if (w.max_atoms > kSmallStruct) {
     TNEP_TRY(copy_offsets(w, st, S));
     TNEP_CUDA(cudaMemsetAsync(w.cell_count.p, 0, sizeof(int) * (w.cells_cap + 1), st));
@@ -332,7 +353,8 @@ tnep_status build_lists(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, const
   a.cap_A = w.cap_A;
   a.cells_cap = w.cells_cap;
   a.status = w.d_status;
-  TNEP_CUDA(launch_neighbor_pipeline(a, st));
+  TNEP_CUDA(launch_neighbor_pipeline(a, !w.wide, st));
+  w.prepared = a;
   TNEP_TRY(pin_mark(w, st));
   return TNEP_OK;
 }
@@ -349,6 +371,8 @@ tnep_status skin_lists(tnep_ctx* c, Workspace& w, Workspace& sw, cudaStream_t st
   std::vector<int> offs(nf + 1);
   for (int k = 0; k <= nf; ++k) offs[k] = k * N;
   TNEP_TRY(ensure_batch(c, w, st, nf, offs.data(), c->cap_R, c->cap_A));
+  TNEP_TRY(ensure_lists(c, w));
+  w.wide = false;
   TNEP_TRY(copy_offsets(w, st, nf));
   SkinArgs a{};
   a.nf = nf;
@@ -390,13 +414,18 @@ tnep_status skin_lists(tnep_ctx* c, Workspace& w, Workspace& sw, cudaStream_t st
 
 // Radial moments of the lists in the workspace (F always; V for rank-1 and W
 // for rank-2 models).
-tnep_status compute_moments(tnep_ctx* c, Workspace& w, cudaStream_t st, int N, bool need_v, bool need_w) {
-  const int T = c->n_types;
-  const int per = T * kMomBasis;
+static tnep_status ensure_moments(tnep_ctx* c, Workspace& w, bool need_v, bool need_w) {
+  const int per = c->n_types * kMomBasis;
   w.mom_v0 = need_v ? per : -1;
   w.mom_w0 = need_w ? per * (need_v ? 4 : 1) : -1;
   const int slots = per * (1 + (need_v ? 3 : 0) + (need_w ? 6 : 0));
   TNEP_CUDA(w.mom.ensure((size_t)slots * w.atom_stride));
+  return TNEP_OK;
+}
+
+tnep_status compute_moments(tnep_ctx* c, Workspace& w, cudaStream_t st, int N, bool need_v, bool need_w) {
+  const int T = c->n_types;
+  TNEP_TRY(ensure_moments(c, w, need_v, need_w));
   RadialArgs r{};
   r.n_atoms = N;
   r.n_types = T;
@@ -481,22 +510,59 @@ tnep_status sum_pass_times(tnep_ctx* c, int n_pass) {
   return TNEP_OK;
 }
 
+// One warp per atom: the FP32-network models up to kWideModels of a variant at
+// a time, then lists and moments for the others.
+static tnep_status run_wide(tnep_ctx* c, Workspace& w, cudaStream_t st, const unsigned char* ghost, size_t per_model,
+                            bool* others) {
+  WideArgs a{};
+  a.nbr = w.prepared;
+  a.sorted_cell = w.atom_slot.p;
+  a.ghost = ghost;
+  a.atom_stride = w.atom_stride;
+  bool need_v = false, need_w = false;
+  *others = false;
+  for (int variant = 0; variant < kVarCount; ++variant) {
+    a.n_models = 0;
+    for (size_t k = 0; k <= c->models.size(); ++k) {
+      if (a.n_models == kWideModels || (k == c->models.size() && a.n_models > 0)) {
+        TNEP_CUDA(launch_wide(variant, true, a, st));
+        a.n_models = 0;
+      }
+      if (k == c->models.size()) break;
+      const Model& m = c->models[k];
+      if (m.variant != variant) continue;
+      if (m.d.mlp_precision != 0) {
+        *others = true;
+        (m.d.rank == 1 ? need_v : need_w) = true;
+        continue;
+      }
+      auto& d = a.model[a.n_models++];
+      d.model = m.d_packed;
+      d.w0t = m.d_w0t;
+      d.Hp = round_up(m.lay.H, 32);
+      d.lay = m.lay;
+      d.per_atom = w.per_atom.p + k * per_model;
+      d.rank = m.d.rank;
+    }
+  }
+  if (*others) {
+    TNEP_TRY(ensure_moments(c, w, need_v, need_w));
+    TNEP_CUDA(w.nbr_A.ensure((size_t)w.atom_stride * w.cap_A));
+    a.nbr.nbr_A = w.nbr_A.p;
+    a.mom = w.mom.p;
+    a.mom_stride = w.atom_stride;
+    a.v0 = w.mom_v0;
+    a.w0 = w.mom_w0;
+    TNEP_CUDA(launch_wide(0, false, a, st));
+  }
+  return TNEP_OK;
+}
+
 tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N, cudaEvent_t ev_done,
                        const unsigned char* ghost, cudaStream_t red_st) {
   const size_t per_model = (size_t)9 * w.atom_stride;
   TNEP_CUDA(w.per_atom.ensure(per_model * c->models.size()));
   TNEP_CUDA(w.out.ensure((size_t)std::max(S, 1) * total_C(c)));
-  TNEP_TRY(compute_moments(c, w, st, N, any_rank(c, 1), any_rank(c, 2)));
-  // per-pair cache of the angular walks, reused by every model in turn
-  // (skipped when the lists' cap would make it larger than 16 GB: a pass of
-  // 2^21 atoms at cap_A = 64 takes 8.6 GB)
-  constexpr size_t kPairCacheMaxBytes = size_t(16) << 30;
-  int quads = 0;
-  for (const auto& m : c->models) quads = std::max(quads, pair_cache_quads(m.d.n_max_A + 1));
-  const int pc_stride = round_up(std::max(N, 1), 128);
-  const size_t pc_elems = (size_t)w.cap_A * quads * pc_stride;
-  const bool use_pc = c->pair_cache && pc_elems * sizeof(float4) <= kPairCacheMaxBytes;
-  if (use_pc) TNEP_CUDA(w.pcache.ensure(pc_elems));
   const int* offsets = w.offsets.p;
   if (red_st) {
     // the previous pass's sums have read the per-atom outputs and offsets
@@ -506,17 +572,35 @@ tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N,
                               st));
     offsets = w.red_offsets.p;
   }
-  for (size_t k = 0; k < c->models.size(); ++k) {
-    const Model& m = c->models[k];
-    FusedArgs f = fused_args(c, w, m, N);
-    f.per_atom = w.per_atom.p + k * per_model;
-    f.per_atom_stride = 0;
-    f.pcache = use_pc ? w.pcache.p : nullptr;
-    f.pc_stride = pc_stride;
-    TNEP_CUDA(launch_fused(m.variant, m.d.rank, f, 1, c->block_atoms, m.d.mlp_precision, st));
+  bool thread_per_atom = true;
+  if (w.wide)
+    TNEP_TRY(run_wide(c, w, st, ghost, per_model, &thread_per_atom));
+  else
+    TNEP_TRY(compute_moments(c, w, st, N, any_rank(c, 1), any_rank(c, 2)));
+  if (thread_per_atom) {
+    // per-pair cache of the angular walks, reused by every model in turn
+    // (skipped when the lists' cap would make it larger than 16 GB: a pass of
+    // 2^21 atoms at cap_A = 64 takes 8.6 GB)
+    constexpr size_t kPairCacheMaxBytes = size_t(16) << 30;
+    int quads = 0;
+    for (const auto& m : c->models) quads = std::max(quads, pair_cache_quads(m.d.n_max_A + 1));
+    const int pc_stride = round_up(std::max(N, 1), 128);
+    const size_t pc_elems = (size_t)w.cap_A * quads * pc_stride;
+    const bool use_pc = c->pair_cache && pc_elems * sizeof(float4) <= kPairCacheMaxBytes;
+    if (use_pc) TNEP_CUDA(w.pcache.ensure(pc_elems));
+    for (size_t k = 0; k < c->models.size(); ++k) {
+      const Model& m = c->models[k];
+      if (w.wide && m.d.mlp_precision == 0) continue;
+      FusedArgs f = fused_args(c, w, m, N);
+      f.per_atom = w.per_atom.p + k * per_model;
+      f.per_atom_stride = 0;
+      f.pcache = use_pc ? w.pcache.p : nullptr;
+      f.pc_stride = pc_stride;
+      TNEP_CUDA(launch_fused(m.variant, m.d.rank, f, 1, c->block_atoms, m.d.mlp_precision, st));
+    }
   }
   if (ev_done) TNEP_CUDA(cudaEventRecord(ev_done, st));
-  if (ghost)
+  if (ghost && thread_per_atom)
     for (size_t k = 0; k < c->models.size(); ++k)
       TNEP_CUDA(launch_zero_ghosts(N, w.sorted_orig.p, ghost, w.per_atom.p + k * per_model, w.atom_stride,
                                    c->models[k].C, st));

@@ -99,6 +99,7 @@ struct Model {
   std::vector<float> params;
   std::vector<float> scaler;
   float* d_packed = nullptr;
+  float* d_w0t = nullptr;  // W0 as the warp-per-atom path reads it (see WideArgs)
 };
 
 // Device workspace of one in-flight batch.
@@ -132,6 +133,8 @@ struct Workspace {
   int cells_cap = 0;
   int cap_R = 0, cap_A = 0;  // caps the lists were built with
   int two_ended = 0;         // radial list layout of the last build (see NbrArgs)
+  bool wide = false;         // the batch is prepared for one warp per atom (no lists built yet)
+  NbrArgs prepared{};        // its arguments
   void release() {
     for (auto* b : {&offsets, &atom_struct, &atom_cell, &atom_slot, &cell_count, &cell_start, &cell_atoms,
                     &sorted_orig, &orig_sorted, &sorted_struct, &struct_cells, &cnt_R, &cnt_A, &nbr_R, &nbr_A,
@@ -204,6 +207,7 @@ struct tnep_ctx {
 namespace tnep {
 
 tnep_status pack_model(tnep_ctx* c, Model& m);
+std::vector<float> pack_w0t(const Model& m, const float* packed);
 void pack_params(const Model& m, int T, const float* flat, const float* scaler, float* out);
 void pack_index_map(const Model& m, int T, int* dst);
 size_t expected_params(const tnep_model_desc& d, int T);
@@ -218,10 +222,12 @@ tnep_status pin_wait(Workspace& w);
 // The boxes [n] for the kernels of one call: the caller's device memory, or a
 // copy in the workspace's pinned memory.
 tnep_status stage_box(Workspace& w, const float* box, int n, const float** dev);
-tnep_status ensure_batch(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, const int* h_offsets, int cap_R,
-                         int cap_A);
+tnep_status ensure_batch(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, const int* h_offsets, int cap_R, int cap_A);
+// wide_atoms > 0: the batch is followed by run_models and has that many atoms
+// to evaluate (without images), so it may take the warp-per-atom path.
 tnep_status build_lists(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, const int* h_offsets, const float* d_pos,
-                        const float* d_box, const int* d_types, int types_period, const ListSpec* spec = nullptr);
+                        const float* d_box, const int* d_types, int types_period, const ListSpec* spec = nullptr,
+                        int wide_atoms = 0);
 tnep_status skin_lists(tnep_ctx* c, Workspace& w, Workspace& sw, cudaStream_t st, int nf, int N, const float* d_pos,
                        const float* d_box, const int* d_types);
 tnep_status compute_moments(tnep_ctx* c, Workspace& w, cudaStream_t st, int N, bool need_v, bool need_w);

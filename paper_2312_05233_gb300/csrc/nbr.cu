@@ -19,6 +19,7 @@
 //           warp-tiled.
 // Pair selection follows the exact float32 recipe documented in tnep.h.
 
+#include "nbr_device.cuh"
 #include "tnep_internal.cuh"
 
 namespace tnep {
@@ -367,64 +368,6 @@ __global__ void __launch_bounds__(kSmallThreads) k_prep_small(NbrArgs a, int* __
   }
 }
 
-// Stencil cells along one axis with their image shift (in units of the box
-// edge, as the float32 product L * k) and their distance in whole cells,
-// max(|offset| - 1, 0), from the centre cell (0 where it is not known).
-// Periodic axes with at least 2k+1 cells wrap and carry the shift that the
-// minimum-image rule would pick for any pair within the cutoff; shorter
-// periodic axes list every cell once and leave the shift to rint (flagged by
-// the return value < 0).
-// `off` receives each stencil cell's offset from the centre cell before wrapping.
-__device__ __forceinline__ int axis_stencil(int c, int nc, float L, int k, int* cell, float* sh, int* unit,
-                                            int* off) {
-  int n = 0;
-  if (L > 0.0f) {
-    if (nc >= 2 * k + 1) {
-      for (int o = -k; o <= k; ++o) {
-        int cc = c + o;
-        float s = 0.0f;
-        if (cc < 0) { cc += nc; s = L; }
-        else if (cc >= nc) { cc -= nc; s = -L; }
-        cell[n] = cc; sh[n] = s; unit[n] = max(abs(o) - 1, 0); off[n] = o; ++n;
-      }
-    } else {
-      for (int o = 0; o < nc; ++o) { cell[n] = o; sh[n] = 0.0f; unit[n] = 0; off[n] = o - c; ++n; }
-      return -n;
-    }
-  } else {
-    const int lo = max(0, c - k), hi = min(nc - 1, c + k);
-    for (int o = lo; o <= hi; ++o) {
-      cell[n] = o; sh[n] = 0.0f; unit[n] = max(abs(o - c) - 1, 0); off[n] = o - c; ++n;
-    }
-  }
-  return n;
-}
-
-// Lower bound on the distance between points of two cells `u` whole cells
-// apart along an axis of edge e, less a margin for positions binned across
-// a face by rounding.
-__device__ __forceinline__ float cell_gap(int u, float e) { return fmaxf((float)u * e - 1e-3f, 0.0f); }
-
-// Margin (Angstrom) for float32 rounding of cell bounds, of binning and of
-// the pair rule in the window scan below.
-constexpr float kWindowMargin = 1e-3f;
-
-// Lower bound on the distance along one axis between a point at x (relative
-// to the grid origin) in cell c and the points of cell c + o, edge e.
-__device__ __forceinline__ float point_cell_gap(float x, int c, int o, float e) {
-  float g = 0.0f;
-  if (o > 0) g = (float)(c + o) * e - x;
-  else if (o < 0) g = x - (float)(c + o + 1) * e;
-  return fmaxf(g - kWindowMargin, 0.0f);
-}
-
-// Minimum-image difference with every operation rounded separately.
-__device__ __forceinline__ float mi_diff(float xj, float xi, float L, float invL) {
-  float d = __fsub_rn(xj, xi);
-  d = __fsub_rn(d, __fmul_rn(L, rintf(__fmul_rn(d, invL))));
-  return d;
-}
-
 // One thread per atom.  Radial entries go to a scratch list tagged with the
 // neighbour type (bits 29-31), then the same thread counting-sorts its own
 // entries by type into the final radial list (stable: ascending scan order
@@ -476,22 +419,6 @@ __global__ void __launch_bounds__(128) k_build(NbrArgs a, const int* sorted_cell
   const int s = a.sorted_struct[i];
   const StructGrid G = a.grids[s];
   const int lc = sorted_cell[i] - G.cell_offset;
-  const int cx = lc % G.nc[0], cy = (lc / G.nc[0]) % G.nc[1], cz = lc / (G.nc[0] * G.nc[1]);
-  const int k = a.cell_div;
-  const int kx = k == 1 ? a.x_div : k;  // x_div subdivides x only, and only with cell_div = 1
-  int xc[9], yc[7], zc[7], xu[9], yu[7], zu[7], xo[9], yo[7], zo[7];
-  float xs[9], ys[7], zs[7];
-  int nx = axis_stencil(cx, G.nc[0], G.L[0], kx, xc, xs, xu, xo);
-  int ny = axis_stencil(cy, G.nc[1], G.L[1], k, yc, ys, yu, yo);
-  int nz = axis_stencil(cz, G.nc[2], G.L[2], k, zc, zs, zu, zo);
-  // stencil cells farther than the cutoff from the centre cell are skipped
-  const float ex = 1.0f / G.cinv[0], ey = 1.0f / G.cinv[1], ez = 1.0f / G.cinv[2];
-  // The shift of a stencil cell equals L * rint((p_j - p_i) / L) for every pair
-  // the cutoff can accept when all coordinates lie in [0, L); otherwise (or
-  // when an axis has too few cells to carry shifts) use rint per pair.  Both
-  // give the float32 rule of the header bit for bit.
-  const bool use_rint = nx < 0 || ny < 0 || nz < 0 || (a.struct_flags[s] & 1);
-  nx = abs(nx); ny = abs(ny); nz = abs(nz);
   // scratch entry e of this thread lives at wR[e * ws]
   int* wR = a.nbr_tmp + (size_t)(i >> 5) * a.cap_R * 32 + (i & 31);
   constexpr int ws = 32;
@@ -549,72 +476,9 @@ __global__ void __launch_bounds__(128) k_build(NbrArgs a, const int* sorted_cell
       }
     }
   };
-  if (kx > 1 && k == 1 && !use_rint) {
-    // Window scan: cells are thin along x.  In each (y, z) row of the stencil
-    // only the x-cells meeting [x_i - h, x_i + h] can hold pairs, where
-    // h^2 = rc_R^2 - (distance from atom i to the row)^2; on a periodic axis
-    // the window splits at the box faces into ranges with shifts +L, 0, -L.
-    // A window longer than the row falls back to the whole row with rint.
-    const float xr = pi.x - G.origin[0], yr = pi.y - G.origin[1], zr = pi.z - G.origin[2];
-    const float rcm = a.rc_R + kWindowMargin, rcm2 = rcm * rcm;
-    const int ncx = G.nc[0];
-    for (int iz = 0; iz < nz; ++iz) {
-      const float gz = point_cell_gap(zr, cz, zo[iz], ez);
-      if (gz * gz >= rcm2) continue;
-      for (int iy = 0; iy < ny; ++iy) {
-        const float gy = point_cell_gap(yr, cy, yo[iy], ey);
-        const float h2 = rcm2 - gy * gy - gz * gz;
-        if (h2 <= 0.0f) continue;
-        const float h = sqrtf(h2) + kWindowMargin;
-        int clo = (int)floorf((xr - h) * G.cinv[0]);
-        int chi = (int)floorf((xr + h) * G.cinv[0]);
-        const int row = G.cell_offset + (zc[iz] * G.nc[1] + yc[iy]) * ncx;
-        const float sy = ys[iy], sz = zs[iz];
-        if (G.L[0] > 0.0f) {
-          if (chi - clo + 1 > ncx) {
-            scan(a.cell_start[row], a.cell_start[row + ncx], 0.0f, sy, sz, true);
-            continue;
-          }
-          if (clo < 0) scan(a.cell_start[row + clo + ncx], a.cell_start[row + ncx], G.L[0], sy, sz, false);
-          const int b0 = max(clo, 0), b1 = min(chi, ncx - 1);
-          if (b0 <= b1) scan(a.cell_start[row + b0], a.cell_start[row + b1 + 1], 0.0f, sy, sz, false);
-          if (chi >= ncx) scan(a.cell_start[row], a.cell_start[row + chi - ncx + 1], -G.L[0], sy, sz, false);
-        } else {
-          clo = max(clo, 0);
-          chi = min(chi, ncx - 1);
-          if (clo <= chi) scan(a.cell_start[row + clo], a.cell_start[row + chi + 1], 0.0f, sy, sz, false);
-        }
-      }
-    }
-  } else {
-    for (int iz = 0; iz < nz; ++iz) {
-      const float gz = cell_gap(zu[iz], ez);
-      if (gz * gz >= rc2R) continue;
-      for (int iy = 0; iy < ny; ++iy) {
-        const float gy = cell_gap(yu[iy], ey);
-        const float gyz = gy * gy + gz * gz;
-        if (gyz >= rc2R) continue;
-        const int row = G.cell_offset + (zc[iz] * G.nc[1] + yc[iy]) * G.nc[0];
-        const float sy = ys[iy], sz = zs[iz];
-        int ix = 0;
-        while (ix < nx) {
-          const float gx = cell_gap(xu[ix], ex);
-          if (gx * gx + gyz >= rc2R) { ++ix; continue; }
-          // merge x-cells that are contiguous, within reach and share a shift into one range
-          int ie = ix + 1;
-          while (ie < nx && xc[ie] == xc[ie - 1] + 1 && xs[ie] == xs[ix]) {
-            const float ge = cell_gap(xu[ie], ex);
-            if (ge * ge + gyz >= rc2R) break;
-            ++ie;
-          }
-          const float sx = xs[ix];
-          const int j0 = a.cell_start[row + xc[ix]], j1 = a.cell_start[row + xc[ie - 1] + 1];
-          ix = ie;
-          scan(j0, j1, sx, sy, sz, use_rint);
-        }
-      }
-    }
-  }
+  const Stencil sten(a, s, G, lc, pi, rc2R);
+  for (int iz = 0; iz < sten.nz; ++iz)
+    for (int iy = 0; iy < sten.ny; ++iy) sten.row(a, G, iy, iz, scan);
   a.cnt_R[i] = cR;
   a.cnt_A[i] = cA;
   if (cR > a.cap_R) atomicMax(&a.status->max_cnt_R, cR);
@@ -779,7 +643,7 @@ __global__ void k_export(int n, const int* sorted_orig, const int* nbr_R, const 
 
 }  // namespace
 
-cudaError_t launch_neighbor_pipeline(const NbrArgs& a, cudaStream_t st) {
+cudaError_t launch_neighbor_pipeline(const NbrArgs& a, bool build, cudaStream_t st) {
   const int S = a.n_structs, N = a.n_atoms;
   if (S <= 0) return cudaSuccess;
   if (a.max_struct <= kSmallStruct) {
@@ -787,10 +651,10 @@ cudaError_t launch_neighbor_pipeline(const NbrArgs& a, cudaStream_t st) {
     const cudaError_t e = cudaFuncSetAttribute(k_prep_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)sizeof(int) * (4 * kSmallStruct + 9));
     if (e != cudaSuccess) return e;
-    count_launches(N > 0 ? 2 : 1);
+    count_launches(1);
     k_prep_small<<<S, kSmallThreads, smem, st>>>(a, a.atom_slot);
   } else {
-    count_launches(7);
+    count_launches(6);
     k_plan<<<S, 256, 0, st>>>(a);
     k_scan_structs<<<1, 1024, 0, st>>>(a);
     // The number of cells in use is known only on the device; the cell scan
@@ -801,7 +665,8 @@ cudaError_t launch_neighbor_pipeline(const NbrArgs& a, cudaStream_t st) {
     // sorted_cell reuses atom_slot (dead after the scatter)
     k_cell_sort<<<1216, 256, 0, st>>>(a, a.atom_slot);
   }
-  if (N > 0) {
+  if (N > 0 && build) {
+    count_launches(1);
     const float rc2R = a.rc_R * a.rc_R, rc2A = a.rc_A * a.rc_A;
     if (a.two_ended)
       k_build<true><<<(N + 127) / 128, 128, 0, st>>>(a, a.atom_slot, rc2R, rc2A);

@@ -136,7 +136,7 @@ tnep_status launch_batch(tnep_server* s, Pipeline& p) {
   }
   TNEP_CUDA(cudaMemcpyAsync(p.d_box.p, p.h_box.p, sizeof(float) * 3 * S, cudaMemcpyHostToDevice, st));
   TNEP_TRY(reset_status(p.ws, st));
-  TNEP_TRY(build_lists(c, p.ws, st, S, p.offsets.data(), p.d_pos.p, p.d_box.p, p.d_types.p, std::max(N, 1)));
+  TNEP_TRY(build_lists(c, p.ws, st, S, p.offsets.data(), p.d_pos.p, p.d_box.p, p.d_types.p, std::max(N, 1), nullptr, N));
   TNEP_TRY(run_models(c, p.ws, st, S, N, nullptr));
   TNEP_CUDA(cudaMemcpyAsync(p.h_out.p, p.ws.out.p, sizeof(double) * S * total_C(c), cudaMemcpyDeviceToHost, st));
   TNEP_CUDA(cudaMemcpyAsync(p.ws.h_status.p, p.ws.d_status, sizeof(DevStatus), cudaMemcpyDeviceToHost, st));

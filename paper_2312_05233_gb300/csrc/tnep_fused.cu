@@ -43,60 +43,6 @@ namespace tnep {
 
 namespace {
 
-// V += sum_lm S_lm * grad p_lm(x, y, z)  (gradient of the polynomial as written).
-// Each order l accumulates into its own partial sums so that the four
-// dependency chains run side by side.
-template <int LMAX>
-__device__ __forceinline__ void harmonic_grad(const float* S, float x, float y, float z, float& vx, float& vy,
-                                              float& vz) {
-  float ax = S[0], ay = S[1], az = S[2];
-  float bx = 0.f, by = 0.f, bz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f, dx = 0.f, dy = 0.f, dz = 0.f;
-  if constexpr (LMAX >= 2) {
-    bx = y * S[3] + z * S[5] + 2.f * x * S[6];
-    by = x * S[3] + z * S[4] - 2.f * y * S[6];
-    bz = y * S[4] + x * S[5] + 6.f * z * S[7];
-    if constexpr (LMAX >= 3) {
-      const float x2 = x * x, y2 = y * y, z2 = z * z;
-      const float xy = x * y, yz = y * z, xz = x * z;
-      const float t5 = 5.f * z2 - 1.f;
-      // p8 = 3x^2y - y^3, p9 = xyz, p10 = y(5z^2-1), p11 = 5z^3 - 3z,
-      // p12 = x(5z^2-1), p13 = z(x^2-y^2), p14 = x^3 - 3xy^2
-      cx = 6.f * xy * S[8] + yz * S[9] + t5 * S[12] + 2.f * xz * S[13] + (3.f * x2 - 3.f * y2) * S[14];
-      cy = (3.f * x2 - 3.f * y2) * S[8] + xz * S[9] + t5 * S[10] - 2.f * yz * S[13] - 6.f * xy * S[14];
-      cz = xy * S[9] + 10.f * yz * S[10] + (15.f * z2 - 3.f) * S[11] + 10.f * xz * S[12] + (x2 - y2) * S[13];
-      if constexpr (LMAX >= 4) {
-        const float t7 = 7.f * z2 - 1.f, t73 = 7.f * z2 - 3.f;
-        const float xyz = xy * z;
-        // p15 = x^3 y - x y^3, p16 = 3x^2yz - y^3 z, p17 = xy(7z^2-1),
-        // p18 = 7yz^3 - 3yz, p19 = 35z^4 - 30z^2 + 3, p20 = xz(7z^2-3),
-        // p21 = (x^2-y^2)(7z^2-1), p22 = x^3 z - 3 x y^2 z, p23 = x^4 - 6x^2y^2 + y^4
-        dx = (3.f * x2 * y - y2 * y) * S[15] + 6.f * xyz * S[16] + y * t7 * S[17] + t73 * z * S[20] +
-             2.f * x * t7 * S[21] + (3.f * x2 - 3.f * y2) * z * S[22] + (4.f * x2 * x - 12.f * x * y2) * S[23];
-        dy = (x2 * x - 3.f * x * y2) * S[15] + (3.f * x2 - 3.f * y2) * z * S[16] + x * t7 * S[17] +
-             t73 * z * S[18] - 2.f * y * t7 * S[21] - 6.f * xyz * S[22] + (4.f * y2 * y - 12.f * x2 * y) * S[23];
-        dz = (3.f * x2 * y - y2 * y) * S[16] + 14.f * xyz * S[17] + (21.f * z2 - 3.f) * y * S[18] +
-             (140.f * z2 - 60.f) * z * S[19] + (21.f * z2 - 3.f) * x * S[20] + 14.f * z * (x2 - y2) * S[21] +
-             (x2 * x - 3.f * x * y2) * S[22];
-      }
-    }
-  }
-  vx += (ax + bx) + (cx + dx);
-  vy += (ay + by) + (cy + dy);
-  vz += (az + bz) + (cz + dz);
-}
-
-// Loads one (t_i, t_j) coefficient block c[n][k] from shared memory.
-template <int NN, int B>
-__device__ __forceinline__ void load_coeffs(const float* blk, float* cc) {
-  constexpr int NV = (NN * B + 3) / 4;
-  const float4* c4 = reinterpret_cast<const float4*>(blk);
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const float4 t = c4[v];
-    cc[4 * v] = t.x; cc[4 * v + 1] = t.y; cc[4 * v + 2] = t.z; cc[4 * v + 3] = t.w;
-  }
-}
-
 // Bytes of shared memory the tensor-core network needs after the scratch:
 // mbarrier + TMEM slot (128 B), the A tile (128 rows x 64: a high and a low
 // bf16 part of 32 columns each) and, per network, the two B tiles (32 rows x

@@ -128,7 +128,8 @@ struct SkinArgs {
 cudaError_t launch_skin_compact(const SkinArgs& a, cudaStream_t st);
 
 // Launches the cell-list + neighbour pipeline on `st`.
-cudaError_t launch_neighbor_pipeline(const NbrArgs& a, cudaStream_t st);
+// (build: up to the neighbour lists; otherwise only cells and sorted atoms).
+cudaError_t launch_neighbor_pipeline(const NbrArgs& a, bool build, cudaStream_t st);
 
 // Radial moments per atom and neighbour type t (SoA, slot-major, stride mom_stride):
 //   F^t_k     = sum_{j of type t} f_k(r_ij)                       slots  t*B + k
@@ -265,6 +266,36 @@ int variant_of(int nR, int nA, int bR, int bA, int lmax, int fb);
 // split high/low BF16 operands, three products (2); 1 and 2 use 128 atoms per CTA.
 size_t fused_smem_bytes(int variant, const ModelLayout& lay, int block, int tcm);
 cudaError_t launch_fused(int variant, int rank, const FusedArgs& a, int n_pop, int block, int tcm, cudaStream_t st);
+
+// One warp per atom for small batches (wide.cu): neighbour lists, radial
+// moments and, when fused, the whole path of up to kWideModels FP32-network
+// models of one variant; otherwise the angular lists, their counts and the
+// moments in the layouts of the general path.
+constexpr int kWideModels = 4;
+// Largest batch of the warp-per-atom path.  Measured calls (two models, GB300),
+// thread / warp per atom: 11,520 atoms of water 238 / 210 us, 19,200 243 / 288 us;
+// six types, 9,696 atoms 400 / 235 us, 34,301 522 / 625 us.
+constexpr int kWideAtoms = 12288;
+constexpr size_t kWideMaxSmem = 100 * 1024;  // two CTAs per SM
+struct WideArgs {
+  NbrArgs nbr;                  // prepared batch (cells, sorted atoms)
+  const int* sorted_cell;
+  const unsigned char* ghost;   // null, or per input atom: an image atom, skipped (fused: contributes zeros)
+  int n_models;
+  struct {
+    const float* model;
+    const float* w0t;           // W0 by float4: [net][Dp / 4][Hp][4], Hp = H rounded up to 32
+    int Hp;
+    ModelLayout lay;
+    float* per_atom;
+    int rank;
+  } model[kWideModels];
+  int atom_stride;
+  float* mom; int mom_stride; int v0, w0;   // not fused: see RadialArgs
+  float w[24];                  // weights of the angular functions (set by the launcher)
+};
+size_t wide_smem_bytes(int n_types, int cap_R, int cap_A);
+cudaError_t launch_wide(int variant, bool fused, const WideArgs& a, cudaStream_t st);
 
 // Per-structure FP64 reduction of per-atom contributions.  `max_atoms` is
 // the largest structure; `partial` holds n_pop * n_structs * reduce_chunks(max_atoms) * 9 doubles.

@@ -3,7 +3,9 @@
 Structures of at most 4095 atoms are prepared by one CTA each, batches with a
 larger one by the general pipeline; atom order, lists and sums are defined to
 be the same, so a structure's tensors and per-atom contributions must not
-depend on what else is in the batch (exact comparison, no tolerance)."""
+depend on what else is in the batch (exact comparison, no tolerance).  Batches
+of at most 12288 atoms take one warp per atom for the FP32 network (and for the
+lists and moments of the tensor-core one), larger ones a thread."""
 
 import numpy as np
 import pytest
@@ -61,3 +63,61 @@ def test_a_structure_alone_and_beside_a_large_one(tn, n_types, precision):
             for m in range(2):
                 assert np.array_equal(out[m][0], all_out[m][k]), (k, m)
                 assert np.array_equal(pa[m], all_pa[m][bt.offsets[k]:bt.offsets[k + 1]]), (k, m)
+
+
+VARIANTS = {"std": {}, "small": dict(n_max_R=3, n_max_A=2, basis_R=6, basis_A=5, l_max=3)}
+
+
+@pytest.mark.parametrize("n_types", [1, 2, 3, 6])
+@pytest.mark.parametrize("variant", ["std", "small"])
+def test_warp_per_atom_equals_thread_per_atom(tn, n_types, variant):
+    """Small batches against the same structures beside 13,000 other atoms; no
+    neighbours, one, more than 32 and more than 64 angular ones (two and three
+    chunks of pairs), types absent from a neighbourhood, n_hidden above 32."""
+    rng = np.random.default_rng(17)
+    structs = [water(64, rng), water(81, rng, 1)]
+    for n in (1, 2, 33):
+        p, t, b = synth.water_cluster(n, rng)
+        structs.append(synth.Structure(p.astype(np.float32), t, b.astype(np.float32)))
+    structs.append(synth.Structure(np.float32([[0, 0, 0]]), np.int32([0]), np.zeros(3, np.float32)))
+    for n in (40, 90):  # dense balls: every atom sees n - 1 others within the angular cutoff
+        v = rng.standard_normal((n, 3))
+        v *= (1.9 * rng.uniform(0.2, 1.0, (n, 1)) ** (1 / 3)) / np.linalg.norm(v, axis=1, keepdims=True)
+        structs.append(synth.Structure(v.astype(np.float32), np.zeros(n, np.int32), np.zeros(3, np.float32)))
+    for s in structs:
+        s.types = (np.arange(len(s.types)) * 7 % 11 % n_types).astype(np.int32)
+    filler = water(4400, rng)
+    filler.types = (np.arange(len(filler.types)) % n_types).astype(np.int32)
+    models = []
+    for rank, hidden in ((1, 30), (2, 30), (2, 40), (1, 5), (1, 64)):
+        hp = synth.HyperParams(n_types=n_types, rank=rank, n_hidden=hidden, **VARIANTS[variant])
+        models.append(tn.Model.from_hyper(hp, synth.model_params(hp, rng), synth.default_q_scaler(hp)[:hp.dim]))
+    with tn.tnep_create(models, n_types, (6.0, 4.0)) as ctx:
+        small, big = synth.concat_structures(structs), synth.concat_structures(structs + [filler])
+        o1, p1 = tn.tnep_eval_batch(ctx, small.offsets, small.pos, small.box, small.types, per_atom=True)
+        o2, p2 = tn.tnep_eval_batch(ctx, big.offsets, big.pos, big.box, big.types, per_atom=True)
+        for m in range(len(models)):
+            assert np.array_equal(p1[m], p2[m][:small.offsets[-1]]), m
+            assert np.array_equal(o1[m], o2[m][:len(structs)]), m
+
+
+def test_small_batch_regrows_its_lists(tn):
+    """More neighbours than the lists hold at first: both routes repeat the
+    batch with larger ones, and refuse above the hard cap."""
+    rng = np.random.default_rng(23)
+    v = rng.standard_normal((300, 3))
+    v *= (2.5 * rng.uniform(0.3, 1.0, (300, 1)) ** (1 / 3)) / np.linalg.norm(v, axis=1, keepdims=True)
+    dense = synth.Structure(v.astype(np.float32), np.arange(300, dtype=np.int32) % 2, np.zeros(3, np.float32))
+    filler = water(4400, rng)
+    outs = []
+    for structs in ([dense], [dense, filler]):
+        bt = synth.concat_structures(structs)
+        with context(tn, 2, 0) as ctx:
+            outs.append(tn.tnep_eval_batch(ctx, bt.offsets, bt.pos, bt.box, bt.types)[0])
+        with context(tn, 2, 0) as ctx:
+            tn.tnep_set_option(ctx, tn.TNEP_OPT_MAX_NEIGHBORS, 200)
+            with pytest.raises(tn.TnepError) as e:
+                tn.tnep_eval_batch(ctx, bt.offsets, bt.pos, bt.box, bt.types)
+            assert e.value.status == 4
+    for a, b in zip(*outs):
+        assert np.array_equal(a[0], b[0])
