@@ -26,7 +26,13 @@ namespace tnep {
 
 namespace {
 
-constexpr int kSmallThreads = 256;
+constexpr int kSmallThreads = 1024;  // 256 for structures of at most 1024 atoms
+// Largest batch of k_build_group, up to two types and more.  Measured neighbour
+// pipelines (GB300), group / thread: water 15,360 atoms 35 / 51 us, 28,800 51 / 55,
+// 41,472 in one box 118 / 125, 76,800 91 / 64; three types, 17,280 atoms 79 / 120, 69,120
+// 161 / 158; six types, 49,600 atoms 150 / 170 us.
+constexpr int kGroupAtoms2 = 32768, kGroupAtoms = 57344;
+constexpr size_t kGroupMaxSmem = 100 * 1024;  // two CTAs per SM
 
 __device__ __forceinline__ void raise_error(DevStatus* st, int code, int s) {
   if (atomicCAS(&st->error, 0, code) == 0) st->bad_struct = s;
@@ -124,16 +130,16 @@ __global__ void k_plan(NbrArgs a) {
   a.struct_cells[s] = G.nc[0] * G.nc[1] * G.nc[2];
 }
 
-// Exclusive scan of in[0..n) into out[0..n], out[n] = total, one CTA of 1024.
+// Exclusive scan of in[0..n) into out[0..n], plus base, out[n] = base + total, one CTA of 1024.
 // Tiles of 4 consecutive elements per thread (coalesced), scanned across the
 // warps and carried into the next tile.  in and out may alias: each thread
 // reads its own elements before writing them.
-__device__ void block_exclusive_scan(const int* in, int* out, int n) {
+__device__ void block_exclusive_scan(const int* in, int* out, int n, int base_value) {
   constexpr int V = 4;
   __shared__ int warp_sums[32];
   __shared__ int carry;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
-  if (tid == 0) carry = 0;
+  if (tid == 0) carry = base_value;
   __syncthreads();
   for (int base = 0; base < n; base += blockDim.x * V) {
     const int k0 = base + tid * V;
@@ -174,7 +180,7 @@ __device__ void block_exclusive_scan(const int* in, int* out, int n) {
 }
 
 __global__ void k_scan_structs(NbrArgs a) {
-  block_exclusive_scan(a.struct_cells, a.struct_cells, a.n_structs);
+  block_exclusive_scan(a.struct_cells, a.struct_cells, a.n_structs, 0);
   __syncthreads();
   for (int s = threadIdx.x; s < a.n_structs; s += blockDim.x) a.grids[s].cell_offset = a.struct_cells[s];
   if (threadIdx.x == 0 && a.struct_cells[a.n_structs] > a.cells_cap) raise_error(a.status, TNEP_ERR_INVALID, -1);
@@ -224,9 +230,14 @@ __global__ void k_bin(NbrArgs a) {
   a.atom_slot[g] = atomicAdd(&a.cell_count[cell], 1);
 }
 
-__global__ void k_scan_cells(NbrArgs a) {
-  const int n_cells = min(a.struct_cells[a.n_structs], a.cells_cap);
-  block_exclusive_scan(a.cell_count, a.cell_start, n_cells);
+// One CTA per structure: its cells hold its atoms, so their starts follow from
+// the structure's first atom (one CTA over all cells: 79 us for 50 frames of
+// 41,472 atoms).  The entry after the last cell is the next structure's first,
+// which both CTAs write with the same value.
+__global__ void __launch_bounds__(1024) k_scan_cells(NbrArgs a) {
+  const int s = blockIdx.x;
+  const int c0 = min(a.struct_cells[s], a.cells_cap), c1 = min(a.struct_cells[s + 1], a.cells_cap);
+  block_exclusive_scan(a.cell_count + c0, a.cell_start + c0, c1 - c0, a.offsets[s]);
 }
 
 __global__ void k_scatter(NbrArgs a) {
@@ -276,11 +287,14 @@ __global__ void k_cell_sort(NbrArgs a, int* sorted_cell) {
 // general pipeline.
 // Dynamic shared memory: 4 n + 9 ints (counts / starts of up to 2 n + 8 cells,
 // then per atom its cell and slot, and the atoms by cell), n = max_struct.
+constexpr int kSlotBits = 14;
+static_assert(kSmallStruct < (1 << kSlotBits) && 2 * kSmallStruct + 8 < (1 << (31 - kSlotBits)), "cell and slot share a word");
+
 __global__ void __launch_bounds__(kSmallThreads) k_prep_small(NbrArgs a, int* __restrict__ sorted_cell) {
   extern __shared__ int sm_prep[];
   __shared__ StructGrid Gs;
   __shared__ int flag, carry, warp_sums[32];
-  const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
+  const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int a0 = a.src_offsets[s], a1 = a.src_offsets[s + 1], n = a1 - a0;
   {
     StructGrid G;
@@ -307,7 +321,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_prep_small(NbrArgs a, int* __
   const StructGrid G = Gs;
   const int ncell = G.nc[0] * G.nc[1] * G.nc[2];
   int* cnt = sm_prep;               // ncell + 1
-  int* where = cnt + 2 * n + 9;     // cell << 12 | slot
+  int* where = cnt + 2 * n + 9;     // cell << kSlotBits | slot
   int* ids = where + n;
   for (int c = tid; c <= ncell; c += blockDim.x) cnt[c] = 0;
   __syncthreads();
@@ -317,7 +331,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_prep_small(NbrArgs a, int* __
     const float x0 = p[0], x1 = p[1], x2 = p[2];
     out |= outside_box(x0, x1, x2, G);
     const int cell = (cell_coord(x2, G, 2) * G.nc[1] + cell_coord(x1, G, 1)) * G.nc[0] + cell_coord(x0, G, 0);
-    where[l] = (cell << 12) | atomicAdd(&cnt[cell], 1);
+    where[l] = (cell << kSlotBits) | atomicAdd(&cnt[cell], 1);
   }
   if (out) flag = 1;
   __syncthreads();
@@ -345,11 +359,11 @@ __global__ void __launch_bounds__(kSmallThreads) k_prep_small(NbrArgs a, int* __
     __syncthreads();
   }
   if (tid == 0) a.struct_flags[s] = flag;
-  for (int l = tid; l < n; l += blockDim.x) ids[cnt[where[l] >> 12] + (where[l] & 4095)] = l;
+  for (int l = tid; l < n; l += blockDim.x) ids[cnt[where[l] >> kSlotBits] + (where[l] & ((1 << kSlotBits) - 1))] = l;
   __syncthreads();
   // order every cell's atoms by input index
   for (int e = tid; e < n; e += blockDim.x) {
-    const int l = ids[e], cell = where[l] >> 12;
+    const int l = ids[e], cell = where[l] >> kSlotBits;
     const int b = cnt[cell], m = cnt[cell + 1];
     int rank = 0;
     for (int f = b; f < m; ++f) rank += ids[f] < l;
@@ -366,6 +380,39 @@ __global__ void __launch_bounds__(kSmallThreads) k_prep_small(NbrArgs a, int* __
     a.pos4[dst] = make_float4(a.pos[3 * (size_t)id], a.pos[3 * (size_t)id + 1], a.pos[3 * (size_t)id + 2],
                               __int_as_float(t));
   }
+}
+
+// Stencil cells along one axis with their image shift (in units of the box
+// edge, as the float32 product L * k) and their distance in whole cells,
+// max(|offset| - 1, 0), from the centre cell (0 where it is not known).
+// Periodic axes with at least 2k+1 cells wrap and carry the shift that the
+// minimum-image rule would pick for any pair within the cutoff; shorter
+// periodic axes list every cell once and leave the shift to rint (flagged by
+// the return value < 0).
+// `off` receives each stencil cell's offset from the centre cell before wrapping.
+__device__ __forceinline__ int axis_stencil(int c, int nc, float L, int k, int* cell, float* sh, int* unit,
+                                            int* off) {
+  int n = 0;
+  if (L > 0.0f) {
+    if (nc >= 2 * k + 1) {
+      for (int o = -k; o <= k; ++o) {
+        int cc = c + o;
+        float s = 0.0f;
+        if (cc < 0) { cc += nc; s = L; }
+        else if (cc >= nc) { cc -= nc; s = -L; }
+        cell[n] = cc; sh[n] = s; unit[n] = max(abs(o) - 1, 0); off[n] = o; ++n;
+      }
+    } else {
+      for (int o = 0; o < nc; ++o) { cell[n] = o; sh[n] = 0.0f; unit[n] = 0; off[n] = o - c; ++n; }
+      return -n;
+    }
+  } else {
+    const int lo = max(0, c - k), hi = min(nc - 1, c + k);
+    for (int o = lo; o <= hi; ++o) {
+      cell[n] = o; sh[n] = 0.0f; unit[n] = max(abs(o - c) - 1, 0); off[n] = o - c; ++n;
+    }
+  }
+  return n;
 }
 
 // One thread per atom.  Radial entries go to a scratch list tagged with the
@@ -419,6 +466,22 @@ __global__ void __launch_bounds__(128) k_build(NbrArgs a, const int* sorted_cell
   const int s = a.sorted_struct[i];
   const StructGrid G = a.grids[s];
   const int lc = sorted_cell[i] - G.cell_offset;
+  const int cx = lc % G.nc[0], cy = (lc / G.nc[0]) % G.nc[1], cz = lc / (G.nc[0] * G.nc[1]);
+  const int k = a.cell_div;
+  const int kx = k == 1 ? a.x_div : k;  // x_div subdivides x only, and only with cell_div = 1
+  int xc[9], yc[7], zc[7], xu[9], yu[7], zu[7], xo[9], yo[7], zo[7];
+  float xs[9], ys[7], zs[7];
+  int nx = axis_stencil(cx, G.nc[0], G.L[0], kx, xc, xs, xu, xo);
+  int ny = axis_stencil(cy, G.nc[1], G.L[1], k, yc, ys, yu, yo);
+  int nz = axis_stencil(cz, G.nc[2], G.L[2], k, zc, zs, zu, zo);
+  // stencil cells farther than the cutoff from the centre cell are skipped
+  const float ex = 1.0f / G.cinv[0], ey = 1.0f / G.cinv[1], ez = 1.0f / G.cinv[2];
+  // The shift of a stencil cell equals L * rint((p_j - p_i) / L) for every pair
+  // the cutoff can accept when all coordinates lie in [0, L); otherwise (or
+  // when an axis has too few cells to carry shifts) use rint per pair.  Both
+  // give the float32 rule of the header bit for bit.
+  const bool use_rint = nx < 0 || ny < 0 || nz < 0 || (a.struct_flags[s] & 1);
+  nx = abs(nx); ny = abs(ny); nz = abs(nz);
   // scratch entry e of this thread lives at wR[e * ws]
   int* wR = a.nbr_tmp + (size_t)(i >> 5) * a.cap_R * 32 + (i & 31);
   constexpr int ws = 32;
@@ -476,16 +539,80 @@ __global__ void __launch_bounds__(128) k_build(NbrArgs a, const int* sorted_cell
       }
     }
   };
-  const Stencil sten(a, s, G, lc, pi, rc2R);
-  for (int iz = 0; iz < sten.nz; ++iz)
-    for (int iy = 0; iy < sten.ny; ++iy) sten.row(a, G, iy, iz, scan);
+  if (kx > 1 && k == 1 && !use_rint) {
+    // Window scan: cells are thin along x.  In each (y, z) row of the stencil
+    // only the x-cells meeting [x_i - h, x_i + h] can hold pairs, where
+    // h^2 = rc_R^2 - (distance from atom i to the row)^2; on a periodic axis
+    // the window splits at the box faces into ranges with shifts +L, 0, -L.
+    // A window longer than the row falls back to the whole row with rint.
+    const float xr = pi.x - G.origin[0], yr = pi.y - G.origin[1], zr = pi.z - G.origin[2];
+    const float rcm = a.rc_R + kWindowMargin, rcm2 = rcm * rcm;
+    const int ncx = G.nc[0];
+    for (int iz = 0; iz < nz; ++iz) {
+      const float gz = point_cell_gap(zr, cz, zo[iz], ez);
+      if (gz * gz >= rcm2) continue;
+      for (int iy = 0; iy < ny; ++iy) {
+        const float gy = point_cell_gap(yr, cy, yo[iy], ey);
+        const float h2 = rcm2 - gy * gy - gz * gz;
+        if (h2 <= 0.0f) continue;
+        const float h = sqrtf(h2) + kWindowMargin;
+        int clo = (int)floorf((xr - h) * G.cinv[0]);
+        int chi = (int)floorf((xr + h) * G.cinv[0]);
+        const int row = G.cell_offset + (zc[iz] * G.nc[1] + yc[iy]) * ncx;
+        const float sy = ys[iy], sz = zs[iz];
+        if (G.L[0] > 0.0f) {
+          if (chi - clo + 1 > ncx) {
+            scan(a.cell_start[row], a.cell_start[row + ncx], 0.0f, sy, sz, true);
+            continue;
+          }
+          if (clo < 0) scan(a.cell_start[row + clo + ncx], a.cell_start[row + ncx], G.L[0], sy, sz, false);
+          const int b0 = max(clo, 0), b1 = min(chi, ncx - 1);
+          if (b0 <= b1) scan(a.cell_start[row + b0], a.cell_start[row + b1 + 1], 0.0f, sy, sz, false);
+          if (chi >= ncx) scan(a.cell_start[row], a.cell_start[row + chi - ncx + 1], -G.L[0], sy, sz, false);
+        } else {
+          clo = max(clo, 0);
+          chi = min(chi, ncx - 1);
+          if (clo <= chi) scan(a.cell_start[row + clo], a.cell_start[row + chi + 1], 0.0f, sy, sz, false);
+        }
+      }
+    }
+  } else {
+    for (int iz = 0; iz < nz; ++iz) {
+      const float gz = cell_gap(zu[iz], ez);
+      if (gz * gz >= rc2R) continue;
+      for (int iy = 0; iy < ny; ++iy) {
+        const float gy = cell_gap(yu[iy], ey);
+        const float gyz = gy * gy + gz * gz;
+        if (gyz >= rc2R) continue;
+        const int row = G.cell_offset + (zc[iz] * G.nc[1] + yc[iy]) * G.nc[0];
+        const float sy = ys[iy], sz = zs[iz];
+        int ix = 0;
+        while (ix < nx) {
+          const float gx = cell_gap(xu[ix], ex);
+          if (gx * gx + gyz >= rc2R) { ++ix; continue; }
+          // merge x-cells that are contiguous, within reach and share a shift into one range
+          int ie = ix + 1;
+          while (ie < nx && xc[ie] == xc[ie - 1] + 1 && xs[ie] == xs[ix]) {
+            const float ge = cell_gap(xu[ie], ex);
+            if (ge * ge + gyz >= rc2R) break;
+            ++ie;
+          }
+          const float sx = xs[ix];
+          const int j0 = a.cell_start[row + xc[ix]], j1 = a.cell_start[row + xc[ie - 1] + 1];
+          ix = ie;
+          scan(j0, j1, sx, sy, sz, use_rint);
+        }
+      }
+    }
+  }
   a.cnt_R[i] = cR;
   a.cnt_A[i] = cA;
   if (cR > a.cap_R) atomicMax(&a.status->max_cnt_R, cR);
   if (cA > a.cap_A) atomicMax(&a.status->max_cnt_A, cA);
   if constexpr (TWO) {
-    a.seg_R[i] = cR - c1;
-    a.seg_R[(size_t)a.seg_stride + i] = c1;
+    // (clipped to the row: readers stay in it when the lists overflowed)
+    a.seg_R[i] = min(cR - c1, a.cap_R);
+    a.seg_R[(size_t)a.seg_stride + i] = min(c1, a.cap_R);
     return;
   }
   // counting sort of the radial entries by neighbour type; the scratch rows
@@ -528,6 +655,244 @@ __global__ void __launch_bounds__(128) k_build(NbrArgs a, const int* sorted_cell
 #pragma unroll
   for (int u = 0; u < kMaxTypes; ++u)
     if (u < a.n_types) a.seg_R[(size_t)u * a.seg_stride + i] = cnt[u];
+}
+
+// A 16-bit counter per type, four to a word.
+struct TypeCounts {
+  unsigned long long w0, w1;
+  __device__ __forceinline__ int get(unsigned t) const {
+    return (int)((t < 4 ? w0 : w1) >> (16 * (t & 3))) & 0xffff;
+  }
+  __device__ __forceinline__ void add(unsigned t, int n) {
+    const unsigned long long v = (unsigned long long)n << (16 * (t & 3));
+    if (t < 4) w0 += v; else w1 += v;
+  }
+};
+
+// The same lists with eight lanes per atom, for batches that do not fill the
+// chip with a thread per atom (rule at launch_neighbor_pipeline), where k_build
+// is a serial scan on a few warps: 49,600 atoms of six types 177 us there.  A CTA of
+// 256 threads takes one 32-atom tile of the lists; the lanes of an atom's group
+// find the stencil rows' ranges, lay the candidates of eight rows end to end
+// and test eight at a time, one ballot a candidate placing what is accepted;
+// types and angular entries are then split from the accepted list, so the
+// orders are those of the serial scan.  (A contiguous eighth of the sequence
+// per lane, without ballots, was slower: 32 lanes then read 32 lines a load.)  Lists are kept in shared memory (with
+// more than two types also grouped by type there: each lane counts a contiguous
+// eighth, a scan over the lanes gives the places) and leave as whole 128-byte
+// rows.  Bound by issue slots.
+constexpr int kGroup = 8, kTile = 32, kGroupThreads = kGroup * kTile;
+constexpr int kGroupRanges = 3 * kGroup;
+// Tagged entries: type in bits 29-31, angular in bit 28, so at most 2^28 atoms.
+constexpr int kAngular = 1 << 28, kBatchMask = kAngular - 1;
+struct GroupRange {
+  int off, end, code;  // candidate j = position + off, for positions before `end`; shifts (2 bits an axis), rint
+};
+__host__ __device__ inline int group_list_words(int cap) { return kTile * (cap + 1); }
+inline size_t group_smem_bytes(int cap_R, int cap_A) {
+  return sizeof(int) * ((size_t)group_list_words(cap_R) * 2 + group_list_words(cap_A)) +
+         sizeof(GroupRange) * kTile * kGroupRanges;
+}
+
+__global__ void __launch_bounds__(kGroupThreads) k_build_group(const __grid_constant__ NbrArgs a,
+                                                               const int* __restrict__ sorted_cell, float rc2R,
+                                                               float rc2A) {
+  extern __shared__ int sm_group[];
+  __shared__ int s_front[kTile], s_back[kTile], s_ang[kTile];
+  const int T = a.n_types;
+  int* listR = sm_group;                                         // grouped by type
+  int* listT = listR + group_list_words(a.cap_R);                // append order, tagged: type, angular
+  int* listA = listT + group_list_words(a.cap_R);
+  GroupRange* all = reinterpret_cast<GroupRange*>(listA + group_list_words(a.cap_A));
+  const int g = threadIdx.x / kGroup, l = threadIdx.x % kGroup;
+  const int i0 = blockIdx.x * kTile, i = i0 + g;
+  const bool valid = i < a.n_atoms;
+  const int ii = valid ? i : a.n_atoms - 1;
+  int* gR = listR + g * (a.cap_R + 1);
+  int* gT = listT + g * (a.cap_R + 1);
+  int* gA = listA + g * (a.cap_A + 1);
+  GroupRange* ranges = all + g * kGroupRanges;
+  const float4 pi = a.pos4[ii];
+  const int s = a.sorted_struct[ii];
+  const StructGrid G = a.grids[s];
+  const Stencil sten(a, s, G, sorted_cell[ii] - G.cell_offset, pi, rc2R);
+  const int rows = valid ? sten.rows() : 0;
+  int nR = 0;
+  const unsigned below = (1u << l) - 1u;
+  const int sh = threadIdx.x & 24;  // first lane of the group in its warp
+  auto code_of = [](float v) { return v > 0.f ? 1 : (v < 0.f ? 2 : 0); };
+  for (int r0 = 0; __any_sync(0xffffffffu, r0 < rows); r0 += kGroup) {
+    int j0[3] = {0, 0, 0}, len[3] = {0, 0, 0}, code[3] = {0, 0, 0}, nseg = 0;
+    if (r0 + l < rows) {
+      const int iz = (r0 + l) / sten.ny, iy = (r0 + l) - iz * sten.ny;
+      sten.row(a, G, iy, iz, [&](int b, int e, float x, float y, float z, bool rint_pairs) {
+        if (e <= b) return;
+        const int c = code_of(x) | code_of(y) << 2 | code_of(z) << 4 | (rint_pairs ? 64 : 0);
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+          if (u == nseg) { j0[u] = b; len[u] = e - b; code[u] = c; }
+        ++nseg;
+      });
+    }
+    int seg = nseg, pos = len[0] + len[1] + len[2];
+#pragma unroll
+    for (int o = 1; o < kGroup; o <<= 1) {
+      const int us = __shfl_up_sync(0xffffffffu, seg, o, kGroup), up = __shfl_up_sync(0xffffffffu, pos, o, kGroup);
+      if (l >= o) { seg += us; pos += up; }
+    }
+    const int total = __shfl_sync(0xffffffffu, pos, kGroup - 1, kGroup);
+    seg -= nseg;
+    pos -= len[0] + len[1] + len[2];
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      if (u < nseg) {
+        ranges[seg + u] = GroupRange{j0[u] - pos, pos + len[u], code[u]};
+        pos += len[u];
+      }
+    }
+    __syncwarp();
+    const GroupRange* q = ranges - 1;
+    int off = 0, end = 0;
+    float sx = 0.f, sy = 0.f, sz = 0.f;
+    bool rint_pairs = false;
+    for (int p0 = 0; __any_sync(0xffffffffu, p0 < total); p0 += 2 * kGroup) {
+      // two candidates per lane, their loads in flight together
+      int v[2] = {0, 0};
+      bool in[2] = {false, false};
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int p = p0 + u * kGroup + l;
+        if (p < total) {
+          if (p >= end) {
+            do ++q;
+            while (p >= q->end);
+            off = q->off;
+            end = q->end;
+            const int c = q->code;
+            sx = (c & 3) == 1 ? G.L[0] : ((c & 3) == 2 ? -G.L[0] : 0.f);
+            sy = (c & 12) == 4 ? G.L[1] : ((c & 12) == 8 ? -G.L[1] : 0.f);
+            sz = (c & 48) == 16 ? G.L[2] : ((c & 48) == 32 ? -G.L[2] : 0.f);
+            rint_pairs = c & 64;
+          }
+          const int j = p + off;
+          const float4 pj = __ldg(&a.pos4[j]);
+          float dx, dy, dz;
+          if (!rint_pairs) {  // (a zero shift subtracts exactly nothing)
+            dx = __fsub_rn(__fsub_rn(pj.x, pi.x), sx);
+            dy = __fsub_rn(__fsub_rn(pj.y, pi.y), sy);
+            dz = __fsub_rn(__fsub_rn(pj.z, pi.z), sz);
+          } else {
+            dx = mi_diff(pj.x, pi.x, G.L[0], G.invL[0]);
+            dy = mi_diff(pj.y, pi.y, G.L[1], G.invL[1]);
+            dz = mi_diff(pj.z, pi.z, G.L[2], G.invL[2]);
+          }
+          const float r2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+          in[u] = r2 < rc2R && j != i;  // an atom is not its own neighbour
+          v[u] = j | (int)((unsigned)__float_as_int(pj.w) << kTypeShift) | (r2 < rc2A ? kAngular : 0);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const unsigned m = (__ballot_sync(0xffffffffu, in[u]) >> sh) & 0xffu;
+        const int e = nR + __popc(m & below);
+        if (in[u] && e < a.cap_R) gT[e] = v[u];
+        nR += __popc(m);
+      }
+    }
+    __syncwarp();  // the ranges are read before the next rows replace them
+  }
+  // the accepted entries in scan order -> angular list, and for up to two types
+  // the radial list (type 1 from the back)
+  const int n = min(nR, a.cap_R);
+  int c0 = 0, c1 = 0, cA = 0;
+  __syncwarp();
+  for (int e0 = 0; __any_sync(0xffffffffu, e0 < n); e0 += kGroup) {
+    const bool on = e0 + l < n;
+    const int v = on ? gT[e0 + l] : 0, j = v & kBatchMask;
+    const unsigned mA = (__ballot_sync(0xffffffffu, on && (v & kAngular)) >> sh) & 0xffu;
+    if (on && (v & kAngular)) {
+      const int e = cA + __popc(mA & below);
+      if (e < a.cap_A) gA[e] = j;
+    }
+    cA += __popc(mA);
+    if (T <= 2) {
+      const bool one = T == 2 && ((unsigned)v >> kTypeShift) != 0;
+      const unsigned m0 = (__ballot_sync(0xffffffffu, on && !one) >> sh) & 0xffu;
+      const unsigned m1 = (__ballot_sync(0xffffffffu, on && one) >> sh) & 0xffu;
+      if (on) {
+        if (one) gR[a.cap_R - 1 - (c1 + __popc(m1 & below))] = j;
+        else gR[c0 + __popc(m0 & below)] = j;
+      }
+      c0 += __popc(m0);
+      c1 += __popc(m1);
+    }
+  }
+  if (valid && l == 0) {
+    a.cnt_R[i] = nR;
+    a.cnt_A[i] = cA;
+    if (nR > a.cap_R) atomicMax(&a.status->max_cnt_R, nR);
+    if (cA > a.cap_A) atomicMax(&a.status->max_cnt_A, cA);
+    if (T <= 2) a.seg_R[i] = c0;
+    if (T == 2) a.seg_R[(size_t)a.seg_stride + i] = c1;
+  }
+  if (T > 2) {
+    // stable counting sort: 16-bit counts of four types per word
+    const int per = (n + kGroup - 1) / kGroup, b = min(n, l * per), e = min(n, b + per);
+    TypeCounts cnt{};
+    for (int k = b; k < e; ++k) cnt.add((unsigned)gT[k] >> kTypeShift, 1);
+    TypeCounts inc = cnt;
+#pragma unroll
+    for (int o = 1; o < kGroup; o <<= 1) {
+      const unsigned long long x = __shfl_up_sync(0xffffffffu, inc.w0, o, kGroup);
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, inc.w1, o, kGroup);
+      if (l >= o) { inc.w0 += x; inc.w1 += y; }
+    }
+    const TypeCounts tot{__shfl_sync(0xffffffffu, inc.w0, kGroup - 1, kGroup),
+                         __shfl_sync(0xffffffffu, inc.w1, kGroup - 1, kGroup)};
+    // next place of every type for this lane's entries
+    TypeCounts at{inc.w0 - cnt.w0, inc.w1 - cnt.w1};
+    int run = 0;
+#pragma unroll
+    for (int t = 0; t < kMaxTypes; ++t) {
+      const int c = tot.get(t);
+      at.add(t, run);
+      if (valid && t < T && l == t) a.seg_R[(size_t)t * a.seg_stride + i] = c;
+      run += c;
+    }
+    for (int k = b; k < e; ++k) {
+      const int v = gT[k];
+      const unsigned t = (unsigned)v >> kTypeShift;
+      gR[at.get(t)] = v & kBatchMask;
+      at.add(t, 1);
+    }
+  }
+  if (l == 0) {
+    s_front[g] = valid ? (T == 2 ? c0 : n) : 0;
+    s_back[g] = valid ? c1 : 0;
+    s_ang[g] = valid ? min(cA, a.cap_A) : 0;
+  }
+  __syncthreads();
+  // rows of the tile, one warp a row: lane = atom
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int front = s_front[lane], back = s_back[lane], ang = s_ang[lane];
+  int mf = front, mb = back, ma = ang;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    mf = max(mf, __shfl_xor_sync(0xffffffffu, mf, o));
+    mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+    ma = max(ma, __shfl_xor_sync(0xffffffffu, ma, o));
+  }
+  const int* lR = listR + lane * (a.cap_R + 1);
+  const int* lA = listA + lane * (a.cap_A + 1);
+  int* outR = a.nbr_R + (size_t)blockIdx.x * a.cap_R * kTile + lane;
+  int* outA = a.nbr_A + (size_t)blockIdx.x * a.cap_A * kTile + lane;
+  for (int k = w; k < mf; k += kGroupThreads / 32)
+    if (k < front) outR[(size_t)k * kTile] = lR[k];
+  for (int k = w; k < mb; k += kGroupThreads / 32)
+    if (k < back) outR[(size_t)(a.cap_R - 1 - k) * kTile] = lR[a.cap_R - 1 - k];
+  for (int k = w; k < ma; k += kGroupThreads / 32)
+    if (k < ang) outA[(size_t)k * kTile] = lA[k];
 }
 
 // Frames of a pass in the first frame's cell order, with their boxes.
@@ -652,7 +1017,7 @@ cudaError_t launch_neighbor_pipeline(const NbrArgs& a, bool build, cudaStream_t 
                                                (int)sizeof(int) * (4 * kSmallStruct + 9));
     if (e != cudaSuccess) return e;
     count_launches(1);
-    k_prep_small<<<S, kSmallThreads, smem, st>>>(a, a.atom_slot);
+    k_prep_small<<<S, a.max_struct <= 1024 ? 256 : kSmallThreads, smem, st>>>(a, a.atom_slot);
   } else {
     count_launches(6);
     k_plan<<<S, 256, 0, st>>>(a);
@@ -660,7 +1025,7 @@ cudaError_t launch_neighbor_pipeline(const NbrArgs& a, bool build, cudaStream_t 
     // The number of cells in use is known only on the device; the cell scan
     // and the per-cell sort read it from struct_cells[S].
     k_bin<<<(N + 255) / 256, 256, 0, st>>>(a);
-    k_scan_cells<<<1, 1024, 0, st>>>(a);
+    k_scan_cells<<<S, 1024, 0, st>>>(a);
     k_scatter<<<(N + 255) / 256, 256, 0, st>>>(a);
     // sorted_cell reuses atom_slot (dead after the scatter)
     k_cell_sort<<<1216, 256, 0, st>>>(a, a.atom_slot);
@@ -668,7 +1033,13 @@ cudaError_t launch_neighbor_pipeline(const NbrArgs& a, bool build, cudaStream_t 
   if (N > 0 && build) {
     count_launches(1);
     const float rc2R = a.rc_R * a.rc_R, rc2A = a.rc_A * a.rc_A;
-    if (a.two_ended)
+    const size_t smem = group_smem_bytes(a.cap_R, a.cap_A);
+    if (N <= (a.n_types <= 2 ? kGroupAtoms2 : kGroupAtoms) && smem <= kGroupMaxSmem) {
+      const cudaError_t e = cudaFuncSetAttribute(k_build_group, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)kGroupMaxSmem);
+      if (e != cudaSuccess) return e;
+      k_build_group<<<(N + kTile - 1) / kTile, kGroupThreads, smem, st>>>(a, a.atom_slot, rc2R, rc2A);
+    } else if (a.two_ended)
       k_build<true><<<(N + 127) / 128, 128, 0, st>>>(a, a.atom_slot, rc2R, rc2A);
     else
       k_build<false><<<(N + 127) / 128, 128, 0, st>>>(a, a.atom_slot, rc2R, rc2A);

@@ -51,9 +51,9 @@ __host__ __device__ __forceinline__ size_t nbr_index(int i, int k, int cap) {
 }
 
 // Arguments of the neighbour-list pipeline.
-// Structures up to this size are prepared by one CTA each (nbr.cu): a cell's
-// atom slot takes 12 bits, and 64 KB of shared memory hold the counts.
-constexpr int kSmallStruct = 4095;
+// Structures up to this size are prepared by one CTA each (nbr.cu): their cells
+// and atoms take 224 of the 227 KB of shared memory.
+constexpr int kSmallStruct = 14000;
 struct NbrArgs {
   int n_structs;
   int n_atoms;

@@ -1,6 +1,6 @@
 """Routes that are chosen by the sizes of a batch give the same bits.
 
-Structures of at most 4095 atoms are prepared by one CTA each, batches with a
+Structures of at most 14000 atoms are prepared by one CTA each, batches with a
 larger one by the general pipeline; atom order, lists and sums are defined to
 be the same, so a structure's tensors and per-atom contributions must not
 depend on what else is in the batch (exact comparison, no tolerance).  Batches
@@ -42,7 +42,7 @@ def context(tn, n_types, precision, seed=3):
 @pytest.mark.parametrize("precision", [0, 2])
 def test_a_structure_alone_and_beside_a_large_one(tn, n_types, precision):
     rng = np.random.default_rng(11)
-    structs = [water(1366, rng, 2), water(1366, rng, 3), water(64, rng), water(65, rng, 1)]  # 4096, 4095, 192, 194 atoms
+    structs = [water(4667, rng), water(4667, rng, 1), water(345, rng, 11), water(342, rng, 2), water(65, rng, 1)]  # 14001, 14000, 1024, 1024, 194 atoms
     p, t, b = synth.water_cluster(7, rng)
     structs.append(synth.Structure(p.astype(np.float32), t, b.astype(np.float32)))
     structs.append(synth.Structure(np.zeros((0, 3), np.float32), np.zeros(0, np.int32), np.zeros(3, np.float32)))
