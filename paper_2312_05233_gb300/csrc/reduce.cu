@@ -23,7 +23,8 @@ namespace {
 // half-warp adding one and the upper half the other, which needs 12 additions
 // for nine components instead of 45.
 struct ReduceArgs {
-  ReduceModel m[4];       // blockIdx.z
+  ReduceModel m[4];
+  int split;              // blockIdx.z: model, or (split) 3 * model + group of three components
   const int* offsets;
   int S, n_chunks;
   size_t pa_pop_stride, out_pop_stride;  // individuals (blockIdx.y)
@@ -59,46 +60,49 @@ __device__ __forceinline__ double warp_tree(const double* v, int lane) {
   return t[0] + __shfl_xor_sync(0xffffffffu, t[0], 1);
 }
 
-template <int C>
-__device__ __forceinline__ void reduce_chunk(const ReduceArgs& a, const ReduceModel& m) {
+// Components [c0, c0 + NC) of model `mi`, which has C.
+template <int NC>
+__device__ __forceinline__ void reduce_chunk(const ReduceArgs& a, const ReduceModel& m, int mi, int C, int c0) {
   const int s = blockIdx.x / a.n_chunks, chunk = blockIdx.x % a.n_chunks, p = blockIdx.y;
   const int a0 = a.offsets[s] + chunk * kReduceChunk;
   const int a1 = min(a.offsets[s + 1], a0 + kReduceChunk);
-  const float* pa = m.per_atom + (size_t)p * a.pa_pop_stride;
+  const float* pa = m.per_atom + (size_t)p * a.pa_pop_stride + (size_t)c0 * a.atom_stride;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   __shared__ double red[9][8];
   // warps past the chunk's end hold zeros
   const bool any = a0 + 32 * w < a1;
   double v = 0.0;
   if (any) {
-    double acc[C];
+    double acc[NC];
 #pragma unroll
-    for (int c = 0; c < C; ++c) acc[c] = 0.0;
+    for (int c = 0; c < NC; ++c) acc[c] = 0.0;
     for (int g = a0 + threadIdx.x; g < a1; g += blockDim.x) {
 #pragma unroll
-      for (int c = 0; c < C; ++c) acc[c] += (double)pa[(size_t)c * a.atom_stride + g];
+      for (int c = 0; c < NC; ++c) acc[c] += (double)pa[(size_t)c * a.atom_stride + g];
     }
-    v = warp_tree<C>(acc, lane);
+    v = warp_tree<NC>(acc, lane);
   }
 #pragma unroll
-  for (int c = 0; c < C; ++c)
+  for (int c = 0; c < NC; ++c)
     if (lane == lane_of(c)) red[c][w] = v;
   __syncthreads();
-  if (threadIdx.x < C) {
+  if (threadIdx.x < NC) {
     double t = 0.0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) t += red[threadIdx.x][k];
     if (a.n_chunks == 1)
-      m.out[(size_t)p * a.out_pop_stride + (size_t)s * C + threadIdx.x] = t;
+      m.out[(size_t)p * a.out_pop_stride + (size_t)s * C + c0 + threadIdx.x] = t;
     else
-      a.partial[((((size_t)blockIdx.z * gridDim.y + p) * a.S + s) * a.n_chunks + chunk) * 9 + threadIdx.x] = t;
+      a.partial[((((size_t)mi * gridDim.y + p) * a.S + s) * a.n_chunks + chunk) * 9 + c0 + threadIdx.x] = t;
   }
 }
 
 __global__ void __launch_bounds__(256) k_reduce_partial(const __grid_constant__ ReduceArgs a) {
-  const ReduceModel m = a.m[blockIdx.z];
-  if (m.C == 3) reduce_chunk<3>(a, m);
-  else reduce_chunk<9>(a, m);
+  const int mi = a.split ? blockIdx.z / 3 : blockIdx.z, c0 = a.split ? 3 * (blockIdx.z % 3) : 0;
+  const ReduceModel m = a.m[mi];
+  if (c0 >= m.C) return;
+  if (a.split || m.C == 3) reduce_chunk<3>(a, m, mi, m.C, c0);
+  else reduce_chunk<9>(a, m, mi, 9, 0);
 }
 
 // One warp per (model, individual, structure).
@@ -123,7 +127,10 @@ __global__ void k_reduce_final(const __grid_constant__ ReduceArgs a, int n_pop) 
 
 cudaError_t launch_reduce_args(ReduceArgs& a, int n_models, int n_pop, cudaStream_t st) {
   count_launches(a.n_chunks == 1 ? 1 : 2);
-  k_reduce_partial<<<dim3(a.S * a.n_chunks, n_pop, n_models), 256, 0, st>>>(a);
+  // few CTAs: three components each (20 structures of 8,640 atoms, rank 2: 21 us
+  // with 100 CTAs of nine); many: all nine, whose folded tree costs less
+  a.split = (long long)a.S * a.n_chunks * n_pop * n_models <= 608;
+  k_reduce_partial<<<dim3(a.S * a.n_chunks, n_pop, n_models * (a.split ? 3 : 1)), 256, 0, st>>>(a);
   if (a.n_chunks > 1) {
     const long long nt = 32LL * a.S * n_pop;
     k_reduce_final<<<dim3((unsigned)((nt + 127) / 128), 1, n_models), 128, 0, st>>>(a, n_pop);
