@@ -27,8 +27,11 @@ __global__ void __launch_bounds__(128, 3) k_radial(const __grid_constant__ Radia
   const float rcinv = 1.f / a.rc_R;
   float* mom = a.mom + i;
   const size_t ms = a.mom_stride;
+  // all types, or (grid.y = n_types) type blockIdx.y alone
+  const int t0 = gridDim.y > 1 ? blockIdx.y : 0, t1 = gridDim.y > 1 ? t0 + 1 : a.n_types;
   int start = 0;
-  for (int t = 0; t < a.n_types; ++t) {
+  for (int t = 0; t < t0; ++t) start += a.seg_R[(size_t)t * a.seg_stride + i];
+  for (int t = t0; t < t1; ++t) {
     const int n = a.seg_R[(size_t)t * a.seg_stride + i];
     // accumulators in basis pairs (k = 2q, 2q + 1), one packed multiply-add
     // per pair; the last index of an odd basis size is accumulated alone
@@ -160,12 +163,17 @@ __global__ void __launch_bounds__(128, 3) k_radial(const __grid_constant__ Radia
   }
 }
 
+// Up to one wave (three CTAs on each SM) every type gets a thread of its own:
+// the kernel then lasts as long as one type's walk instead of all of them.
+constexpr int kSplitBlocks = 456;
+
 }  // namespace
 
 cudaError_t launch_radial_moments(const RadialArgs& a, cudaStream_t st) {
   if (a.n_atoms <= 0) return cudaSuccess;
   count_launches(1);
-  const int grid = (a.n_atoms + 127) / 128;
+  const int blocks = (a.n_atoms + 127) / 128;
+  const dim3 grid(blocks, blocks <= kSplitBlocks ? a.n_types : 1);
   const bool hv = a.v0 >= 0, hw = a.w0 >= 0;
   if (hv && hw) k_radial<true, true><<<grid, 128, 0, st>>>(a);
   else if (hv) k_radial<true, false><<<grid, 128, 0, st>>>(a);
