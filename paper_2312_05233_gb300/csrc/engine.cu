@@ -464,6 +464,7 @@ FusedArgs fused_args(tnep_ctx* c, Workspace& w, const Model& m, int N) {
   f.v0 = w.mom_v0;
   f.w0 = w.mom_w0;
   f.status = w.d_status;
+  f.work_next = w.d_status->work_next;
   f.nbr_A = w.nbr_A.p;
   f.cnt_A = w.cnt_A.p;
   f.cap_A = w.cap_A;
@@ -559,6 +560,23 @@ static tnep_status run_wide(tnep_ctx* c, Workspace& w, cudaStream_t st, const un
   return TNEP_OK;
 }
 
+// The workspace's side stream, ordered after what st holds now.
+static tnep_status fork_side(Workspace& w, cudaStream_t st) {
+  if (!w.side) TNEP_CUDA(cudaStreamCreateWithFlags(&w.side, cudaStreamNonBlocking));
+  if (!w.ev_fork) TNEP_CUDA(cudaEventCreateWithFlags(&w.ev_fork, cudaEventDisableTiming));
+  if (!w.ev_join) TNEP_CUDA(cudaEventCreateWithFlags(&w.ev_join, cudaEventDisableTiming));
+  TNEP_CUDA(cudaEventRecord(w.ev_fork, st));
+  TNEP_CUDA(cudaStreamWaitEvent(w.side, w.ev_fork, 0));
+  return TNEP_OK;
+}
+
+// What st holds next comes after the side stream's work.
+static tnep_status join_side(Workspace& w, cudaStream_t st) {
+  TNEP_CUDA(cudaEventRecord(w.ev_join, w.side));
+  TNEP_CUDA(cudaStreamWaitEvent(st, w.ev_join, 0));
+  return TNEP_OK;
+}
+
 tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N, cudaEvent_t ev_done,
                        const unsigned char* ghost, cudaStream_t red_st) {
   const size_t per_model = (size_t)9 * w.atom_stride;
@@ -588,17 +606,30 @@ tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N,
     const int pc_stride = round_up(std::max(N, 1), 128);
     const size_t pc_elems = (size_t)w.cap_A * quads * pc_stride;
     const bool use_pc = c->pair_cache && pc_elems * sizeof(float4) <= kPairCacheMaxBytes;
-    if (use_pc) TNEP_CUDA(w.pcache.ensure(pc_elems));
-    for (size_t k = 0; k < c->models.size(); ++k) {
+    std::vector<size_t> run;
+    for (size_t k = 0; k < c->models.size(); ++k)
+      if (!(w.wide && c->models[k].d.mlp_precision == 0)) run.push_back(k);
+    // Batches of a few waves: every other model on a side stream (with a pair
+    // cache and a work counter of its own), so that one model's CTAs fill the
+    // slots the other leaves.
+    const bool fork = run.size() > 1 && N <= kForkAtoms;
+    if (use_pc) TNEP_CUDA(w.pcache.ensure(pc_elems * (fork ? 2 : 1)));
+    if (fork) TNEP_TRY(fork_side(w, st));
+    cudaError_t e = cudaSuccess;
+    for (size_t r = 0; r < run.size() && e == cudaSuccess; ++r) {
+      const size_t k = run[r];
       const Model& m = c->models[k];
-      if (w.wide && m.d.mlp_precision == 0) continue;
+      const int side = fork ? (int)(r & 1) : 0;
       FusedArgs f = fused_args(c, w, m, N);
       f.per_atom = w.per_atom.p + k * per_model;
       f.per_atom_stride = 0;
-      f.pcache = use_pc ? w.pcache.p : nullptr;
+      f.pcache = use_pc ? w.pcache.p + side * pc_elems : nullptr;
       f.pc_stride = pc_stride;
-      TNEP_CUDA(launch_fused(m.variant, m.d.rank, f, 1, c->block_atoms, m.d.mlp_precision, st));
+      f.work_next += side;
+      e = launch_fused(m.variant, m.d.rank, f, 1, c->block_atoms, m.d.mlp_precision, side ? w.side : st);
     }
+    if (fork) TNEP_TRY(join_side(w, st));  // also after a failed launch: nothing is left behind on the side stream
+    TNEP_CUDA(e);
   }
   if (ev_done) TNEP_CUDA(cudaEventRecord(ev_done, st));
   if (ghost && thread_per_atom)

@@ -102,6 +102,10 @@ struct Model {
   float* d_w0t = nullptr;  // W0 as the warp-per-atom path reads it (see WideArgs)
 };
 
+// Largest batch whose models run on two streams: 1,024 CTAs of the fused kernel
+// a model on 304 slots.
+constexpr int kForkAtoms = 131072;
+
 // Device workspace of one in-flight batch.
 struct Workspace {
   DevBuf<int> offsets, atom_struct, atom_cell, atom_slot, cell_count, cell_start, cell_atoms;
@@ -129,6 +133,9 @@ struct Workspace {
   PinBuf<float> h_box;
   cudaEvent_t ev_pin = nullptr;
   bool pin_read = false;
+  // every other model of a small batch runs on `side`, between two events
+  cudaStream_t side = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int atom_stride = 0;
   int cells_cap = 0;
   int cap_R = 0, cap_A = 0;  // caps the lists were built with
@@ -151,6 +158,14 @@ struct Workspace {
     if (ev_pin) cudaEventDestroy(ev_pin);
     ev_pin = nullptr;
     pin_read = false;
+    if (side) {
+      cudaStreamSynchronize(side);
+      cudaStreamDestroy(side);
+    }
+    side = nullptr;
+    if (ev_fork) cudaEventDestroy(ev_fork);
+    if (ev_join) cudaEventDestroy(ev_join);
+    ev_fork = ev_join = nullptr;
   }
 };
 

@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(BLK, 256 / BLK) k_fused(const __grid_constant_
   // varies fastest so that CTAs running together share an atom block's lists.
   // Without the tensor cores each CTA takes item blockIdx.x.  With them the
   // CTAs are persistent: each starts with item blockIdx.x and takes the next
-  // from the counter a.status->work_next (gridDim.x + its value, zeroed before
+  // from the counter *a.work_next (gridDim.x + its value, zeroed before
   // the launch), fetched by thread 0 between the two network products and
   // handed to the CTA through shared memory across the second product's
   // barrier; the model, the weight tiles made from it, the mbarrier and the
@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(BLK, 256 / BLK) k_fused(const __grid_constant_
     if (ok) {
       // the next work item; its latency is hidden behind the network
       int nxt = 0;
-      if (tid == 0) nxt = (int)gridDim.x + atomicAdd(&a.status->work_next, 1);
+      if (tid == 0) nxt = (int)gridDim.x + atomicAdd(a.work_next, 1);
 #pragma unroll
       for (int k = 0; k < 32; ++k) z[k] = 0.f;
       read_row(z);
@@ -786,12 +786,12 @@ cudaError_t launch_block(int rank, const FusedArgs& a_in, int n_pop, size_t smem
   if (e != cudaSuccess) return e;
   dim3 grid;
   if constexpr (TCM != 0) {
-    if (!a.status) return cudaErrorInvalidValue;
+    if (!a.status || !a.work_next) return cudaErrorInvalidValue;
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     grid = dim3((unsigned)std::min<long long>(n_work, 2LL * sms));
-    e = cudaMemsetAsync(&a.status->work_next, 0, sizeof(int), st);
+    e = cudaMemsetAsync(a.work_next, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
   } else {
     const int nblk = (a.n_atoms + BLK - 1) / BLK;

@@ -24,7 +24,7 @@ struct DevStatus {
   int max_cnt_R;    // largest radial neighbour count seen above the cap
   int max_cnt_A;    // largest angular neighbour count seen above the cap
   int skin_violation;  // an atom moved more than skin / 2 (or the box changed) within a pass
-  int work_next;    // work counter of the persistent fused kernel (zeroed before each of its launches)
+  int work_next[2];  // work counters of the persistent fused kernel, one per stream (zeroed before each launch)
 };
 
 // Per-structure cell grid (orthorhombic, periodic or open per axis).
@@ -195,6 +195,7 @@ struct FusedArgs {
   int n_pop;                 // individuals (set by the launcher)
   const float* amom; int amom_slots;   // angular moments (factored population path), else null
   DevStatus* status;         // error word (bounded waits of the tensor-core path)
+  int* work_next;            // work counter of the tensor-core path's persistent CTAs
   long long wait_tries;      // try_wait limit of the tensor-core network's product waits
   // Per-pair cache of the angular walk (single-individual launches, else
   // null): the forward walk stores, for pair k of atom i, r_ij and 1/|r_ij|,
