@@ -12,11 +12,10 @@
 // the contributions of the image atoms ("ghosts") are zeroed before the
 // per-structure reduction, so only the cell's own atoms are summed.
 //
-//   k_cell_plan     per structure: H^-1, plane spacings, delta (float64)
-//   k_cell_expand   one CTA per structure, atoms in chunks of 256: per atom
-//                   the image ranges, a block-wide scan of the counts, then
-//                   (write pass) the wrapped atom and its images in a fixed
-//                   order (atom, then n0, n1, n2)
+//   k_cell_count    one CTA per structure: H^-1, plane spacings, delta
+//                   (float64), and where each atom's images start
+//   k_cell_expand   one warp per atom: the wrapped atom and its images in a
+//                   fixed order (atom, then n0, n1, n2)
 //   k_zero_ghosts   per sorted atom of the expanded batch
 
 #include <cuda_runtime.h>
@@ -39,10 +38,8 @@ struct CellInfo {
 
 constexpr int kExpandThreads = 256;
 
-__global__ void k_cell_plan(int S, const float* __restrict__ cell, float rc, CellInfo* __restrict__ info,
-                            DevStatus* status) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= S) return;
+// H^-1, plane spacings and delta (float64) of structure s.
+__device__ CellInfo plan_cell(int s, const float* __restrict__ cell, float rc, DevStatus* status) {
   CellInfo ci{};
   bool any = false;
   for (int k = 0; k < 9; ++k) {
@@ -75,12 +72,13 @@ __global__ void k_cell_plan(int S, const float* __restrict__ cell, float rc, Cel
       for (int a = 0; a < 3; ++a) ci.delta[a] = (double)rc / (vol / nrm[a]) + 1e-6;
     }
   }
-  info[s] = ci;
+  return ci;
 }
 
 __device__ __forceinline__ void frac_of(const CellInfo& ci, const float* p, double* sf) {
   for (int a = 0; a < 3; ++a) {
-    const double v = (double)p[0] * ci.Hinv[a] + (double)p[1] * ci.Hinv[3 + a] + (double)p[2] * ci.Hinv[6 + a];
+    const double v = fma((double)p[2], ci.Hinv[6 + a],
+                         fma((double)p[0], ci.Hinv[a], __dmul_rn((double)p[1], ci.Hinv[3 + a])));
     sf[a] = v - floor(v);
   }
 }
@@ -91,85 +89,118 @@ __device__ __forceinline__ void image_range(double s, double delta, int& lo, int
   hi = (int)ceil(1.0 + delta - s) - 1;
 }
 
-// count pass (out_pos == nullptr): n_ghost[s]; write pass: expanded atoms.
-__global__ void __launch_bounds__(kExpandThreads) k_cell_expand(int S, const int* __restrict__ off,
-                                                                const float* __restrict__ pos,
-                                                                const int* __restrict__ types,
-                                                                const CellInfo* __restrict__ info,
-                                                                int* __restrict__ n_ghost,
-                                                                const int* __restrict__ new_off,
-                                                                float* __restrict__ out_pos,
-                                                                int* __restrict__ out_types,
-                                                                unsigned char* __restrict__ ghost) {
-  __shared__ int scan[kExpandThreads];
-  __shared__ int base_sh;
-  const int s = blockIdx.x;
+// One CTA per structure: its plan, and per atom the first of its images among
+// the structure's (exclusive scan of the image counts in atom order);
+// n_ghost[s] is their sum.
+__global__ void __launch_bounds__(kExpandThreads) k_cell_count(const int* __restrict__ off,
+                                                               const float* __restrict__ pos,
+                                                               const float* __restrict__ cell, float rc,
+                                                               CellInfo* __restrict__ info, int* __restrict__ first,
+                                                               int* __restrict__ atom_struct,
+                                                               int* __restrict__ n_ghost, DevStatus* status) {
+  __shared__ int warp_sums[kExpandThreads / 32];
+  __shared__ CellInfo ci_sh;
+  const int s = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int a0 = off[s], a1 = off[s + 1], n = a1 - a0;
-  const CellInfo ci = info[s];
-  const int o0 = new_off ? new_off[s] : 0;
-  // the structure's own atoms first
-  if (out_pos) {
-    for (int k = threadIdx.x; k < n; k += kExpandThreads) {
-      const int a = a0 + k;
-      float* q = out_pos + 3 * (size_t)(o0 + k);
-      if (ci.periodic) {
-        double sf[3];
-        frac_of(ci, pos + 3 * (size_t)a, sf);
-        for (int c = 0; c < 3; ++c)
-          q[c] = (float)(sf[0] * ci.H[c] + sf[1] * ci.H[3 + c] + sf[2] * ci.H[6 + c]);
-      } else {
-        q[0] = pos[3 * (size_t)a]; q[1] = pos[3 * (size_t)a + 1]; q[2] = pos[3 * (size_t)a + 2];
-      }
-      out_types[o0 + k] = types[a];
-      ghost[o0 + k] = 0;
-    }
+  if (threadIdx.x == 0) {
+    ci_sh = plan_cell(s, cell, rc, status);
+    info[s] = ci_sh;
   }
-  if (!ci.periodic) {
-    if (!out_pos && threadIdx.x == 0) n_ghost[s] = 0;
-    return;
-  }
-  if (threadIdx.x == 0) base_sh = 0;
   __syncthreads();
+  const CellInfo ci = ci_sh;
+  int carry = 0;
   for (int c0 = 0; c0 < n; c0 += kExpandThreads) {
     const int k = c0 + threadIdx.x;
-    int cnt = 0, lo[3] = {0, 0, 0}, hi[3] = {-1, -1, -1};
-    double sf[3] = {0.0, 0.0, 0.0};
-    if (k < n) {
+    int cnt = 0;
+    if (k < n && ci.periodic) {
+      double sf[3];
       frac_of(ci, pos + 3 * (size_t)(a0 + k), sf);
-      for (int a = 0; a < 3; ++a) image_range(sf[a], ci.delta[a], lo[a], hi[a]);
-      cnt = (hi[0] - lo[0] + 1) * (hi[1] - lo[1] + 1) * (hi[2] - lo[2] + 1) - 1;  // n = 0 is the atom itself
+      cnt = 1;
+      for (int a = 0; a < 3; ++a) {
+        int lo, hi;
+        image_range(sf[a], ci.delta[a], lo, hi);
+        cnt *= hi - lo + 1;
+      }
+      --cnt;  // n = 0 is the atom itself
     }
-    scan[threadIdx.x] = cnt;
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane == 31) warp_sums[w] = incl;
     __syncthreads();
-    // inclusive Hillis-Steele scan (fixed order)
-    for (int w = 1; w < kExpandThreads; w <<= 1) {
-      const int v = threadIdx.x >= w ? scan[threadIdx.x - w] : 0;
-      __syncthreads();
-      scan[threadIdx.x] += v;
-      __syncthreads();
+    int before = carry;
+    for (int u = 0; u < kExpandThreads / 32; ++u) {
+      if (u < w) before += warp_sums[u];
+      carry += warp_sums[u];
     }
-    const int excl = scan[threadIdx.x] - cnt;
-    const int base = base_sh;
-    if (out_pos && cnt > 0) {
-      int g = o0 + n + base + excl;
-      const int t = types[a0 + k];
-      for (int n0 = lo[0]; n0 <= hi[0]; ++n0)
-        for (int n1 = lo[1]; n1 <= hi[1]; ++n1)
-          for (int n2 = lo[2]; n2 <= hi[2]; ++n2) {
-            if (n0 == 0 && n1 == 0 && n2 == 0) continue;
-            const double f0 = sf[0] + n0, f1 = sf[1] + n1, f2 = sf[2] + n2;
-            float* q = out_pos + 3 * (size_t)g;
-            for (int c = 0; c < 3; ++c) q[c] = (float)(f0 * ci.H[c] + f1 * ci.H[3 + c] + f2 * ci.H[6 + c]);
-            out_types[g] = t;
-            ghost[g] = 1;
-            ++g;
-          }
+    if (k < n) {
+      first[a0 + k] = before + incl - cnt;
+      atom_struct[a0 + k] = s;
     }
-    __syncthreads();
-    if (threadIdx.x == kExpandThreads - 1) base_sh = base + scan[kExpandThreads - 1];
     __syncthreads();
   }
-  if (!out_pos && threadIdx.x == 0) n_ghost[s] = base_sh;
+  if (threadIdx.x == 0) n_ghost[s] = carry;
+}
+
+// One warp per atom: the wrapped atom at its own place (the structure's atoms
+// come first, active[] holds these places) and its images, lane by lane, in the
+// order of n0, n1, n2.  (One CTA per structure with a serial loop over the
+// images of each atom took 48 us for 24 small cells.)
+__global__ void __launch_bounds__(128) k_cell_expand(int N, const int* __restrict__ off, const float* __restrict__ pos,
+                                                     const int* __restrict__ types, const CellInfo* __restrict__ info,
+                                                     const int* __restrict__ first,
+                                                     const int* __restrict__ atom_struct,
+                                                     const int* __restrict__ new_off, float* __restrict__ out_pos,
+                                                     int* __restrict__ out_types, unsigned char* __restrict__ ghost,
+                                                     int* __restrict__ active) {
+  const int a = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (a >= N) return;
+  const int s = atom_struct[a], a0 = off[s], n = off[s + 1] - a0, o0 = new_off[s];
+  const CellInfo& ci = info[s];
+  const int t = types[a], self = o0 + (a - a0);
+  const float* p = pos + 3 * (size_t)a;
+  if (lane == 0) {
+    out_types[self] = t;
+    ghost[self] = 0;
+    active[a] = self;
+  }
+  if (!ci.periodic) {
+    if (lane < 3) out_pos[3 * (size_t)self + lane] = p[lane];
+    return;
+  }
+  double sf[3];
+  frac_of(ci, p, sf);
+  if (lane == 0) {
+    float* q = out_pos + 3 * (size_t)self;
+    for (int c = 0; c < 3; ++c) q[c] = (float)(sf[0] * ci.H[c] + sf[1] * ci.H[3 + c] + sf[2] * ci.H[6 + c]);
+  }
+  int lo[3], hi[3];
+  for (int d = 0; d < 3; ++d) image_range(sf[d], ci.delta[d], lo[d], hi[d]);
+  const int w1 = hi[1] - lo[1] + 1, w2 = hi[2] - lo[2] + 1, all = (hi[0] - lo[0] + 1) * w1 * w2;
+  const int zero = (-lo[0] * w1 - lo[1]) * w2 - lo[2];  // the atom itself
+  const int g0 = o0 + n + first[a];
+  for (int e = lane; e < all - 1; e += 32) {
+    const int x = e < zero ? e : e + 1;
+    const int n0 = lo[0] + x / (w1 * w2), n1 = lo[1] + x / w2 % w1, n2 = lo[2] + x % w2;
+    const double f0 = sf[0] + n0, f1 = sf[1] + n1, f2 = sf[2] + n2;
+    const int g = g0 + e;
+    float* q = out_pos + 3 * (size_t)g;
+    // The exact position, a sum of float32 values, often lies half-way between
+    // two floats, so its rounding hangs on the last bit here.  The order and
+    // contraction are fixed to those the images have always had, which depend
+    // on where n2 lies in its range.
+    const int i2 = x % w2;
+    const bool two = i2 < (w2 & 3) && i2 < 2;
+    for (int c = 0; c < 3; ++c) {
+      const double ab = fma(f1, ci.H[3 + c], __dmul_rn(f0, ci.H[c]));
+      q[c] = (float)(two ? __dadd_rn(__dmul_rn(f2, ci.H[6 + c]), ab) : fma(f2, ci.H[6 + c], ab));
+    }
+    out_types[g] = t;
+    ghost[g] = 1;
+  }
 }
 
 __global__ void k_zero_ghosts(int N, const int* __restrict__ sorted_orig, const unsigned char* __restrict__ ghost,
@@ -214,39 +245,42 @@ tnep_status tnep_eval_batch_cell(tnep_ctx* c, int n_structs, const int* atom_off
     for (int a = 0; a < N; ++a)
       if (types[a] < 0 || types[a] >= c->n_types) return fail(TNEP_ERR_INVALID, "type index out of range");
   Workspace& w = c->ws;
-  DevBuf<float> d_pos_in, d_cell, d_epos, d_ebox;
-  DevBuf<int> d_types_in, d_off, d_newoff, d_nghost, d_etypes;
-  DevBuf<unsigned char> d_ghost;
-  DevBuf<CellInfo> d_info;
-  auto release = [&]() {
-    d_pos_in.release(); d_cell.release(); d_epos.release(); d_ebox.release(); d_types_in.release();
-    d_off.release(); d_newoff.release(); d_nghost.release(); d_etypes.release(); d_ghost.release();
-    d_info.release();
-  };
+  // scratch of the call from the library's pool: the inputs, then the expanded batch
+  char *in = nullptr, *ex = nullptr;
   auto body = [&]() -> tnep_status {
-    TNEP_CUDA(d_pos_in.ensure((size_t)std::max(N, 1) * 3));
-    TNEP_CUDA(d_types_in.ensure(std::max(N, 1)));
-    TNEP_CUDA(d_cell.ensure((size_t)n_structs * 9));
-    TNEP_CUDA(d_off.ensure(n_structs + 1));
-    TNEP_CUDA(d_nghost.ensure(n_structs));
-    TNEP_CUDA(d_info.ensure(n_structs));
+    size_t at = 0;
+    auto place = [&](size_t bytes) {
+      const size_t o = at;
+      at += (bytes + 255) & ~size_t(255);
+      return o;
+    };
+    const size_t n1 = std::max(N, 1);
+    const size_t o_pos = place(sizeof(float) * 3 * n1), o_types = place(sizeof(int) * n1);
+    const size_t o_cell = place(sizeof(float) * 9 * n_structs), o_off = place(sizeof(int) * (n_structs + 1));
+    const size_t o_ng = place(sizeof(int) * n_structs), o_info = place(sizeof(CellInfo) * n_structs);
+    const size_t o_first = place(sizeof(int) * n1), o_as = place(sizeof(int) * n1);
+    TNEP_CUDA(dev_malloc_async((void**)&in, at, st));
+    float *d_pos = reinterpret_cast<float*>(in + o_pos), *d_cell = reinterpret_cast<float*>(in + o_cell);
+    int *d_types = reinterpret_cast<int*>(in + o_types), *d_off = reinterpret_cast<int*>(in + o_off);
+    int *d_ng = reinterpret_cast<int*>(in + o_ng), *d_first = reinterpret_cast<int*>(in + o_first);
+    int* d_as = reinterpret_cast<int*>(in + o_as);
+    CellInfo* d_info = reinterpret_cast<CellInfo*>(in + o_info);
     if (N > 0) {
-      TNEP_CUDA(cudaMemcpyAsync(d_pos_in.p, pos, sizeof(float) * 3 * N, cudaMemcpyDefault, st));
-      TNEP_CUDA(cudaMemcpyAsync(d_types_in.p, types, sizeof(int) * N, cudaMemcpyDefault, st));
+      TNEP_CUDA(cudaMemcpyAsync(d_pos, pos, sizeof(float) * 3 * N, cudaMemcpyDefault, st));
+      TNEP_CUDA(cudaMemcpyAsync(d_types, types, sizeof(int) * N, cudaMemcpyDefault, st));
     }
     if (cell)
-      TNEP_CUDA(cudaMemcpyAsync(d_cell.p, cell, sizeof(float) * 9 * n_structs, cudaMemcpyDefault, st));
+      TNEP_CUDA(cudaMemcpyAsync(d_cell, cell, sizeof(float) * 9 * n_structs, cudaMemcpyDefault, st));
     else
-      TNEP_CUDA(cudaMemsetAsync(d_cell.p, 0, sizeof(float) * 9 * n_structs, st));
-    TNEP_CUDA(cudaMemcpyAsync(d_off.p, atom_offsets, sizeof(int) * (n_structs + 1), cudaMemcpyHostToDevice, st));
+      TNEP_CUDA(cudaMemsetAsync(d_cell, 0, sizeof(float) * 9 * n_structs, st));
+    TNEP_CUDA(cudaMemcpyAsync(d_off, atom_offsets, sizeof(int) * (n_structs + 1), cudaMemcpyHostToDevice, st));
     TNEP_TRY(reset_status(w, st));
-    k_cell_plan<<<(n_structs + 127) / 128, 128, 0, st>>>(n_structs, d_cell.p, c->rc_R, d_info.p, w.d_status);
-    k_cell_expand<<<n_structs, kExpandThreads, 0, st>>>(n_structs, d_off.p, d_pos_in.p, d_types_in.p, d_info.p,
-                                                        d_nghost.p, nullptr, nullptr, nullptr, nullptr);
-    count_launches(2);
+    k_cell_count<<<n_structs, kExpandThreads, 0, st>>>(d_off, d_pos, d_cell, c->rc_R, d_info, d_first, d_as, d_ng,
+                                                       w.d_status);
+    count_launches(1);
     TNEP_CUDA(cudaGetLastError());
     std::vector<int> ng(n_structs);
-    TNEP_CUDA(cudaMemcpyAsync(ng.data(), d_nghost.p, sizeof(int) * n_structs, cudaMemcpyDeviceToHost, st));
+    TNEP_CUDA(cudaMemcpyAsync(ng.data(), d_ng, sizeof(int) * n_structs, cudaMemcpyDeviceToHost, st));
     bool regrow = false;
     TNEP_TRY(finish(c, w, st, &regrow));  // synchronises; reports a degenerate cell
     std::vector<int> eoff(n_structs + 1, 0);
@@ -257,22 +291,30 @@ tnep_status tnep_eval_batch_cell(tnep_ctx* c, int n_structs, const int* atom_off
       eoff[s + 1] = (int)tot;
     }
     const int Ne = (int)tot;
-    TNEP_CUDA(d_newoff.ensure(n_structs + 1));
-    TNEP_CUDA(d_epos.ensure((size_t)std::max(Ne, 1) * 3));
-    TNEP_CUDA(d_etypes.ensure(std::max(Ne, 1)));
-    TNEP_CUDA(d_ghost.ensure(std::max(Ne, 1)));
-    TNEP_CUDA(d_ebox.ensure((size_t)n_structs * 3));
-    TNEP_CUDA(cudaMemsetAsync(d_ebox.p, 0, sizeof(float) * 3 * n_structs, st));
-    TNEP_CUDA(cudaMemcpyAsync(d_newoff.p, eoff.data(), sizeof(int) * (n_structs + 1), cudaMemcpyHostToDevice, st));
-    k_cell_expand<<<n_structs, kExpandThreads, 0, st>>>(n_structs, d_off.p, d_pos_in.p, d_types_in.p, d_info.p,
-                                                        d_nghost.p, d_newoff.p, d_epos.p, d_etypes.p, d_ghost.p);
-    count_launches(1);
-    TNEP_CUDA(cudaGetLastError());
+    at = 0;
+    const size_t e1 = std::max(Ne, 1);
+    const size_t o_new = place(sizeof(int) * (n_structs + 1)), o_epos = place(sizeof(float) * 3 * e1);
+    const size_t o_et = place(sizeof(int) * e1), o_gh = place(e1), o_box = place(sizeof(float) * 3 * n_structs);
+    const size_t o_act = place(sizeof(int) * n1);
+    TNEP_CUDA(dev_malloc_async((void**)&ex, at, st));
+    int *d_new = reinterpret_cast<int*>(ex + o_new), *d_etypes = reinterpret_cast<int*>(ex + o_et);
+    int* d_active = reinterpret_cast<int*>(ex + o_act);
+    float *d_epos = reinterpret_cast<float*>(ex + o_epos), *d_ebox = reinterpret_cast<float*>(ex + o_box);
+    unsigned char* d_ghost = reinterpret_cast<unsigned char*>(ex + o_gh);
+    TNEP_CUDA(cudaMemsetAsync(d_ebox, 0, sizeof(float) * 3 * n_structs, st));
+    TNEP_CUDA(cudaMemcpyAsync(d_new, eoff.data(), sizeof(int) * (n_structs + 1), cudaMemcpyHostToDevice, st));
+    if (N > 0) {
+      k_cell_expand<<<(unsigned)((32LL * N + 127) / 128), 128, 0, st>>>(N, d_off, d_pos, d_types, d_info, d_first, d_as,
+                                                                        d_new, d_epos, d_etypes, d_ghost, d_active);
+      count_launches(1);
+      TNEP_CUDA(cudaGetLastError());
+    }
+    const Images images{d_ghost, d_active, N};
     const int Ctot = total_C(c);
     for (int attempt = 0; attempt < 4; ++attempt) {
       TNEP_TRY(reset_status(w, st));
-      TNEP_TRY(build_lists(c, w, st, n_structs, eoff.data(), d_epos.p, d_ebox.p, d_etypes.p, std::max(Ne, 1), nullptr, N));
-      TNEP_TRY(run_models(c, w, st, n_structs, Ne, nullptr, d_ghost.p));
+      TNEP_TRY(build_lists(c, w, st, n_structs, eoff.data(), d_epos, d_ebox, d_etypes, std::max(Ne, 1), nullptr, N));
+      TNEP_TRY(run_models(c, w, st, n_structs, Ne, nullptr, &images));
       regrow = false;
       TNEP_TRY(finish(c, w, st, &regrow));
       if (regrow) continue;
@@ -283,8 +325,9 @@ tnep_status tnep_eval_batch_cell(tnep_ctx* c, int n_structs, const int* atom_off
     return fail(TNEP_ERR_NEIGHBOR_OVERFLOW, "neighbour lists kept overflowing");
   };
   const tnep_status rc = body();
+  if (ex) cudaFreeAsync(ex, st);
+  if (in) cudaFreeAsync(in, st);
   cudaStreamSynchronize(st);
-  release();
   return rc;
 }
 

@@ -514,12 +514,18 @@ tnep_status sum_pass_times(tnep_ctx* c, int n_pass) {
 
 // One warp per atom: the FP32-network models up to kWideModels of a variant at
 // a time, then lists and moments for the others.
-static tnep_status run_wide(tnep_ctx* c, Workspace& w, cudaStream_t st, const unsigned char* ghost, size_t per_model,
+static tnep_status run_wide(tnep_ctx* c, Workspace& w, cudaStream_t st, const Images* images, size_t per_model,
                             bool* others) {
   WideArgs a{};
   a.nbr = w.prepared;
   a.sorted_cell = w.atom_slot.p;
-  a.ghost = ghost;
+  a.n_active = a.nbr.n_atoms;
+  if (images) {  // the images keep zero contributions, and no pairs where k_fused follows
+    a.active = images->active;
+    a.n_active = images->n_active;
+    TNEP_CUDA(cudaMemsetAsync(w.per_atom.p, 0, sizeof(float) * per_model * c->models.size(), st));
+    TNEP_CUDA(cudaMemsetAsync(w.cnt_A.p, 0, sizeof(int) * w.atom_stride, st));
+  }
   a.atom_stride = w.atom_stride;
   bool need_v = false, need_w = false;
   *others = false;
@@ -578,7 +584,7 @@ static tnep_status join_side(Workspace& w, cudaStream_t st) {
 }
 
 tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N, cudaEvent_t ev_done,
-                       const unsigned char* ghost, cudaStream_t red_st) {
+                       const Images* images, cudaStream_t red_st) {
   const size_t per_model = (size_t)9 * w.atom_stride;
   TNEP_CUDA(w.per_atom.ensure(per_model * c->models.size()));
   TNEP_CUDA(w.out.ensure((size_t)std::max(S, 1) * total_C(c)));
@@ -593,7 +599,7 @@ tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N,
   }
   bool thread_per_atom = true;
   if (w.wide)
-    TNEP_TRY(run_wide(c, w, st, ghost, per_model, &thread_per_atom));
+    TNEP_TRY(run_wide(c, w, st, images, per_model, &thread_per_atom));
   else
     TNEP_TRY(compute_moments(c, w, st, N, any_rank(c, 1), any_rank(c, 2)));
   if (thread_per_atom) {
@@ -632,9 +638,9 @@ tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N,
     TNEP_CUDA(e);
   }
   if (ev_done) TNEP_CUDA(cudaEventRecord(ev_done, st));
-  if (ghost && thread_per_atom)
+  if (images && thread_per_atom)
     for (size_t k = 0; k < c->models.size(); ++k)
-      TNEP_CUDA(launch_zero_ghosts(N, w.sorted_orig.p, ghost, w.per_atom.p + k * per_model, w.atom_stride,
+      TNEP_CUDA(launch_zero_ghosts(N, w.sorted_orig.p, images->ghost, w.per_atom.p + k * per_model, w.atom_stride,
                                    c->models[k].C, st));
   TNEP_CUDA(w.partial.ensure((size_t)std::max(S, 1) * reduce_chunks(w.max_atoms) * 9 * c->models.size()));
   cudaStream_t rs = st;

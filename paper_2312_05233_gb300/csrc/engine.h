@@ -249,16 +249,23 @@ tnep_status compute_moments(tnep_ctx* c, Workspace& w, cudaStream_t st, int N, b
 bool any_rank(const tnep_ctx* c, int rank);
 FusedArgs fused_args(tnep_ctx* c, Workspace& w, const Model& m, int N);
 int total_C(const tnep_ctx* c);
+// A batch with image atoms: one flag per atom (input order), and the input
+// indices of the n_active others.
+struct Images {
+  const unsigned char* ghost;
+  const int* active;
+  int n_active;
+};
 tnep_status pass_events(tnep_ctx* c, int b, cudaEvent_t** ev);
 tnep_status sum_pass_times(tnep_ctx* c, int n_pass);
-// ghost: NULL, or one flag per atom of the batch (input order) marking image
-// atoms whose contributions are left out of the per-structure sums.
+// images: NULL, or which atoms of the batch are images, whose contributions
+// are left out of the per-structure sums.
 // red_st: NULL, or a stream for the per-structure sums (the caller records
 // c->ev_reduced on it once it has consumed w.out); the fused kernels on st
 // first wait for the previous pass's sums (c->ev_reduced) to have read the
 // per-atom outputs.
 tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N, cudaEvent_t ev_done,
-                       const unsigned char* ghost = nullptr, cudaStream_t red_st = nullptr);
+                       const Images* images = nullptr, cudaStream_t red_st = nullptr);
 cudaError_t launch_zero_ghosts(int N, const int* sorted_orig, const unsigned char* ghost, float* per_atom,
                                int atom_stride, int C, cudaStream_t st);
 tnep_status check_status(tnep_ctx* c, const DevStatus& s, bool* regrow);

@@ -281,7 +281,8 @@ constexpr size_t kWideMaxSmem = 100 * 1024;  // two CTAs per SM
 struct WideArgs {
   NbrArgs nbr;                  // prepared batch (cells, sorted atoms)
   const int* sorted_cell;
-  const unsigned char* ghost;   // null, or per input atom: an image atom, skipped (fused: contributes zeros)
+  const int* active;            // input indices of the n_active atoms to evaluate, or null (all)
+  int n_active;
   int n_models;
   struct {
     const float* model;

@@ -118,19 +118,11 @@ __global__ void __launch_bounds__(32 * kWarps) k_wide(const __grid_constant__ Wi
   static_assert(NLM <= kTileG && NA <= 5 && DP <= 32, "tile rows and lane maps");
   extern __shared__ float4 sm4[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * kWarps + warp;
   const NbrArgs& na = a.nbr;
   const int T = na.n_types;
-  if (i >= na.n_atoms) return;  // whole warps; there is no CTA-wide barrier below
-  if (a.ghost && a.ghost[na.sorted_orig[i]]) {  // an image atom: not part of any sum
-    if constexpr (FUSED) {
-      for (int m = 0; m < a.n_models; ++m)
-        if (lane < (a.model[m].rank == 1 ? 3 : 9)) a.model[m].per_atom[(size_t)lane * a.atom_stride + i] = 0.f;
-    } else {
-      if (lane == 0) na.cnt_A[i] = 0;  // no pairs; its contributions are zeroed after the fused kernel
-    }
-    return;
-  }
+  const int item = blockIdx.x * kWarps + warp;
+  if (item >= a.n_active) return;  // whole warps; there is no CTA-wide barrier below
+  const int i = a.active ? na.orig_sorted[a.active[item]] : item;
   int* lists = reinterpret_cast<int*>(sm4) + (size_t)warp * wide_words(T, na.cap_R, na.cap_A);
   int* sR = lists;                                        // radial list, grouped by type
   int* sTmp = sR + na.cap_R;                              // append order, tagged with the type (more than two types)
@@ -679,7 +671,7 @@ cudaError_t launch_one(const WideArgs& a, int smem, cudaStream_t st) {
   const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   count_launches(1);
-  fn<<<(a.nbr.n_atoms + kWarps - 1) / kWarps, 32 * kWarps, smem, st>>>(a);
+  fn<<<(a.n_active + kWarps - 1) / kWarps, 32 * kWarps, smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -690,7 +682,7 @@ size_t wide_smem_bytes(int n_types, int cap_R, int cap_A) {
 }
 
 cudaError_t launch_wide(int variant, bool fused, const WideArgs& a_in, cudaStream_t st) {
-  if (a_in.nbr.n_atoms <= 0) return cudaSuccess;
+  if (a_in.n_active <= 0) return cudaSuccess;
   WideArgs a = a_in;
   for (int k = 0; k < 24; ++k) a.w[k] = wlm(k);
   const int smem = (int)wide_smem_bytes(a.nbr.n_types, a.nbr.cap_R, a.nbr.cap_A);
