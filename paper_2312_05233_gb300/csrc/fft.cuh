@@ -1,7 +1,7 @@
 // Batched complex FFT in float64 for the correlation and cosine-transform
 // tails (spectrum.cu, raman.cu): N = 2^m (m >= 8), Stockham passes of radix
-// 16 (with one pass of radix 2, 4 or 8 between the first and the last where m
-// is not a multiple of 4), one butterfly per thread in registers.
+// 16 or 8 (with one smaller one between the first and the last where m is not a
+// multiple of 4 or 3), one butterfly per thread in registers.
 //
 // What bounds it: the FP64 pipe (two lanes per clock and SM, 64 times fewer
 // than FP32), about 3.5 instructions per point and radix-2 stage whatever the
@@ -31,6 +31,10 @@ namespace fft {
 
 constexpr int kMinLog = 8;
 constexpr int kThreads = 128;
+// Passes of fewer threads than this run in CTAs of one warp, so that a single
+// transform's butterflies spread over the SMs (2048 of them in 16 CTAs: 12 us a
+// pass, FP64 issue of 16 SMs).
+constexpr long long kSpreadBelow = 152 * 256;
 
 // Sign flip and swap without the FP64 pipe.
 __device__ __forceinline__ double flip(double v, unsigned sign) {
@@ -72,8 +76,9 @@ __device__ __forceinline__ void dft4(double2& a, double2& b, double2& c, double2
   d = sub(t1, t3);
 }
 
-// In place, natural order in and out.
-template <int R, bool INV>
+// In place, natural order in and out.  HALF: the upper half of v is zero
+// (radix 16 only).
+template <int R, bool INV, bool HALF = false>
 __device__ __forceinline__ void dft(double2* v) {
   constexpr double h = 0.70710678118654752440;
   if constexpr (R == 2) {
@@ -105,8 +110,16 @@ __device__ __forceinline__ void dft(double2* v) {
 #pragma unroll
     for (int n2 = 0; n2 < 4; ++n2) {
 #pragma unroll
-      for (int n1 = 0; n1 < 4; ++n1) y[n2][n1] = v[4 * n1 + n2];
-      dft4<INV>(y[n2][0], y[n2][1], y[n2][2], y[n2][3]);
+      for (int n1 = 0; n1 < (HALF ? 2 : 4); ++n1) y[n2][n1] = v[4 * n1 + n2];
+      if constexpr (HALF) {
+        const double2 a = y[n2][0], b = y[n2][1], r = rot<INV>(b);
+        y[n2][0] = add(a, b);
+        y[n2][1] = add(a, r);
+        y[n2][2] = sub(a, b);
+        y[n2][3] = sub(a, r);
+      } else {
+        dft4<INV>(y[n2][0], y[n2][1], y[n2][2], y[n2][3]);
+      }
     }
     // y[n2][k1] *= exp(-+2 pi i n2 k1 / 16)
     auto w = [](double2 a, double c, double s) {  // a (c -+ i s)
@@ -136,7 +149,9 @@ __device__ __forceinline__ void dft(double2* v) {
 }
 
 // Plain element access of `batch` transforms of length N.
+// A load with kHalfZero gives zeros for the upper half (it is not called there).
 struct LoadPlain {
+  static constexpr bool kHalfZero = false;
   const double2* p;
   int logN;
   __device__ __forceinline__ double2 operator()(int f, unsigned i) const { return p[((size_t)f << logN) + i]; }
@@ -151,19 +166,24 @@ template <int LOGR, bool INV, class Load, class Store>
 __global__ void __launch_bounds__(kThreads) k_pass(const Load ld, const Store st, const double2* __restrict__ tab,
                                                    int logN, int logp, int batch) {
   constexpr int R = 1 << LOGR;
-  const long long g = (long long)blockIdx.x * kThreads + threadIdx.x;
+  const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int f = (int)(g >> (logN - LOGR));
   if (f >= batch) return;
   const unsigned j = (unsigned)(g & ((1ll << (logN - LOGR)) - 1));
+  constexpr bool HALF = Load::kHalfZero && R == 16;
   double2 v[R];
 #pragma unroll
-  for (int r = 0; r < R; ++r) v[r] = ld(f, j + ((unsigned)r << (logN - LOGR)));
+  for (int r = 0; r < (Load::kHalfZero ? R / 2 : R); ++r) v[r] = ld(f, j + ((unsigned)r << (logN - LOGR)));
+  if constexpr (Load::kHalfZero && !HALF) {
+#pragma unroll
+    for (int r = R / 2; r < R; ++r) v[r] = make_double2(0.0, 0.0);
+  }
   const unsigned k = j & ((1u << logp) - 1);
   if (logp > 0) {
 #pragma unroll
     for (int r = 1; r < R; ++r) v[r] = mul(v[r], twiddle<INV>(tab, (k * r) << (logN - logp - LOGR), logN));
   }
-  dft<R, INV>(v);
+  dft<R, INV, HALF>(v);
   const unsigned o = ((j >> logp) << (logp + LOGR)) + k;
 #pragma unroll
   for (int r = 0; r < R; ++r) st(f, o + ((unsigned)r << logp), v[r]);
@@ -173,7 +193,8 @@ template <int LOGR, bool INV, class Load, class Store>
 cudaError_t pass(const Load& ld, const Store& st, const double2* tab, int logN, int logp, int batch, cudaStream_t s) {
   const long long n = (long long)batch << (logN - LOGR);
   count_launches(1);
-  k_pass<LOGR, INV><<<(unsigned)((n + kThreads - 1) / kThreads), kThreads, 0, s>>>(ld, st, tab, logN, logp, batch);
+  const int threads = n < kSpreadBelow ? 32 : kThreads;
+  k_pass<LOGR, INV><<<(unsigned)((n + threads - 1) / threads), threads, 0, s>>>(ld, st, tab, logN, logp, batch);
   return cudaGetLastError();
 }
 
@@ -181,13 +202,13 @@ cudaError_t pass(const Load& ld, const Store& st, const double2* tab, int logN, 
 // exp(+i ...), no 1/N), loading element i of array f as ld(f, i) and storing
 // through st(f, i, value).  a and b: scratch of batch << logN elements each;
 // the first pass writes a, so ld may read b.
-template <bool INV, class Load, class Store>
-cudaError_t transform(const Load& ld, const Store& st, double2* a, double2* b, const double2* tab, int logN,
-                      int batch, cudaStream_t s) {
-  cudaError_t e = pass<4, INV>(ld, StorePlain{a, logN}, tab, logN, 0, batch, s);
-  int logp = 4;
-  for (int left = logN - 8; left > 0 && e == cudaSuccess;) {
-    const int r = (left & 3) ? (left & 3) : 4;
+template <int LOGB, bool INV, class Load, class Store>
+cudaError_t transform_radix(const Load& ld, const Store& st, double2* a, double2* b, const double2* tab, int logN,
+                            int batch, cudaStream_t s) {
+  cudaError_t e = pass<LOGB, INV>(ld, StorePlain{a, logN}, tab, logN, 0, batch, s);
+  int logp = LOGB;
+  for (int left = logN - 2 * LOGB; left > 0 && e == cudaSuccess;) {
+    const int r = left % LOGB ? left % LOGB : LOGB;
     const LoadPlain l{a, logN};
     const StorePlain o{b, logN};
     if (r == 1) e = pass<1, INV>(l, o, tab, logN, logp, batch, s);
@@ -199,11 +220,27 @@ cudaError_t transform(const Load& ld, const Store& st, double2* a, double2* b, c
     left -= r;
   }
   if (e != cudaSuccess) return e;
-  return pass<4, INV>(LoadPlain{a, logN}, st, tab, logN, logp, batch, s);
+  return pass<LOGB, INV>(LoadPlain{a, logN}, st, tab, logN, logp, batch, s);
+}
+
+// Radix 16 where its butterflies fill the chip.  An SM's four quarters issue
+// half an FP64 lane a clock each, so a lone warp's radix-16 butterfly takes
+// 288 x 64 cycles (11 us a pass of four stages, whatever the size, below one
+// warp per quarter); radix 8 takes 80 x 64 for three.
+inline int base_radix(int logN, int batch) { return ((long long)batch << logN) < 300000 ? 3 : 4; }
+
+template <bool INV, class Load, class Store>
+cudaError_t transform(const Load& ld, const Store& st, double2* a, double2* b, const double2* tab, int logN,
+                      int batch, cudaStream_t s) {
+  if (base_radix(logN, batch) == 3) return transform_radix<3, INV>(ld, st, a, b, tab, logN, batch, s);
+  return transform_radix<4, INV>(ld, st, a, b, tab, logN, batch, s);
 }
 
 // Index of the buffer (0 = a, 1 = b) the last pass of a transform reads.
-inline int last_source(int logN) { return ((logN - 8 + 3) / 4) & 1; }
+inline int last_source(int logN, int batch) {
+  const int base = base_radix(logN, batch);
+  return ((logN - 2 * base + base - 1) / base) & 1;
+}
 
 inline int log2_at_least(long long n) {
   int m = kMinLog;

@@ -24,6 +24,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <utility>
 
 #include "engine.h"
@@ -149,12 +150,13 @@ __global__ void k_rlags(const double* __restrict__ C, int T, int M, double* __re
 
 // Segment b of pack k (transform k nb + b): its L = N/2 samples, then zeros.
 struct LoadSegment {
+  static constexpr bool kHalfZero = true;
   const double2* z;
   int T, nb, logN;
   __device__ __forceinline__ double2 operator()(int f, unsigned i) const {
     const int k = f / nb, b = f - k * nb;
     const long long t = ((long long)b << (logN - 1)) + i;
-    if (i >= (1u << (logN - 1)) || t >= T) return make_double2(0.0, 0.0);
+    if (t >= T) return make_double2(0.0, 0.0);
     return __ldg(z + (size_t)k * T + t);
   }
 };
@@ -241,19 +243,24 @@ __global__ void __launch_bounds__(128) k_rcross(const double2* __restrict__ z, i
   else cross_rows<2>(z, logN, nb, b0, b1, f, dst);
 }
 
-// Pairs 2f and 2f + 1 (spectra of real sequences) as one complex spectrum,
-// the chunks summed in order.
+// The chunks of k_rcross summed in order into the first.
+__global__ void __launch_bounds__(256) k_rsum_chunks(double2* __restrict__ part, long long n, int chunks) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double2 v = part[i];
+  for (int c = 1; c < chunks; ++c) v = fft::add(v, part[c * n + i]);
+  part[i] = v;
+}
+
+// Pairs 2f and 2f + 1 (spectra of real sequences) as one complex spectrum.
 struct LoadCross {
+  static constexpr bool kHalfZero = false;
   const double2* part;
-  int chunks, logN;
+  int logN;
   __device__ __forceinline__ double2 operator()(int f, unsigned i) const {
     const unsigned N = 1u << logN, half = N >> 1, g = i <= half ? i : N - i;
-    double2 u = make_double2(0.0, 0.0), v = u;
-    for (int c = 0; c < chunks; ++c) {
-      const double2* s = part + ((size_t)c * 45 + 2 * f) * (half + 1) + g;
-      u = fft::add(u, s[0]);
-      if (2 * f + 1 < 45) v = fft::add(v, s[half + 1]);
-    }
+    const double2* s = part + (size_t)(2 * f) * (half + 1) + g;
+    const double2 u = s[0], v = 2 * f + 1 < 45 ? s[half + 1] : make_double2(0.0, 0.0);
     return i <= half ? make_double2(u.x - v.y, u.y + v.x) : make_double2(u.x + v.y, v.x - u.y);
   }
 };
@@ -297,27 +304,70 @@ __global__ void k_rpolar(const double* __restrict__ L, int M, int O, const doubl
 // Crystal turned by theta about `axis` (the laser direction): incoming
 // polarization R^T X, observed R^T X (parallel) or R^T Y (crossed), with X, Y
 // the two crystal axes orthogonal to `axis` in cyclic order.
-__global__ void k_rporto(const double* __restrict__ L, int M, int O, const double* __restrict__ theta, int axis,
-                         double* __restrict__ par, double* __restrict__ crs) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)O * (M + 1)) return;
-  const int o = (int)(i / (M + 1)), k = (int)(i % (M + 1));
+//
+// With e = (c, -s) and y = (s, c) on the axes (a, b), the weights are
+//   parallel (aa, ab, ba, bb) = (c^2, -cs, -cs, s^2), crossed = (cs, -s^2, c^2, -cs),
+// so each spectrum is a quadratic form in (u, v, z) = (c^2, cs, s^2): six
+// coefficients per frequency, then six multiply-adds per angle instead of 90 (the
+// contraction over all nine components was FP64-bound: 147 us for 181 angles and
+// 2001 frequencies).  Entries of L outside the plane have weight zero; they are
+// still multiplied by it, so a NaN or infinity there shows as before.
+// grid (frequency tiles, angle chunks)
+constexpr int kPortoAngles = 16;
+__global__ void __launch_bounds__(128) k_rporto(const double* __restrict__ L, int M, int O,
+                                                const double* __restrict__ theta, int axis, double* __restrict__ par,
+                                                double* __restrict__ crs) {
+  __shared__ double mono[kPortoAngles][6];  // u^2, uv, uz, v^2, vz, z^2
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
   const int a = (axis + 1) % 3, b = (axis + 2) % 3;
-  double sn, cs;
-  sincos(theta[o], &sn, &cs);
-  double e[3] = {0.0, 0.0, 0.0}, y[3] = {0.0, 0.0, 0.0};
-  e[a] = cs; e[b] = -sn;
-  y[a] = sn; y[b] = cs;
-  double wp[9], wc[9];
+  const int id[4] = {a * 3 + a, a * 3 + b, b * 3 + a, b * 3 + b};
+  const double* Lk = L + (size_t)min(k, M) * 81;
+  double zero = 0.0, q[4][4];
+  for (int r = 0; r < 9; ++r) {
+    const bool row = r / 3 != axis && r % 3 != axis;
+    for (int c = 0; c < 9; ++c)
+      if (!row || c / 3 == axis || c % 3 == axis) zero = fma(Lk[r * 9 + c], 0.0, zero);
+  }
 #pragma unroll
-  for (int g = 0; g < 3; ++g)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      wp[g * 3 + d] = e[g] * e[d];
-      wc[g * 3 + d] = y[g] * e[d];
+    for (int j = 0; j < 4; ++j) q[i][j] = Lk[id[i] * 9 + id[j]];
+  const double p[6] = {q[0][0],
+                       -((q[0][1] + q[1][0]) + (q[0][2] + q[2][0])),
+                       q[0][3] + q[3][0],
+                       (q[1][1] + q[2][2]) + (q[1][2] + q[2][1]),
+                       -((q[1][3] + q[3][1]) + (q[2][3] + q[3][2])),
+                       q[3][3]};
+  const double x[6] = {q[2][2],
+                       (q[0][2] + q[2][0]) - (q[2][3] + q[3][2]),
+                       -(q[1][2] + q[2][1]),
+                       (q[0][0] + q[3][3]) - (q[0][3] + q[3][0]),
+                       (q[1][3] + q[3][1]) - (q[0][1] + q[1][0]),
+                       q[1][1]};
+  for (long long o0 = (long long)blockIdx.y * kPortoAngles; o0 < O; o0 += (long long)gridDim.y * kPortoAngles) {
+    const int no = (int)min((long long)kPortoAngles, O - o0);
+    __syncthreads();
+    if ((int)threadIdx.x < no) {
+      double sn, cs;
+      sincos(theta[o0 + threadIdx.x], &sn, &cs);
+      const double u = cs * cs, v = cs * sn, z = sn * sn;
+      double* m = mono[threadIdx.x];
+      m[0] = u * u; m[1] = u * v; m[2] = u * z; m[3] = v * v; m[4] = v * z; m[5] = z * z;
     }
-  par[i] = contract(L + (size_t)k * 81, wp);
-  crs[i] = contract(L + (size_t)k * 81, wc);
+    __syncthreads();
+    if (k > M) continue;
+    for (int o = 0; o < no; ++o) {
+      double vp = zero, vx = zero;
+#pragma unroll
+      for (int t = 0; t < 6; ++t) {
+        vp = fma(p[t], mono[o][t], vp);
+        vx = fma(x[t], mono[o][t], vx);
+      }
+      const size_t at = (size_t)(o0 + o) * (M + 1) + k;
+      par[at] = vp;
+      crs[at] = vx;
+    }
+  }
 }
 
 unsigned blocks_for(long long n, int threads) { return (unsigned)((n + threads - 1) / threads); }
@@ -394,13 +444,16 @@ tnep_status tnep_raman_tensor(const double* series, int T, double dt_fs, int max
       double2 *zx = reinterpret_cast<double2*>(d_x), *cross = reinterpret_cast<double2*>(d + o_cross);
       k_rprep<true><<<blocks_for(T, 256), 256, 0, st>>>(d_s, T, d_part, n_part, subtract_mean, d_x);
       e = launch_fft_table(logN, tw, st);
-      double2* fin = fft::last_source(logN) == 0 ? zb : za;
+      double2* fin = fft::last_source(logN, kPacks * nb) == 0 ? zb : za;
       if (e == cudaSuccess)
         e = fft::transform<false>(LoadSegment{zx, T, nb, logN}, fft::StorePlain{fin, logN}, za, zb, tw, logN,
                                   kPacks * nb, st);
       if (e == cudaSuccess) {
         k_rcross<<<dim3((half + 1 + 127) / 128, 3, chunks), 128, 0, st>>>(fin, logN, nb, per_chunk, cross);
-        e = fft::transform<true>(LoadCross{cross, chunks, logN},
+        const long long n = 45LL * (half + 1);
+        count_launches(1);
+        if (chunks > 1) k_rsum_chunks<<<blocks_for(n, 256), 256, 0, st>>>(cross, n, chunks);
+        e = fft::transform<true>(LoadCross{cross, logN},
                                  StoreLags{d_lags, T, M, 1.0 / (8.0 * (double)(1ll << logN))}, za, zb, tw, logN,
                                  23, st);
       }
@@ -457,7 +510,8 @@ tnep_status tnep_raman_porto_map(const double* L, int max_lag, int n_theta, cons
   cudaError_t e = cudaMemcpyAsync(d_l, L, sizeof(double) * nL, cudaMemcpyDefault, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_t, theta, sizeof(double) * n_theta, cudaMemcpyDefault, st);
   if (e == cudaSuccess) {
-    k_rporto<<<blocks_for((long long)nO, 256), 256, 0, st>>>(d_l, max_lag, n_theta, d_t, axis, d_p, d_c);
+    k_rporto<<<dim3(blocks_for(max_lag + 1LL, 128), std::min(blocks_for(n_theta, kPortoAngles), 65535u)), 128, 0, st>>>(
+        d_l, max_lag, n_theta, d_t, axis, d_p, d_c);
     count_launches(1);
     e = cudaGetLastError();
   }

@@ -151,24 +151,39 @@ __global__ void __launch_bounds__(256) k_prep(const double* __restrict__ series,
 // One warp per lag: short series are bound by FP64 issue (IR, T = 2000,
 // M = 1000: 4.5e6 multiply-adds), where the CTA-wide tree this replaces cost
 // as much again (21 us).
-__global__ void __launch_bounds__(256) k_acf(const double* __restrict__ x, int T, int M, int kind,
+__global__ void __launch_bounds__(64) k_acf(const double* __restrict__ x, int T, int M, int kind,
                                              double* __restrict__ acf) {
   const int tau = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (tau > M) return;
   const int n = T - tau;
   double acc = 0.0, acc2 = 0.0;
-  if (kind == TNEP_SPECTRUM_IR) {
-    const double* y = x + (size_t)tau * 3;
-    for (long long i = lane; i < 3LL * n; i += 64) {
-      acc = fma(x[i], y[i], acc);
-      if (i + 32 < 3LL * n) acc2 = fma(x[i + 32], y[i + 32], acc2);
+  if (kind != TNEP_SPECTRUM_RAMAN_ANISO) {
+    // products of the flat signal with itself tau samples on, four loads of each in flight
+    const int cx = kind == TNEP_SPECTRUM_IR ? 3 : 1;
+    const double* y = x + (size_t)tau * cx;
+    const long long m = (long long)n * cx;
+    // (one warp per quarter of an SM: the next group loads under this one's FP64 issue)
+    constexpr int U = 4;
+    double s4[U] = {0.0, 0.0, 0.0, 0.0}, xa[U], xb[U];
+    long long i = lane;
+    const long long full = m / (32 * U) * (32 * U);
+    if (full > 0) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) { xa[u] = x[i + 32 * u]; xb[u] = y[i + 32 * u]; }
     }
-  } else if (kind == TNEP_SPECTRUM_RAMAN_ISO) {
-    const double* y = x + tau;
-    for (int i = lane; i < n; i += 64) {
-      acc = fma(x[i], y[i], acc);
-      if (i + 32 < n) acc2 = fma(x[i + 32], y[i + 32], acc2);
+    for (; i < full; i += 32 * U) {
+      double na[U], nb[U];
+      const long long nx = i + 32 * U < full ? i + 32 * U : i;
+#pragma unroll
+      for (int u = 0; u < U; ++u) { na[u] = x[nx + 32 * u]; nb[u] = y[nx + 32 * u]; }
+#pragma unroll
+      for (int u = 0; u < U; ++u) s4[u] = fma(xa[u], xb[u], s4[u]);
+#pragma unroll
+      for (int u = 0; u < U; ++u) { xa[u] = na[u]; xb[u] = nb[u]; }
     }
+    for (; i < m; i += 32) acc = fma(x[i], y[i], acc);
+    acc += s4[0] + s4[1];
+    acc2 += s4[2] + s4[3];
   } else {
     for (int t = lane; t < n; t += 32) {
       const double* a = x + (size_t)t * 9;
@@ -208,22 +223,42 @@ __device__ __forceinline__ void store_cos(const CosineOut& o, int seq, int k, in
 }
 
 // One warp per (frequency, sequence); the table index k tau mod 2M advances by
-// 32 k mod 2M (the 64-bit remainder per term cost more than the FP64 sums).
-__global__ void __launch_bounds__(256) k_cosine(const double* __restrict__ lags, const double* __restrict__ tab,
-                                                int M, const CosineOut o) {
+// 32 k mod 2M (the 64-bit remainder per term cost more than the FP64 sums), four
+// terms in flight.
+__global__ void __launch_bounds__(64) k_cosine(const double* __restrict__ lags, const double* __restrict__ tab,
+                                               int M, const CosineOut o) {
   const int k = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (k > M) return;
   const double* c = lags + (size_t)blockIdx.y * (M + 1);
   const unsigned period = 2u * (unsigned)M;
-  const unsigned step = (unsigned)((32ull * (unsigned)k) % period);
-  unsigned idx = (unsigned)(((unsigned long long)k * (unsigned)(1 + lane)) % period);
-  double acc = 0.0;
-  for (int tau = 1 + lane; tau <= M; tau += 32) {
-    acc = fma(c[tau], __ldg(tab + idx), acc);
-    idx += step;
-    idx -= idx >= period ? period : 0u;
+  unsigned step, idx;
+  if (M < (1 << 26)) {
+    step = (32u * (unsigned)k) % period;
+    idx = ((unsigned)k * (unsigned)(1 + lane)) % period;
+  } else {
+    step = (unsigned)((32ull * (unsigned)k) % period);
+    idx = (unsigned)(((unsigned long long)k * (unsigned)(1 + lane)) % period);
   }
-  acc = warp_sum(acc);
+  auto next = [&](unsigned i) {  // both below the period, which fits 31 bits
+    i += step;
+    return i >= period ? i - period : i;
+  };
+  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+  int tau = 1 + lane;
+  for (; tau + 96 <= M; tau += 128) {
+    const unsigned i1 = next(idx), i2 = next(i1), i3 = next(i2);
+    const double t0 = __ldg(tab + idx), t1 = __ldg(tab + i1), t2 = __ldg(tab + i2), t3 = __ldg(tab + i3);
+    a0 = fma(c[tau], t0, a0);
+    a1 = fma(c[tau + 32], t1, a1);
+    a2 = fma(c[tau + 64], t2, a2);
+    a3 = fma(c[tau + 96], t3, a3);
+    idx = next(i3);
+  }
+  for (; tau <= M; tau += 32) {
+    a0 = fma(c[tau], __ldg(tab + idx), a0);
+    idx = next(idx);
+  }
+  const double acc = warp_sum((a0 + a1) + (a2 + a3));
   if (lane == 0) store_cos(o, blockIdx.y, k, M, o.dt * fma(2.0, acc, c[0]));
 }
 
@@ -245,6 +280,7 @@ __global__ void __launch_bounds__(256) k_chirp_tables(int M, double2* __restrict
 
 // Sequences 0..nseq-1: C(tau) w_tau (half of it at 0); sequence nseq: conj(w_|n|).
 struct LoadChirp {
+  static constexpr bool kHalfZero = false;
   const double* lags;
   const double2* w;
   int M, nseq, logP;
@@ -263,6 +299,7 @@ struct LoadChirp {
   }
 };
 struct LoadChirpProduct {
+  static constexpr bool kHalfZero = false;
   const double2* z;
   int nseq, logP;
   __device__ __forceinline__ double2 operator()(int f, unsigned i) const {
@@ -359,17 +396,19 @@ __global__ void __launch_bounds__(128) k_spec_power(const double2* __restrict__ 
 
 // Segment b of pack k (transform k nb + b): its L = N/2 samples, then zeros.
 struct LoadSegment {
+  static constexpr bool kHalfZero = true;
   const double2* z;
   int T, nb, logN;
   __device__ __forceinline__ double2 operator()(int f, unsigned i) const {
     const int k = f / nb, b = f - k * nb;
     const long long t = ((long long)b << (logN - 1)) + i;
-    if (i >= (1u << (logN - 1)) || t >= T) return make_double2(0.0, 0.0);
+    if (t >= T) return make_double2(0.0, 0.0);
     return __ldg(z + (size_t)k * T + t);
   }
 };
 // The spectrum of a real sequence, its chunks summed in order.
 struct LoadPower {
+  static constexpr bool kHalfZero = false;
   const double2* part;
   int chunks, logN;
   __device__ __forceinline__ double2 operator()(int, unsigned i) const {
@@ -413,7 +452,7 @@ cudaError_t spectrum_fft(const double* series, int T, int M, int subtract_mean, 
   if (e != cudaSuccess) return e;
   k_prep<KIND, true><<<(T + 255) / 256, 256, 0, st>>>(series, T, part, sum_blocks, subtract_mean,
                                                       reinterpret_cast<double*>(zx));
-  double2* fin = fft::last_source(p.logN) == 0 ? b : a;
+  double2* fin = fft::last_source(p.logN, p.packs * p.nb) == 0 ? b : a;
   e = fft::transform<false>(LoadSegment{zx, T, p.nb, p.logN}, fft::StorePlain{fin, p.logN}, a, b, tab,
                                         p.logN, p.packs * p.nb, st);
   if (e != cudaSuccess) return e;
@@ -474,7 +513,7 @@ cudaError_t launch_cosine(const double* lags, int M, int nseq, const CosineOut& 
       tab = t;
     }
     count_launches(1);
-    k_cosine<<<dim3((M + 1 + 7) / 8, nseq), 256, 0, st>>>(lags, tab, M, o);
+    k_cosine<<<dim3((M + 1 + 1) / 2, nseq), 64, 0, st>>>(lags, tab, M, o);
     return cudaGetLastError();
   }
   const int logP = chirp_log(M);
@@ -485,7 +524,7 @@ cudaError_t launch_cosine(const double* lags, int M, int nseq, const CosineOut& 
   double2* tw = c.take<double2>(fft::table_size(logP));
   count_launches(1);
   k_chirp_tables<<<(unsigned)((M + 1 + fft::table_size(logP) + 255) / 256), 256, 0, st>>>(M, w, logP, tw);
-  double2* fin = fft::last_source(logP) == 0 ? b : a;
+  double2* fin = fft::last_source(logP, nseq + 1) == 0 ? b : a;
   double2* other = fin == a ? b : a;
   cudaError_t e = fft::transform<false>(LoadChirp{lags, w, M, nseq, logP}, fft::StorePlain{fin, logP}, a, b, tw, logP,
                                         nseq + 1, st);
@@ -544,7 +583,7 @@ cudaError_t launch_spectrum(const double* series, int T, int C, double dt_fs, in
       k_prep<TNEP_SPECTRUM_RAMAN_ISO, false><<<grid, 256, 0, st>>>(series, T, part, nsum, subtract_mean, x);
     else
       k_prep<TNEP_SPECTRUM_RAMAN_ANISO, false><<<grid, 256, 0, st>>>(series, T, part, nsum, subtract_mean, x);
-    k_acf<<<(unsigned)((32LL * (M + 1) + 255) / 256), 256, 0, st>>>(x, T, M, kind, acf);
+    k_acf<<<(unsigned)((32LL * (M + 1) + 63) / 64), 64, 0, st>>>(x, T, M, kind, acf);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) return e;

@@ -90,3 +90,29 @@ def test_raman_tensor_routes(tn, T, M):
             ref[:, p, q] = ref[:, q, p] = cosine(c, 2.0)
     np.testing.assert_allclose(L, ref, rtol=0, atol=slack * REL * np.abs(ref).max())
     np.testing.assert_allclose(f, np.arange(M + 1) / (2 * M * 2.0) / 2.99792458e-5, rtol=1e-14)
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("n_theta", [1, 16, 17])
+def test_porto_map_of_any_tensor(tn, axis, n_theta):
+    """The six-coefficient form against the full contraction w L w, for tensors
+    that are not symmetric in their pairs; relative to sum |w| |L| |w| the
+    rounding is a few eps."""
+    rng = np.random.default_rng(axis + 10 * n_theta)
+    M = 130
+    L = rng.standard_normal((M + 1, 9, 9))
+    th = rng.uniform(0, 2 * np.pi, n_theta)
+    th[0] = 0.0
+    par, crs = tn.tnep_raman_porto_map(L, th, axis=axis)
+    a, b = (axis + 1) % 3, (axis + 2) % 3
+    e, y = np.zeros((n_theta, 3)), np.zeros((n_theta, 3))
+    e[:, a], e[:, b], y[:, a], y[:, b] = np.cos(th), -np.sin(th), np.sin(th), np.cos(th)
+    for got, seen in ((par, e), (crs, y)):
+        w = (seen[:, :, None] * e[:, None, :]).reshape(n_theta, 9)
+        ref = np.einsum("op,kpq,oq->ok", w, L, w)
+        size = np.einsum("op,kpq,oq->ok", np.abs(w), np.abs(L), np.abs(w))
+        assert np.all(np.abs(got - ref) <= 1e-14 * size.max())
+    L[3, axis * 3, 0] = np.nan  # an entry of weight zero
+    L[5, a * 3 + a, a * 3 + a] = np.inf
+    par, _ = tn.tnep_raman_porto_map(L, th + 0.1, axis=axis)
+    assert np.isnan(par[:, 3]).all() and np.isfinite(par[:, 4]).all() and np.isposinf(par[:, 5]).all()
