@@ -53,6 +53,7 @@ tnep_status tnep_create(const tnep_model_desc* models, int n_models, int n_types
   if (!c) return fail(TNEP_ERR_OOM, "host allocation failed");
   g_contexts.fetch_add(1);
   c->device = device;
+  c->sms = prop.multiProcessorCount;
   c->n_types = n_types;
   c->rc_R = cutoffs[0];
   c->rc_A = cutoffs[1];

@@ -603,18 +603,27 @@ tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N,
   else
     TNEP_TRY(compute_moments(c, w, st, N, any_rank(c, 1), any_rank(c, 2)));
   if (thread_per_atom) {
-    // per-pair cache of the angular walks, reused by every model in turn
-    // (skipped when the lists' cap would make it larger than 16 GB: a pass of
-    // 2^21 atoms at cap_A = 64 takes 8.6 GB)
+    // Per-pair cache of the angular walks, reused by every model in turn: a
+    // column per thread of the tensor-core network's persistent CTAs (two per
+    // SM), or one per atom for the FP32 network (skipped when the lists' cap
+    // would make it larger than 16 GB: a pass of 2^21 atoms at cap_A = 64 takes
+    // 8.6 GB).
     constexpr size_t kPairCacheMaxBytes = size_t(16) << 30;
-    int quads = 0;
-    for (const auto& m : c->models) quads = std::max(quads, pair_cache_quads(m.d.n_max_A + 1));
-    const int pc_stride = round_up(std::max(N, 1), 128);
+    std::vector<size_t> run;
+    int quads = 0, pc_stride = 0;
+    auto stride_of = [&](const Model& m) {
+      const int all = round_up(std::max(N, 1), 128);
+      return m.d.mlp_precision != 0 ? std::min(all, 2 * c->sms * 128) : all;
+    };
+    for (size_t k = 0; k < c->models.size(); ++k) {
+      const Model& m = c->models[k];
+      if (w.wide && m.d.mlp_precision == 0) continue;
+      run.push_back(k);
+      quads = std::max(quads, pair_cache_quads(m.d.n_max_A + 1));
+      pc_stride = std::max(pc_stride, stride_of(m));
+    }
     const size_t pc_elems = (size_t)w.cap_A * quads * pc_stride;
     const bool use_pc = c->pair_cache && pc_elems * sizeof(float4) <= kPairCacheMaxBytes;
-    std::vector<size_t> run;
-    for (size_t k = 0; k < c->models.size(); ++k)
-      if (!(w.wide && c->models[k].d.mlp_precision == 0)) run.push_back(k);
     // Batches of a few waves: every other model on a side stream (with a pair
     // cache and a work counter of its own), so that one model's CTAs fill the
     // slots the other leaves.
@@ -630,7 +639,7 @@ tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N,
       f.per_atom = w.per_atom.p + k * per_model;
       f.per_atom_stride = 0;
       f.pcache = use_pc ? w.pcache.p + side * pc_elems : nullptr;
-      f.pc_stride = pc_stride;
+      f.pc_stride = stride_of(m);
       f.work_next += side;
       e = launch_fused(m.variant, m.d.rank, f, 1, c->block_atoms, m.d.mlp_precision, side ? w.side : st);
     }

@@ -180,6 +180,7 @@ struct tnep_ctx {
   template <class T> using PinBuf = tnep::PinBuf<T>;
   template <class T> using DevBuf = tnep::DevBuf<T>;
   int device = 0;
+  int sms = 0;
   cudaStream_t stream = nullptr, copy_stream = nullptr;
   cudaEvent_t ev_copied[2] = {nullptr, nullptr}, ev_consumed[2] = {nullptr, nullptr};
   // trajectories: the per-frame sums of a pass run on red_stream while the

@@ -170,6 +170,10 @@ __global__ void __launch_bounds__(BLK, 256 / BLK) k_fused(const __grid_constant_
   // the last atom and store nothing.
   if (!TC && !valid) return true;
   const int i = valid ? i_raw : a.n_atoms - 1;
+  // column of the pair cache: the thread's own among the resident CTAs where
+  // these are persistent (76 MB in use, so that pairs are read back from L2
+  // before they are evicted), else the atom's
+  const int pslot = TC ? blockIdx.x * BLK + tid : i_raw;
 
   const float4 pi = a.pos4[i];
   const int ti = __float_as_int(pi.w);
@@ -271,7 +275,7 @@ __global__ void __launch_bounds__(BLK, 256 / BLK) k_fused(const __grid_constant_
         for (int n = 0; n < NA; ++n) { v[4 + n] = g[n]; v[4 + NA + n] = dg[n]; }
 #pragma unroll
         for (int u = 4 + 2 * NA; u < 4 * NQ; ++u) v[u] = 0.f;
-        float4* dst = a.pcache + (size_t)kk * NQ * a.pc_stride + i_raw;
+        float4* dst = a.pcache + (size_t)kk * NQ * a.pc_stride + pslot;
 #pragma unroll
         for (int q = 0; q < NQ; ++q)
           __stcg(dst + (size_t)q * a.pc_stride, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
@@ -628,7 +632,7 @@ __global__ void __launch_bounds__(BLK, 256 / BLK) k_fused(const __grid_constant_
     constexpr int NQ = pair_cache_quads(NA);
     NbrWalk wB(a.nbr_A, a.pos4, i, a.cap_A, 0, (FACT || PC) ? 0 : nA, pi);
     // cached pairs: the next pair's quads are loaded one iteration ahead
-    const float4* pcs = PC ? a.pcache + i_raw : nullptr;  // own slots also past the end (tensor-core path)
+    const float4* pcs = PC ? a.pcache + pslot : nullptr;  // own slots also past the end (tensor-core path)
     float4 nxt[PC ? NQ : 1];
     if constexpr (PC) {
       if (nA > 0) {

@@ -200,9 +200,12 @@ struct FusedArgs {
   // Per-pair cache of the angular walk (single-individual launches, else
   // null): the forward walk stores, for pair k of atom i, r_ij and 1/|r_ij|,
   // g_n and g_n' in pair_cache_quads(NA) float4 at
-  // pcache[(k * quads + q) * pc_stride + i]; the backward walk reads them back
-  // instead of repeating the neighbour gather, the minimum image, the basis
-  // and the coefficient sums.
+  // pcache[(k * quads + q) * pc_stride + column]; the backward walk reads them
+  // back instead of repeating the neighbour gather, the minimum image, the basis
+  // and the coefficient sums.  The column is the atom, or with the tensor-core
+  // network's persistent CTAs (pc_stride = 128 times their number) the thread, so
+  // that 38,912 columns serve any number of atoms and stay in L2: 2,073,600
+  // atoms of water, two models, 7,219 -> 7,160 us (and 8.6 GB less).
   float4* pcache;
   int pc_stride;
 };
