@@ -38,6 +38,15 @@ struct ReduceArgs {
 __device__ __forceinline__ int lane_of(int c) {
   return ((c & 1) << 4) | ((c & 2) << 2) | (c & 4) | ((c & 8) >> 2);
 }
+// float32 -> float64 with integer instructions (exact; the conversion
+// instruction shares the FP64 pipe).  Subnormals, infinities and NaN take it.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), mag = u & 0x7fffffffu;
+  if (mag - 0x00800000u < 0x7f000000u)  // normal
+    return __hiloint2double((int)((u & 0x80000000u) | ((mag >> 3) + (896u << 20))), (int)(u << 29));
+  return mag == 0u ? __hiloint2double((int)u, 0) : (double)x;
+}
+
 template <int C>
 __device__ __forceinline__ double warp_tree(const double* v, int lane) {
   double t[C];
@@ -76,9 +85,14 @@ __device__ __forceinline__ void reduce_chunk(const ReduceArgs& a, const ReduceMo
     double acc[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) acc[c] = 0.0;
-    for (int g = a0 + threadIdx.x; g < a1; g += blockDim.x) {
+    int g = a0 + threadIdx.x;
+    if (g < a1) {  // the first addition would be to zero
 #pragma unroll
-      for (int c = 0; c < NC; ++c) acc[c] += (double)pa[(size_t)c * a.atom_stride + g];
+      for (int c = 0; c < NC; ++c) acc[c] = widen(pa[(size_t)c * a.atom_stride + g]);
+      for (g += blockDim.x; g < a1; g += blockDim.x) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) acc[c] += widen(pa[(size_t)c * a.atom_stride + g]);
+      }
     }
     v = warp_tree<NC>(acc, lane);
   }
