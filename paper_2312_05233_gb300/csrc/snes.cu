@@ -116,24 +116,40 @@ __global__ void __launch_bounds__(kSnesThreads) k_snes_fitness(SnesFitnessArgs a
     a.loss[k] = a.rmse[k] + a.lambda1 * (r1[0] / a.d) + a.lambda2 * sqrt(r2[0] / a.d);
 }
 
-// Ascending loss, NaN last, ties by index.
-__device__ __forceinline__ bool before(double a, int i, double b, int j) {
-  const bool na = isnan(a), nb = isnan(b);
-  if (na != nb) return nb;
-  if (!na && a != b) return a < b;
-  return i < j;
+// Orders losses ascending, NaN last, -0 = 0, as integers (a double comparison
+// holds an SM quarter's FP64 pipe for 64 cycles).
+__device__ __forceinline__ unsigned long long loss_key(double x) {
+  if (isnan(x)) return ~0ull;
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x), sign = 1ull << 63;
+  if (u == sign) return sign;  // -0 as +0
+  return u & sign ? ~u : u | sign;
+}
+// Ties by index.
+__device__ __forceinline__ bool before(unsigned long long a, int i, unsigned long long b, int j) {
+  return a != b ? a < b : i < j;
 }
 
 // Every CTA ranks the P losses itself (P <= 1024), then updates its slice of
 // the parameters; CTA 0 also writes the generation summary and advances the
 // generation counter (read only by the next generation's sampling launch).
-__global__ void __launch_bounds__(kSnesThreads) k_snes_update(SnesUpdateArgs a) {
+// Bound by FP64 issue (half a lane a clock and SM quarter): CTAs of two warps
+// spread the parameters over the chip, the losses are read once, and the
+// summary has a CTA of its own beside the others' sums (P = 50, d = 2282: 43
+// us with CTAs of 256 threads that read the losses from global memory).
+constexpr int kUpdateThreads = 64;
+__global__ void __launch_bounds__(kUpdateThreads) k_snes_update(SnesUpdateArgs a) {
   __shared__ double util[kMaxSnesPop];
   __shared__ double w[kMaxSnesPop];
+  __shared__ double loss[kMaxSnesPop];
+  __shared__ unsigned long long key[kMaxSnesPop];
   __shared__ double wsum;
   const int P = a.P;
   const double lhalf = log(P / 2.0 + 1.0);
-  for (int r = threadIdx.x; r < P; r += kSnesThreads) w[r] = fmax(0.0, lhalf - log((double)(r + 1)));
+  for (int r = threadIdx.x; r < P; r += kUpdateThreads) {
+    w[r] = fmax(0.0, lhalf - log((double)(r + 1)));
+    loss[r] = a.loss[r];
+    key[r] = loss_key(loss[r]);
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     double acc = 0.0;
@@ -141,27 +157,32 @@ __global__ void __launch_bounds__(kSnesThreads) k_snes_update(SnesUpdateArgs a) 
     wsum = acc;
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < P; k += kSnesThreads) {
-    const double lk = a.loss[k];
+  for (int k = threadIdx.x; k < P; k += kUpdateThreads) {
+    const unsigned long long lk = key[k];
     int rank = 0;
-    for (int j = 0; j < P; ++j) rank += before(a.loss[j], j, lk, k) ? 1 : 0;
+    for (int j = 0; j < P; ++j) rank += before(key[j], j, lk, k) ? 1 : 0;
     util[k] = w[rank] / wsum - 1.0 / P;
   }
   __syncthreads();
-  if (blockIdx.x == 0 && threadIdx.x == 0 && a.history) {
-    int best = 0;
-    double mean = 0.0;
-    for (int k = 0; k < P; ++k) {
-      if (before(a.loss[k], k, a.loss[best], best)) best = k;
-      mean += a.loss[k];
+  if (blockIdx.x == gridDim.x - 1) {  // a CTA of its own: the generation's summary
+    if (threadIdx.x == 0 && a.history) {
+      int best = 0;
+      double mean = 0.0;
+      for (int k = 0; k < P; ++k) {
+        if (before(key[k], k, key[best], best)) best = k;
+        mean += loss[k];
+      }
+      a.history[0] = loss[best];
+      a.history[1] = a.rmse ? a.rmse[best] : 0.0;
+      a.history[2] = mean / P;
     }
-    a.history[0] = a.loss[best];
-    a.history[1] = a.rmse ? a.rmse[best] : 0.0;
-    a.history[2] = mean / P;
+    if (threadIdx.x == 0 && a.generation) *a.generation += 1;
+    return;
   }
-  const int i = blockIdx.x * kSnesThreads + threadIdx.x;
+  const int i = blockIdx.x * kUpdateThreads + threadIdx.x;
   if (i < a.d) {
     double gm = 0.0, gs = 0.0;
+#pragma unroll 4
     for (int k = 0; k < P; ++k) {
       const double sk = a.s[(size_t)k * a.d + i];
       gm += util[k] * sk;
@@ -171,7 +192,6 @@ __global__ void __launch_bounds__(kSnesThreads) k_snes_update(SnesUpdateArgs a) 
     a.mu[i] = a.mu[i] + a.eta_mu * sg * gm;
     a.sigma[i] = sg * exp(0.5 * a.eta_sigma * gs);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && a.generation) *a.generation += 1;
 }
 
 }  // namespace
@@ -195,7 +215,7 @@ cudaError_t launch_snes_fitness(const SnesFitnessArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_snes_update(const SnesUpdateArgs& a, cudaStream_t st) {
-  k_snes_update<<<(a.d + kSnesThreads - 1) / kSnesThreads, kSnesThreads, 0, st>>>(a);
+  k_snes_update<<<(a.d + kUpdateThreads - 1) / kUpdateThreads + 1, kUpdateThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
