@@ -19,7 +19,10 @@
 // (x1 y1, x1 y2, x2 y1, x1 y3, x2 y2, x3 y1; the rest is below 2^-24).
 //
 // One CTA (128 threads) takes one tile of 5 atoms of one centre type and 25
-// individuals.  TMEM lane r = 5 p + n holds row (p, n).
+// individuals at a time.  TMEM lane r = 5 p + n holds row (p, n).  CTAs are
+// persistent (two per SM): the barriers and TMEM columns are set up once, the
+// next item's operands arrive during the last round's epilogue, and
+// the radial descriptor is formed while operands are still on their way.
 //   1. bulk copies (cp.async.bulk, mbarrier) of the coefficient tile and of
 //      the 5 atoms' B blocks; one product A for all 5 atoms (N = 128
 //      columns); lane (p, n) reads its A_{n,lm}(i) and forms q_nl and the
@@ -44,6 +47,9 @@
 // nothing.
 
 #include <cuda_bf16.h>
+
+#include <algorithm>
+#include <numeric>
 
 #include "tc_sm100.cuh"
 #include "tnep_device.cuh"
@@ -206,25 +212,10 @@ __global__ void __launch_bounds__(128, 2) k_pop_tc(const __grid_constant__ PopTc
   const uint32_t bar_r = tc::smem_addr(&bars[4]);
 
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int tile = blockIdx.x / a.n_mt, mt = blockIdx.x % a.n_mt;
-  const int* td = a.tiles + (size_t)tile * 8;
-  const int tau = td[5], count = td[6];
   const int pl = tid / 5, x = tid % 5;            // (individual, n) in phases 1 and 3; (individual, atom) in 2
-  const int p = mt * kPT + pl;
-  const bool prow = tid < kPT * 5 && p < a.n_pop;  // a real (individual, .) row
   const int T = a.n_types;
   const size_t xs = a.mom_tc_stride;
-  auto atom_of = [&](int i) { return td[i]; };      // a.n_atoms (zero block) for empty slots
-  auto x_src = [&](int i) { return a.mom_tc + (size_t)atom_of(i) * xs + kBBytes; };
-  // thread 0: bulk copies of round r's X blocks (the zero block past the tile)
-  auto load_round = [&](int r) {
-    tc::mbar_expect_tx(bar_x, AG * XB);
-    for (int ia = 0; ia < AG; ++ia) {
-      const int i = AG * r + ia;
-      tc::bulk_g2s(s_base + kOffX0 + ia * XB, i < kNT ? x_src(i) : a.mom_tc + (size_t)a.n_atoms * xs + kBBytes,
-                   XB, bar_x);
-    }
-  };
+  const int n_items = a.n_tiles * a.n_mt;
 
   // ---------------------------------------------------------------- set-up
   if (tid == 0) {
@@ -238,24 +229,72 @@ __global__ void __launch_bounds__(128, 2) k_pop_tc(const __grid_constant__ PopTc
   const uint32_t tmem = *tslot;
   const uint32_t lane_base = tmem + ((uint32_t)(32 * warp) << 16);
 
-  // what thread 0 has issued and seen complete, per barrier (for the give-up path)
+  // uses of each barrier: what thread 0 has issued and seen complete (for the
+  // waits' parities and the give-up path), and completions every thread has seen
   int n_commit = 0, x_issued = 0, x_seen = 0, r_issued = 0, r_seen = 0;
-  int load_issued = 1, load_seen = 0;  // uses of bar_load: phase 1, then phase 3
-  bool w_issued = false, w_seen = false;
+  int load_issued = 0, load_seen = 0;  // two an item: phase 1, then phase 3
+  int w_issued = 0, w_seen = 0;
+  int mma_done = 0, r_done = 0, w_done = 0;
+  bool ok = true;
   volatile int* s_flag = reinterpret_cast<volatile int*>(smem + kOffBar + 52);
-  if (tid == 0) {
+  // thread 0: bulk copies of an item's coefficient tile and B blocks
+  auto load_operands = [&](int it) {
+    const int* td = a.tiles + (size_t)(it / a.n_mt) * 8;
     tc::mbar_expect_tx(bar_load, kCoefBytes + kNT * kBBytes);
-    tc::bulk_g2s(s_base + kOffC, a.coef_tc + (size_t)(tau * a.n_mt + mt) * kCoefBytes, kCoefBytes, bar_load);
+    tc::bulk_g2s(s_base + kOffC, a.coef_tc + (size_t)(td[5] * a.n_mt + it % a.n_mt) * kCoefBytes, kCoefBytes, bar_load);
     for (int i = 0; i < kNT; ++i)
-      tc::bulk_g2s(s_base + kOffB + i * kBBytes, a.mom_tc + (size_t)atom_of(i) * xs, kBBytes, bar_load);
+      tc::bulk_g2s(s_base + kOffB + i * kBBytes, a.mom_tc + (size_t)td[i] * xs, kBBytes, bar_load);
+    ++load_issued;
+  };
+  if (tid == 0) load_operands(blockIdx.x);
+
+  // Items: (tile, individual tile), one every gridDim.x; the grid is no larger
+  // than their number.
+  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+  const int tile = item / a.n_mt, mt = item % a.n_mt;
+  const int* td = a.tiles + (size_t)tile * 8;
+  const int tau = td[5], count = td[6];
+  const int p = mt * kPT + pl;
+  const bool prow = tid < kPT * 5 && p < a.n_pop;  // a real (individual, .) row
+  const bool mine = prow && x < count;             // thread (p, atom x) of phase 2
+  auto atom_of = [&](int i) { return td[i]; };      // a.n_atoms (zero block) for empty slots
+  auto x_src = [&](int i) { return a.mom_tc + (size_t)atom_of(i) * xs + kBBytes; };
+  // thread 0: bulk copies of round r's X blocks (the zero block past the tile)
+  auto load_round = [&](int r) {
+    tc::mbar_expect_tx(bar_x, AG * XB);
+    for (int ia = 0; ia < AG; ++ia) {
+      const int i = AG * r + ia;
+      tc::bulk_g2s(s_base + kOffX0 + ia * XB, i < kNT ? x_src(i) : a.mom_tc + (size_t)a.n_atoms * xs + kBBytes,
+                   XB, bar_x);
+    }
+  };
+
+  // ---------------------------------------------------------------- 0. radial descriptor
+  // thread (p, atom x): q_n from the radial moments, while the operands arrive
+  float qr[NR];
+#pragma unroll
+  for (int n = 0; n < NR; ++n) qr[n] = 0.f;
+  if (mine) {
+    const ModelLayout& Ly = a.lay;
+    const float* cR_i = a.params + (size_t)p * Ly.words + Ly.off_cR + tau * T * Ly.stride_cR;
+    const float* mom = a.mom + atom_of(x);
+    for (int t = 0; t < T; ++t) {
+      float Fk[BR];
+#pragma unroll
+      for (int k = 0; k < BR; ++k) Fk[k] = mom[(size_t)(t * kMomBasis + k) * a.mom_stride];
+      const float* cc = cR_i + t * Ly.stride_cR;
+#pragma unroll
+      for (int n = 0; n < NR; ++n)
+#pragma unroll
+        for (int k = 0; k < BR; ++k) qr[n] += __ldg(cc + n * BR + k) * Fk[k];
+    }
   }
 
   // ---------------------------------------------------------------- 1. A for all atoms, q_nl
-  bool ok = true;
-  int mma_done = 0;  // completions of bar_mma observed by every thread
+  ok = true;
   if (tid == 0) {
-    ok = tc::mbar_wait_bounded(bar_load, 0, kTries);
-    if (ok) load_seen = 1;
+    ok = tc::mbar_wait_bounded(bar_load, load_seen & 1, kTries);
+    if (ok) ++load_seen;
     if (ok) {
       tc::fence_after_sync();
       issue_split_products(tmem, s_base + kOffC, s_base + kOffB, tc::idesc_bf16_f32(128, 128));
@@ -263,9 +302,9 @@ __global__ void __launch_bounds__(128, 2) k_pop_tc(const __grid_constant__ PopTc
       ++n_commit;
     }
   }
-  ok = __syncthreads_and(ok && tc::mbar_wait_bounded(bar_mma, 0, kTries)) != 0;
+  ok = __syncthreads_and(ok && tc::mbar_wait_bounded(bar_mma, mma_done & 1, kTries)) != 0;
   if (!ok) goto give_up;
-  mma_done = 1;
+  ++mma_done;
   // the product has read the operand buffers: stage every individual's W0
   // block over them now (one bulk copy each, issued by thread ip), to land
   // during q and 2a.  Thread 0 arms the byte count; a copy that completes
@@ -274,7 +313,7 @@ __global__ void __launch_bounds__(128, 2) k_pop_tc(const __grid_constant__ PopTc
     const int nw = min(kPT, a.n_pop - mt * kPT);
     if (tid == 0) {
       tc::mbar_expect_tx(bar_w, nw * kW0Bytes);
-      w_issued = true;
+      ++w_issued;
     }
     if (tid < nw) {
       const int net = a.lay.nets > 1 ? tau : 0;
@@ -308,26 +347,9 @@ __global__ void __launch_bounds__(128, 2) k_pop_tc(const __grid_constant__ PopTc
   // ---------------------------------------------------------------- 2. network (Eq. 1), radial part
   {
     const ModelLayout& Ly = a.lay;
-    const bool mine = prow && x < count;  // thread (p, atom x)
-    // 2a. thread (p, atom x): radial descriptor q_n from the radial moments,
-    // then the scaled descriptor s = q * q_scaler in place
+    // 2a. thread (p, atom x): the scaled descriptor s = q * q_scaler in place
     if (mine) {
       const float* model = a.params + (size_t)p * Ly.words;
-      const float* cR_i = model + Ly.off_cR + tau * T * Ly.stride_cR;
-      const float* mom = a.mom + atom_of(x);
-      float q[NR];
-#pragma unroll
-      for (int n = 0; n < NR; ++n) q[n] = 0.f;
-      for (int t = 0; t < T; ++t) {
-        float Fk[BR];
-#pragma unroll
-        for (int k = 0; k < BR; ++k) Fk[k] = mom[(size_t)(t * kMomBasis + k) * a.mom_stride];
-        const float* cc = cR_i + t * Ly.stride_cR;
-#pragma unroll
-        for (int n = 0; n < NR; ++n)
-#pragma unroll
-          for (int k = 0; k < BR; ++k) q[n] += __ldg(cc + n * BR + k) * Fk[k];
-      }
       float* qd = qbuf + (pl * kNT + x) * kQS;
       // all scaler loads first (generic stores below would otherwise order them)
       float scl[DP];
@@ -345,7 +367,7 @@ __global__ void __launch_bounds__(128, 2) k_pop_tc(const __grid_constant__ PopTc
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int d = 4 * v + u;
-          r4[u] = d < NR ? q[d < NR ? d : 0] * scl[d] : (d < 30 ? r4[u] * scl[d] : 0.f);
+          r4[u] = d < NR ? qr[d < NR ? d : 0] * scl[d] : (d < 30 ? r4[u] * scl[d] : 0.f);
         }
         q4[v] = make_float4(r4[0], r4[1], r4[2], r4[3]);
       }
@@ -366,9 +388,10 @@ __global__ void __launch_bounds__(128, 2) k_pop_tc(const __grid_constant__ PopTc
         pb0[u] = v ? __ldg(model + Ly.off_b0 + net * H + h) : 0.f;
         pw1[u] = v ? __ldg(model + Ly.off_w1 + net * H + h) : 0.f;
       }
-      const bool okw = __syncthreads_and(tc::mbar_wait_bounded(bar_w, 0, kTries)) != 0;
+      const bool okw = __syncthreads_and(tc::mbar_wait_bounded(bar_w, w_done & 1, kTries)) != 0;
       if (!okw) goto give_up;
-      if (tid == 0) w_seen = true;
+      ++w_done;
+      if (tid == 0) ++w_seen;
 #pragma unroll
       for (int u = 0; u < NPR; ++u) {
         const int r = tid + 128 * u, ip = r / 30, h = r % 30;
@@ -450,11 +473,7 @@ __global__ void __launch_bounds__(128, 2) k_pop_tc(const __grid_constant__ PopTc
     __syncthreads();
     // reload the coefficient tile and the B blocks for phase 3, and round 0's X blocks
     if (tid == 0) {
-      tc::mbar_expect_tx(bar_load, kCoefBytes + kNT * kBBytes);
-      tc::bulk_g2s(s_base + kOffC, a.coef_tc + (size_t)(tau * a.n_mt + mt) * kCoefBytes, kCoefBytes, bar_load);
-      for (int i = 0; i < kNT; ++i)
-        tc::bulk_g2s(s_base + kOffB + i * kBBytes, a.mom_tc + (size_t)atom_of(i) * xs, kBBytes, bar_load);
-      load_issued = 2;
+      load_operands(item);
       load_round(0);
       ++x_issued;
     }
@@ -507,14 +526,14 @@ __global__ void __launch_bounds__(128, 2) k_pop_tc(const __grid_constant__ PopTc
     // r's epilogue).
     bool okl = true;
     if (tid == 0) {
-      okl = tc::mbar_wait_bounded(bar_load, 1, kTries);
-      if (okl) load_seen = 2;
+      okl = tc::mbar_wait_bounded(bar_load, load_seen & 1, kTries);
+      if (okl) ++load_seen;
     }
 #pragma unroll 1
     for (int r = 0; r < NROUND; ++r) {
       bool ok0 = okl;
       if (tid == 0 && ok0) {
-        ok0 = tc::mbar_wait_bounded(bar_x, r & 1, kTries);
+        ok0 = tc::mbar_wait_bounded(bar_x, x_seen & 1, kTries);
         if (ok0) {
           ++x_seen;
           tc::fence_after_sync();
@@ -524,13 +543,16 @@ __global__ void __launch_bounds__(128, 2) k_pop_tc(const __grid_constant__ PopTc
           ++r_issued;
         }
       }
-      ok = __syncthreads_and(ok0 && tc::mbar_wait_bounded(bar_r, r & 1, kTries)) != 0;
+      ok = __syncthreads_and(ok0 && tc::mbar_wait_bounded(bar_r, r_done & 1, kTries)) != 0;
       if (!ok) goto give_up;
+      ++r_done;
       if (tid == 0) {
         ++r_seen;
         if (r + 1 < NROUND) {  // round r's products have read the buffer
           load_round(r + 1);
           ++x_issued;
+        } else if (item + (int)gridDim.x < n_items) {  // and the last round's all operands: the next item's
+          load_operands(item + gridDim.x);
         }
       }
       tc::fence_after_sync();
@@ -590,9 +612,12 @@ __global__ void __launch_bounds__(128, 2) k_pop_tc(const __grid_constant__ PopTc
           }
         }
       }
+      // the next item's weight blocks are bulk-copied (async proxy) over the n-sums
+      if (r + 1 == NROUND) tc::fence_proxy_async_smem();
       __syncthreads();  // the n-sums are read before the next round rewrites them
     }
   }
+  }  // items
   if (warp == 0) tc::tmem_dealloc(tmem, TCOLS);
   return;
 
@@ -606,10 +631,10 @@ give_up:
     if (a.status) atomicCAS(&a.status->error, 0, TNEP_ERR_TIMEOUT);
     bool drained = true;
     if (load_issued > load_seen) drained = tc::mbar_wait_bounded(bar_load, (load_issued - 1) & 1, kTries) && drained;
-    if (n_commit > mma_done) drained = tc::mbar_wait_bounded(bar_mma, 0, kTries) && drained;
+    if (n_commit > mma_done) drained = tc::mbar_wait_bounded(bar_mma, (n_commit - 1) & 1, kTries) && drained;
     if (x_issued > x_seen) drained = tc::mbar_wait_bounded(bar_x, (x_issued - 1) & 1, kTries) && drained;
     if (r_issued > r_seen) drained = tc::mbar_wait_bounded(bar_r, (r_issued - 1) & 1, kTries) && drained;
-    if (w_issued && !w_seen) drained = tc::mbar_wait_bounded(bar_w, 0, kTries) && drained;
+    if (w_issued > w_seen) drained = tc::mbar_wait_bounded(bar_w, (w_issued - 1) & 1, kTries) && drained;
     *s_flag = drained ? 1 : 0;
   }
   __syncthreads();
@@ -649,7 +674,15 @@ cudaError_t launch_pop_tc(int rank, const PopTcArgs& a, cudaStream_t st) {
   auto fn = rank == 1 ? k_pop_tc<1> : k_pop_tc<2>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
   if (e != cudaSuccess) return e;
-  fn<<<(unsigned)a.n_tiles * a.n_mt, 128, kSmemBytes, st>>>(a);
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const long long items = (long long)a.n_tiles * a.n_mt;
+  // A CTA takes every grid-th item: a grid coprime to the individual tiles gives
+  // each its share of the partly filled last one.
+  long long grid = std::min<long long>(items, 2LL * sms);
+  while (grid < items && grid > 1 && std::gcd(grid, (long long)a.n_mt) != 1) --grid;
+  fn<<<(unsigned)grid, 128, kSmemBytes, st>>>(a);
   return cudaGetLastError();
 }
 
