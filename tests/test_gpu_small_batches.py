@@ -121,3 +121,37 @@ def test_small_batch_regrows_its_lists(tn):
             assert e.value.status == 4
     for a, b in zip(*outs):
         assert np.array_equal(a[0], b[0])
+
+
+@pytest.mark.parametrize("n_types", [1, 2, 3, 4, 5])
+def test_lists_of_large_batches(tn, n_types):
+    """Beside 60,300 other atoms the lists are built by a thread per atom; the
+    same bits as alone, for lists with types missing and with few entries, and
+    the same neighbours."""
+    rng = np.random.default_rng(31)
+    structs = [water(64, rng), water(100, rng, 2)]
+    for n in (1, 2, 9):
+        p, t, b = synth.water_cluster(n, rng)
+        structs.append(synth.Structure(p.astype(np.float32), t, b.astype(np.float32)))
+    for k, s in enumerate(structs):
+        s.types = ((np.arange(len(s.types)) * 5 % 13 + k) % n_types).astype(np.int32)
+    structs[1].types[:] = n_types - 1
+    filler = water(20100, rng)
+    filler.types = (np.arange(len(filler.types)) % n_types).astype(np.int32)
+    models = []
+    for rank in (1, 2):
+        hp = synth.HyperParams(n_types=n_types, rank=rank)
+        models.append(tn.Model.from_hyper(hp, synth.model_params(hp, rng), synth.default_q_scaler(hp)))
+    small, big = synth.concat_structures(structs), synth.concat_structures(structs + [filler])
+    N = small.offsets[-1]
+    with tn.tnep_create(models, n_types, (6.0, 4.0)) as ctx:
+        o1, p1 = tn.tnep_eval_batch(ctx, small.offsets, small.pos, small.box, small.types, per_atom=True)
+        o2, p2 = tn.tnep_eval_batch(ctx, big.offsets, big.pos, big.box, big.types, per_atom=True)
+        n1 = tn.tnep_neighbors(ctx, small.offsets, small.pos, small.box)
+        n2 = tn.tnep_neighbors(ctx, big.offsets, big.pos, big.box)
+    for m in range(2):
+        assert np.array_equal(p1[m], p2[m][:N]), m
+        assert np.array_equal(o1[m], o2[m][:len(structs)]), m
+    assert np.array_equal(n1[0], n2[0][:N]) and np.array_equal(n1[1], n2[1][:N])
+    for a, b in zip(n1[2:], n2[2:]):
+        assert np.array_equal(np.sort(a, 1), np.sort(b[:N], 1))
