@@ -246,6 +246,12 @@ __global__ void __launch_bounds__(BLK, 256 / BLK) k_fused(const __grid_constant_
       }
     }
     NbrWalk wA(a.nbr_A, a.pos4, i, a.cap_A, 0, FACT ? 0 : nA, pi);
+    // Two pairs per iteration: with two warps per scheduler the walk waits on
+    // the serial recursion of one pair's basis, which the next pair's can fill
+    // (same order of the sums).  2,073,600 atoms of water, two models and the
+    // radial moments: 7,156 -> 6,904 us (split-BF16 network), 7,285 -> 7,273
+    // (FP32); three pairs spill (7,412 and 7,533).
+#pragma unroll 2
     for (int kk = 0; kk < (FACT ? 0 : nA); ++kk) {
       const float4 pj = wA.next(kk);
       const float dx = min_image(pj.x, pi.x, bx.L[0], bx.invL[0]);
