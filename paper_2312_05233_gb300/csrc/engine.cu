@@ -290,7 +290,7 @@ tnep_status ensure_lists(tnep_ctx* c, Workspace& w) {
 }
 
 // Offsets on the device for the kernels of a batch whose preparation does not
-// copy them itself (from the caller's pageable memory: the driver sends a few
+// copy them itself (from the caller's pageable memory: CUDA sends a few
 // bytes with the command, about 10 us less than a copy from pinned memory).
 tnep_status copy_offsets(Workspace& w, cudaStream_t st, int S, const int* h_offsets) {
   TNEP_CUDA(cudaMemcpyAsync(w.offsets.p, h_offsets, sizeof(int) * (S + 1), cudaMemcpyHostToDevice, st));

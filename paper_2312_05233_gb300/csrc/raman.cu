@@ -10,7 +10,7 @@
 //   N a power of two, as in the spectrum tail (X_b, F_b defined there):
 //     prep   two channels per complex value, [5 packs][T], mean removed if asked
 //     fft    5 x (number of segments) transforms of length N
-//     (T = 1e5, M = 2000, tensor and 181-angle map: 6136 -> 844 us a call;
+//     (T = 1e5, M = 2000, tensor and 181-angle map: 6136 -> 644 us a call;
 //     before, one 2^17-point transform per channel and 23 back, and 4240 us of
 //     cosine sums that divided and took a 64-bit remainder in every term)
 //     cross  for the 45 pairs p <= q, sum over the segments b of

@@ -24,7 +24,7 @@
 //
 // What bounds it: FP64 instructions (two lanes per clock and SM) and, for
 // short series, launches.  Measured on a GB300 (whole call, host series in,
-// spectrum out): T = 1e5, M = 1e4, aniso 3392 -> 419 us (before, 2487 us went
+// spectrum out): T = 1e5, M = 1e4, aniso 3392 -> 368 us (before, 2487 us went
 // to the preparation in one CTA, 310 us to 34 radix-2 passes over the whole
 // padded series and 228 us to cosine sums with a 64-bit remainder per term).
 

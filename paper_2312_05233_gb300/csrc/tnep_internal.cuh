@@ -277,8 +277,10 @@ cudaError_t launch_fused(int variant, int rank, const FusedArgs& a, int n_pop, i
 // moments in the layouts of the general path.
 constexpr int kWideModels = 4;
 // Largest batch of the warp-per-atom path.  Measured calls (two models, GB300),
-// thread / warp per atom: 11,520 atoms of water 238 / 210 us, 19,200 243 / 288 us;
-// six types, 9,696 atoms 400 / 235 us, 34,301 522 / 625 us.
+// thread / warp per atom: water, 7,680 atoms 177 / 176 us, 11,520 201 / 208,
+// 19,200 181 / 288; two to six types, 10,137 atoms of clusters 228 / 220 us, 9,696 of
+// mixed requests 224 / 227; one model of perovskite, 8,640 atoms 190 / 170 us: the
+// two forms are level around the line.
 constexpr int kWideAtoms = 12288;
 constexpr size_t kWideMaxSmem = 100 * 1024;  // two CTAs per SM
 struct WideArgs {
