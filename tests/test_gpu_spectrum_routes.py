@@ -116,3 +116,37 @@ def test_porto_map_of_any_tensor(tn, axis, n_theta):
     L[5, a * 3 + a, a * 3 + a] = np.inf
     par, _ = tn.tnep_raman_porto_map(L, th + 0.1, axis=axis)
     assert np.isnan(par[:, 3]).all() and np.isfinite(par[:, 4]).all() and np.isposinf(par[:, 5]).all()
+
+
+def tensor_reference(x, M, dt):
+    """Lineshape tensor of the mean-free x, and a bound on its rounding for each
+    component: a lag is good to 4 eps log2(2 M) of sqrt(C_pp(0) C_qq(0)) times
+    T / (T - tau) <= 2, and 2 M lags of one sign add up."""
+    T = len(x)
+    ref = np.zeros((M + 1, 9, 9))
+    for p in range(9):
+        for q in range(p, 9):
+            c = 0.5 * (correlate(x[:, p], x[:, q], M) + correlate(x[:, q], x[:, p], M))
+            ref[:, p, q] = ref[:, q, p] = cosine(c, dt)
+    size = np.sqrt((x * x).sum(0) / T)
+    return ref, 8 * np.finfo(float).eps * np.log2(2 * M) * 2 * M * dt * np.outer(size, size)
+
+
+# below and above 1e9 terms, one segment and several
+@pytest.mark.parametrize("T,M", [(5000, 1000), (3000, 1500), (20000, 3001)])
+@pytest.mark.parametrize("sub", [True, False])
+@pytest.mark.parametrize("ratio", [1e2, 1e4, 1e8])
+def test_small_tensor_components_keep_their_accuracy(tn, T, M, sub, ratio):
+    """Diagonal channels `ratio` times the others, a constant one and an empty
+    one: the error of every component is relative to its own size."""
+    rng = np.random.default_rng(T + M)
+    s = rng.standard_normal((T, 9)) + (2.0 if not sub else 300.0)
+    s[:, [0, 4, 8]] *= ratio
+    s[:, 5] = 7.0
+    s[:, 7] = 0.0
+    f, L = tn.tnep_raman_tensor(s, 2.0, M, sub)
+    x = s - s.mean(0) if sub else s
+    if sub:
+        x[:, 5] = 0.0
+    ref, tol = tensor_reference(x, M, 2.0)
+    assert np.all(np.abs(L - ref).max(0) <= tol), np.abs(L - ref).max(0) / tol
