@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kSumThreads) k_rsum(const double* __restrict__
 }
 
 // The power of two near the root mean square of x - mean over T samples (zero
-// for a channel of zeros), from the sums of k_rsum: m is the mean less what they
+// for a channel of zeros, NaN for one with a value that is not finite), from the sums of k_rsum: m is the mean less what they
 // were taken about.  The sums may cancel or leave the float range where the
 // first sample is far from the others; the largest magnitude bounds them: the
 // largest |x - mean| lies between half and twice it, the root mean square
@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(kSumThreads) k_rsum(const double* __restrict__
 // overflow or vanish.)
 __device__ __forceinline__ double channel_unit(float sq, int top, double first, double m, int T) {
   if (top == 0) return 0.0;
+  if (top >= 0x7ff00000 || !isfinite(m)) return __hiloint2double(0x7ff80000, 0);
   const int e = rough_unit(first), et = (top >> 20) - 1023;
   const float mr = rough(m, e), var = sq / (float)T - mr * mr;
   const int lo = et - 1 - (34 - __clz(T)) / 2;
@@ -191,9 +192,10 @@ __global__ void __launch_bounds__(256) k_rprep(const double* __restrict__ s, int
       if constexpr (PACK) {
         const double u = channel_unit(sq, top, s[c], subtract_mean ? m - s[c] : 0.0, T);
         unit[c] = u;
-        const double r = u == 0.0 ? 0.0 : __hiloint2double((2046 << 20) - __double2hiint(u), 0);  // 1 / u
+        // 1 / u; a channel that is zero or not finite goes in as zeros
+        const double r = u > 0.0 ? __hiloint2double((2046 << 20) - __double2hiint(u), 0) : 0.0;
         inv[c] = r;
-        mean[c] = m * r;
+        mean[c] = r > 0.0 ? m * r : 0.0;
       }
     }
   }
@@ -208,7 +210,8 @@ __global__ void __launch_bounds__(256) k_rprep(const double* __restrict__ s, int
   x[9] = 0.0;
   if constexpr (PACK) {
 #pragma unroll
-    for (int c = 0; c < 9; ++c) x[c] = fma(s[(size_t)t * 9 + c], inv[c], -mean[c]);  // (s - mean) / unit
+    for (int c = 0; c < 9; ++c)  // (s - mean) / unit
+      x[c] = inv[c] > 0.0 ? fma(s[(size_t)t * 9 + c], inv[c], -mean[c]) : 0.0;
     double2* z = reinterpret_cast<double2*>(out) + t;
 #pragma unroll
     for (int k = 0; k < kPacks; ++k) z[(size_t)k * T] = make_double2(x[2 * k], x[2 * k + 1]);
@@ -269,7 +272,9 @@ __global__ void k_rlags(const double* __restrict__ C, int T, int M, double* __re
 // multiplies the pairs back: each component of the tensor is then as accurate
 // relative to its own size as with direct sums (T = 5,000, M = 1,000, diagonal
 // channels 1e4 times the others: error of the small L_pp over dt C_pp(0) 2.3e-8
-// without, 3.2e-15 with, 9.1e-15 for the direct sums).
+// without, 3.2e-15 with, 9.1e-15 for the direct sums).  A channel with a value
+// that is not finite goes in as zeros and its pairs come out as NaN, so that it
+// does not spoil those that it shares a transform with.
 struct LoadSegment {
   static constexpr bool kHalfZero = true;
   const double2* z;

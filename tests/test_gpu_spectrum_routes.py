@@ -150,3 +150,18 @@ def test_small_tensor_components_keep_their_accuracy(tn, T, M, sub, ratio):
         x[:, 5] = 0.0
     ref, tol = tensor_reference(x, M, 2.0)
     assert np.all(np.abs(L - ref).max(0) <= tol), np.abs(L - ref).max(0) / tol
+
+
+@pytest.mark.parametrize("T,M", [(500, 200), (5000, 1000), (20000, 3001)])
+@pytest.mark.parametrize("sub", [True, False])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_a_channel_that_is_not_finite_spoils_only_its_own_pairs(tn, T, M, sub, bad):
+    s = np.random.default_rng(T).standard_normal((T, 9)) + 0.5
+    s[T // 3, 1] = bad
+    f, L = tn.tnep_raman_tensor(s, 2.0, M, sub)
+    s[T // 3, 1] = 0.0
+    ref, tol = tensor_reference(s - s.mean(0) if sub else s, M, 2.0)
+    mine = np.zeros((9, 9), bool)
+    mine[1], mine[:, 1] = True, True
+    assert not np.isfinite(L[:, mine]).any()
+    assert np.all(np.abs(L - ref).max(0)[~mine] <= tol[~mine])
