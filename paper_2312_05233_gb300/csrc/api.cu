@@ -107,7 +107,7 @@ tnep_status tnep_create(const tnep_model_desc* models, int n_models, int n_types
     c->models.push_back(std::move(m));
     if (e != cudaSuccess) return bail(cuda_fail(e, "model upload"));
     if (fused_smem_bytes(c->models.back().variant, c->models.back().lay, kFusedBlockMax,
-                         c->models.back().d.mlp_precision) > 227 * 1024)
+                         c->models.back().d.mlp_precision) > kFusedMaxSmem)
       return bail(fail(TNEP_ERR_UNSUPPORTED, "model too large for shared memory"));
   }
   *out = c;

@@ -809,7 +809,8 @@ cudaError_t launch_block(int rank, const FusedArgs& a_in, int n_pop, size_t smem
   if (n_work > INT_MAX) return cudaErrorInvalidConfiguration;
   auto fn = rank == 1 ? k_fused<NR, NA, BR, BA, LMAX, FB, 1, BLK, TCM, FACT, PC>
                       : k_fused<NR, NA, BR, BA, LMAX, FB, 2, BLK, TCM, FACT, PC>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the largest size of any model: another host thread's context may set and launch in between
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedMaxSmem);
   if (e != cudaSuccess) return e;
   dim3 grid;
   if constexpr (TCM != 0) {

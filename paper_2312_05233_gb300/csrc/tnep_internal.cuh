@@ -268,6 +268,7 @@ int variant_of(int nR, int nA, int bR, int bA, int lmax, int fb);
 // tcm: network products on the CUDA cores in FP32 (0), on the tensor cores
 // with BF16 operands and FP32 accumulation (1), or on the tensor cores with
 // split high/low BF16 operands, three products (2); 1 and 2 use 128 atoms per CTA.
+constexpr size_t kFusedMaxSmem = 227 * 1024;  // larger models are refused by tnep_create
 size_t fused_smem_bytes(int variant, const ModelLayout& lay, int block, int tcm);
 cudaError_t launch_fused(int variant, int rank, const FusedArgs& a, int n_pop, int block, int tcm, cudaStream_t st);
 

@@ -668,7 +668,8 @@ __global__ void __launch_bounds__(32 * kWarps) k_wide(const __grid_constant__ Wi
 template <int NR, int NA, int BR, int BA, int LMAX, bool FUSED>
 cudaError_t launch_one(const WideArgs& a, int smem, cudaStream_t st) {
   auto fn = k_wide<NR, NA, BR, BA, LMAX, FUSED>;
-  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // the largest size of any call: another host thread's context may set and launch in between
+  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideMaxSmem);
   if (e != cudaSuccess) return e;
   count_launches(1);
   fn<<<(a.n_active + kWarps - 1) / kWarps, 32 * kWarps, smem, st>>>(a);
