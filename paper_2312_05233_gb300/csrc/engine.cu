@@ -626,9 +626,15 @@ tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N,
     const bool use_pc = c->pair_cache && pc_elems * sizeof(float4) <= kPairCacheMaxBytes;
     // Batches of a few waves: every other model on a side stream (with a pair
     // cache and a work counter of its own), so that one model's CTAs fill the
-    // slots the other leaves.
-    const bool fork = run.size() > 1 && N <= kForkAtoms;
-    if (use_pc) TNEP_CUDA(w.pcache.ensure(pc_elems * (fork ? 2 : 1)));
+    // slots the other leaves.  One stream where the second cache would go beyond
+    // the bound or does not fit in memory.
+    bool fork = run.size() > 1 && N <= kForkAtoms &&
+                (!use_pc || 2 * pc_elems * sizeof(float4) <= kPairCacheMaxBytes);
+    if (use_pc) TNEP_CUDA(w.pcache.ensure(pc_elems));
+    if (use_pc && fork && w.pcache_side.ensure(pc_elems) != cudaSuccess) {
+      cudaGetLastError();
+      fork = false;
+    }
     if (fork) TNEP_TRY(fork_side(w, st));
     cudaError_t e = cudaSuccess;
     for (size_t r = 0; r < run.size() && e == cudaSuccess; ++r) {
@@ -638,7 +644,7 @@ tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N,
       FusedArgs f = fused_args(c, w, m, N);
       f.per_atom = w.per_atom.p + k * per_model;
       f.per_atom_stride = 0;
-      f.pcache = use_pc ? w.pcache.p + side * pc_elems : nullptr;
+      f.pcache = !use_pc ? nullptr : side ? w.pcache_side.p : w.pcache.p;
       f.pc_stride = stride_of(m);
       f.work_next += side;
       e = launch_fused(m.variant, m.d.rank, f, 1, c->block_atoms, m.d.mlp_precision, side ? w.side : st);

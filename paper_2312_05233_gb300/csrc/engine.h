@@ -113,6 +113,7 @@ struct Workspace {
   DevBuf<int> nbr_tmp, seg_R, struct_flags;
   DevBuf<float> mom;        // radial moments [slots][atom_stride]
   DevBuf<float4> pcache;    // per-pair cache of the angular walk (see FusedArgs)
+  DevBuf<float4> pcache_side;  // that of the models on `side`
   DevBuf<int> red_offsets;  // structure offsets of the pass whose sums run on the side stream
   int mom_v0 = -1, mom_w0 = -1;
   DevBuf<float4> pos4;
@@ -148,7 +149,7 @@ struct Workspace {
                     &types_stage, &nbr_tmp, &seg_R, &struct_flags})
       b->release();
     pos4.release(); grids.release(); boxes.release(); per_atom.release(); out.release(); partial.release();
-    mom.release(); pcache.release(); red_offsets.release();
+    mom.release(); pcache.release(); pcache_side.release(); red_offsets.release();
     pos_stage[0].release(); pos_stage[1].release(); box_stage.release();
     if (d_status) cudaFree(d_status);
     d_status = nullptr;

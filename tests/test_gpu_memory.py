@@ -1,0 +1,59 @@
+"""Device memory of calls whose models run on two streams."""
+
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+N_MOL = 40000
+# What one atom of a two-type batch takes with lists of 128 and 64 entries: lists
+# with a scratch copy, moments, one pair cache of 64 x 64 bytes, outputs of two
+# models, cells and orders; buffers are allocated a quarter larger.
+ATOM_BYTES = (2 * 128 + 64) * 4 + 2 * 9 * 10 * 4 + 64 * 64 + 2 * 9 * 4 + 128
+ONE_CACHE = int(1.25 * 3 * N_MOL * ATOM_BYTES)
+SECOND_CACHE = int(1.25 * 3 * N_MOL * 64 * 64)
+SLACK = 128 << 20  # roundings of the allocator, code
+
+
+@pytest.fixture(scope="module")
+def tn():
+    from paper_2312_05233_gb300 import tnep
+    return tnep
+
+
+@pytest.fixture(scope="module")
+def structure():
+    rng = np.random.default_rng(41)
+    p, t, b = synth.water_box(N_MOL, rng)
+    return np.mod(p, b).astype(np.float32), t.astype(np.int32), b.astype(np.float32)
+
+
+def context(tn):
+    rng = np.random.default_rng(42)
+    models = []
+    for rank in (1, 2):
+        hp = synth.HyperParams(n_types=2, rank=rank)
+        models.append(tn.Model.from_hyper(hp, synth.model_params(hp, rng), synth.default_q_scaler(hp)))
+    return tn.tnep_create(models, 2, (6.0, 4.0))
+
+
+def test_a_second_pair_cache_that_does_not_fit_is_left_out(tn, structure):
+    """With room for one pair cache only, the models run one after the other:
+    the same bits as with room for two."""
+    import torch
+    pos, types, box = structure
+    with context(tn) as ctx:
+        ref = tn.tnep_eval(ctx, pos[None], box, types)
+    torch.cuda.empty_cache()
+    with context(tn) as ctx:
+        room = ONE_CACHE + SLACK + SECOND_CACHE // 4
+        hold = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+        try:
+            got = tn.tnep_eval(ctx, pos[None], box, types)
+        finally:
+            del hold
+            torch.cuda.empty_cache()
+    for a, b in zip(ref, got):
+        assert np.array_equal(a, b)
