@@ -628,7 +628,7 @@ tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N,
     // cache and a work counter of its own), so that one model's CTAs fill the
     // slots the other leaves.  One stream where the second cache would go beyond
     // the bound or does not fit in memory.
-    bool fork = run.size() > 1 && N <= kForkAtoms &&
+    bool fork = run.size() > 1 && N <= kForkAtoms && !w.one_stream &&
                 (!use_pc || 2 * pc_elems * sizeof(float4) <= kPairCacheMaxBytes);
     if (use_pc) TNEP_CUDA(w.pcache.ensure(pc_elems));
     if (use_pc && fork && w.pcache_side.ensure(pc_elems) != cudaSuccess) {

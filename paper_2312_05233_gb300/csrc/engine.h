@@ -134,7 +134,10 @@ struct Workspace {
   PinBuf<float> h_box;
   cudaEvent_t ev_pin = nullptr;
   bool pin_read = false;
-  // every other model of a small batch runs on `side`, between two events
+  // Every other model of a small batch runs on `side`, between two events,
+  // unless one_stream: a server's batches, whose admitted memory has no second
+  // pair cache and whose pipelines overlap each other.
+  bool one_stream = false;
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int atom_stride = 0;

@@ -291,6 +291,7 @@ tnep_status tnep_server_start(tnep_ctx* ctx, size_t mem_budget_bytes, int max_sl
   s->max_batch_atoms = max_batch_atoms;
   for (int k = 0; k < n_pipelines; ++k) {
     auto p = std::make_unique<Pipeline>();
+    p->ws.one_stream = true;
     cudaError_t e = cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->done_ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = dev_malloc(reinterpret_cast<void**>(&p->ws.d_status), sizeof(DevStatus));

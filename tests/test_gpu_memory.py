@@ -39,6 +39,26 @@ def context(tn):
     return tn.tnep_create(models, 2, (6.0, 4.0))
 
 
+def test_served_batches_stay_within_their_estimate(tn, structure):
+    """120,000 atoms through the server take the memory of one pair cache, which
+    is what the admission counts, and give the bits of the plain call."""
+    import torch
+    pos, types, box = structure
+    with context(tn) as ctx:
+        tn.tnep_eval(ctx, pos[None, :192], np.float32([30, 30, 30]), types[:192])  # loads the kernels
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        with tn.tnep_server_start(ctx, mem_budget_bytes=4 << 30, max_batch_atoms=len(types), n_pipelines=1) as srv:
+            ticket = srv.submit(pos, types, box)
+            counted = srv.stats()["bytes_in_use"]
+            out, _ = srv.wait(ticket)
+            used = before - torch.cuda.mem_get_info()[0]
+        plain = tn.tnep_eval(ctx, pos[None], box, types)
+    assert np.array_equal(out, np.concatenate([plain[0][0], plain[1][0]]))
+    assert used <= ONE_CACHE + SLACK < ONE_CACHE + SECOND_CACHE
+    assert counted == 0 or counted >= 0.9 * 3 * N_MOL * ATOM_BYTES
+
+
 def test_a_second_pair_cache_that_does_not_fit_is_left_out(tn, structure):
     """With room for one pair cache only, the models run one after the other:
     the same bits as with room for two."""
