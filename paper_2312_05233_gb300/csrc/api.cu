@@ -252,6 +252,15 @@ tnep_status tnep_eval(tnep_ctx* c, int n_frames, int n_atoms, const float* pos, 
   if (!out_dev) TNEP_CUDA(c->h_out.ensure((size_t)n_frames * Ctot));
   std::vector<int> offs(fb + 1);
   const cudaStream_t red = n_frames > fb ? c->red_stream : nullptr;
+  // An early return leaves no pass behind that writes `out` or the workspace
+  // (a call of one pass does not wait for red_stream).
+  struct Drain {
+    cudaStream_t st, red;
+    ~Drain() {
+      if (red) cudaStreamSynchronize(red);
+      if (st) cudaStreamSynchronize(st);
+    }
+  } drain{st, red};
   // Verlet-skin reuse needs one box for the whole pass and n_atoms > 0; any
   // violation found on the device (displacement above skin / 2, changed box,
   // box too small for the enlarged cutoff) redoes the call with fresh lists
@@ -326,6 +335,7 @@ tnep_status tnep_eval(tnep_ctx* c, int n_frames, int n_atoms, const float* pos, 
     }
     if (!regrow) {
       c->last_skin_used = use_skin ? 1 : 0;
+      drain = {nullptr, nullptr};  // finish has waited
       if (!out_dev) std::memcpy(out, c->h_out.p, sizeof(double) * (size_t)n_frames * Ctot);
       return TNEP_OK;
     }
