@@ -113,7 +113,11 @@ tnep_status tnep_create(const tnep_model_desc* models, int n_models, int n_types
                         const char* const* type_names, const float cutoffs[2], int device,
                         tnep_ctx** out);
 
-/* Frees every resource of the context (NULL is a no-op). */
+/* Frees every resource of the context.  The scratch of tnep_spectrum, the
+ * tnep_raman calls and tnep_eval_batch_cell comes from a pool of the library that
+ * keeps up to 256 MB per device between calls; it is given back with the last
+ * context, or, in a program without contexts, by tnep_destroy(NULL) (which does
+ * nothing else, and nothing at all while contexts exist). */
 void tnep_destroy(tnep_ctx* ctx);
 
 /* Thread-local message describing the last failed call on this thread. */

@@ -115,7 +115,10 @@ tnep_status tnep_create(const tnep_model_desc* models, int n_models, int n_types
 }
 
 void tnep_destroy(tnep_ctx* c) {
-  if (!c) return;
+  if (!c) {
+    if (g_contexts.load() == 0) trim_pools();
+    return;
+  }
   cudaSetDevice(c->device);
   if (c->stream) cudaStreamSynchronize(c->stream);
   if (c->copy_stream) cudaStreamSynchronize(c->copy_stream);

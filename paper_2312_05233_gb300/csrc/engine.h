@@ -40,8 +40,10 @@ cudaError_t dev_malloc(void** p, size_t bytes);
 // Stream-ordered scratch of one call, from a pool of this library per device
 // that keeps up to kPoolKeepBytes between calls (the runtime's default pool
 // gives everything back at each synchronisation, and mapping it again cost
-// about 200 us a call); freed with cudaFreeAsync.  The pool is trimmed when an
-// allocation does not fit and when the last context goes.
+// about 200 us a call); freed with cudaFreeAsync.  A pool gives what it keeps to
+// its own larger allocations; it is trimmed when another one of the library
+// (dev_malloc) does not fit, when the last context goes, and by
+// tnep_destroy(NULL) where there is none.
 constexpr size_t kPoolKeepBytes = size_t(256) << 20;
 cudaError_t dev_malloc_async(void** p, size_t bytes, cudaStream_t st);
 void trim_pools();

@@ -1,4 +1,8 @@
-"""Device memory of calls whose models run on two streams."""
+"""Device memory: models on two streams, scratch kept between calls."""
+
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -7,6 +11,7 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 N_MOL = 40000
 # What one atom of a two-type batch takes with lists of 128 and 64 entries: lists
 # with a scratch copy, moments, one pair cache of 64 x 64 bytes, outputs of two
@@ -77,3 +82,39 @@ def test_a_second_pair_cache_that_does_not_fit_is_left_out(tn, structure):
             torch.cuda.empty_cache()
     for a, b in zip(ref, got):
         assert np.array_equal(a, b)
+
+
+KEPT = """
+import numpy as np, torch, synth
+from paper_2312_05233_gb300 import tnep as tn
+series = np.random.default_rng(43).standard_normal((250_000, 9))  # about 105 MB of scratch
+hp = synth.HyperParams(n_types=2, rank=1)
+model = tn.Model.from_hyper(hp, synth.model_params(hp, np.random.default_rng(1)), synth.default_q_scaler(hp))
+
+def spectrum():
+    tn.tnep_spectrum(series, 0.5, tn.TNEP_SPECTRUM_RAMAN_ANISO, 10_000)
+
+def held():
+    return free - torch.cuda.mem_get_info()[0]
+
+free = 0
+spectrum()
+tn.lib().tnep_destroy(None)
+free = torch.cuda.mem_get_info()[0]
+spectrum()
+assert 64 << 20 < held() <= 256 << 20, held()
+tn.lib().tnep_destroy(None)
+assert held() <= 4 << 20, held()
+with tn.tnep_create([model], 2, (6.0, 4.0)):  # with a context it stays until the last one goes
+    spectrum()
+    tn.lib().tnep_destroy(None)
+    assert held() >= 64 << 20, held()
+assert held() <= 4 << 20, held()
+"""
+
+
+def test_kept_scratch_is_given_back_without_a_context():
+    """A program that only computes spectra has no context whose end gives the
+    kept scratch back (in a process of its own: no context of another test)."""
+    r = subprocess.run([sys.executable, "-c", KEPT], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
