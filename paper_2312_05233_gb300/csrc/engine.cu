@@ -306,7 +306,8 @@ tnep_status build_lists(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, const
   w.wide = wide_atoms > 0 && wide_atoms <= kWideAtoms && !spec &&
            wide_smem_bytes(c->n_types, w.cap_R, w.cap_A) <= kWideMaxSmem;
   if (!w.wide) TNEP_TRY(ensure_lists(c, w));
-  if (w.max_atoms > kSmallStruct) {
+  const bool by_cta = prepared_by_cta(S, N, w.max_atoms, c->sms);
+  if (!by_cta) {
     TNEP_TRY(copy_offsets(w, st, S, h_offsets));
     TNEP_CUDA(cudaMemsetAsync(w.cell_count.p, 0, sizeof(int) * (w.cells_cap + 1), st));
     TNEP_CUDA(cudaMemsetAsync(w.struct_flags.p, 0, sizeof(int) * S, st));
@@ -315,6 +316,7 @@ tnep_status build_lists(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, const
   a.n_structs = S;
   a.n_atoms = N;
   a.max_struct = w.max_atoms;
+  a.by_cta = by_cta;
   a.offsets = w.offsets.p;
   a.src_offsets = w.h_offsets.p;
   a.offsets_out = w.offsets.p;

@@ -19,6 +19,8 @@
 //           warp-tiled.
 // Pair selection follows the exact float32 recipe documented in tnep.h.
 
+#include <algorithm>
+
 #include "nbr_device.cuh"
 #include "tnep_internal.cuh"
 
@@ -26,7 +28,7 @@ namespace tnep {
 
 namespace {
 
-constexpr int kSmallThreads = 1024;  // 256 for structures of at most 1024 atoms
+constexpr int kSmallThreads = 1024;
 // Largest batch of k_build_group, up to two types and more.  Measured neighbour
 // pipelines (GB300), group / thread: water 15,360 atoms 35 / 51 us, 28,800 51 / 55,
 // 41,472 in one box 118 / 125, 76,800 91 / 64; three types, 17,280 atoms 79 / 120, 69,120
@@ -287,6 +289,8 @@ __global__ void k_cell_sort(NbrArgs a, int* sorted_cell) {
 // general pipeline.
 // Dynamic shared memory: 4 n + 9 ints (counts / starts of up to 2 n + 8 cells,
 // then per atom its cell and slot, and the atoms by cell), n = max_struct.
+inline int small_smem_bytes(int max_struct) { return (int)sizeof(int) * (4 * max_struct + 9); }
+inline int small_threads(int max_struct) { return max_struct <= 1024 ? 256 : kSmallThreads; }
 constexpr int kSlotBits = 14;
 static_assert(kSmallStruct < (1 << kSlotBits) && 2 * kSmallStruct + 8 < (1 << (31 - kSlotBits)), "cell and slot share a word");
 
@@ -1008,16 +1012,31 @@ __global__ void k_export(int n, const int* sorted_orig, const int* nbr_R, const 
 
 }  // namespace
 
+// Every CTA of k_prep_small has the shared memory and threads of the largest
+// structure, so beside a large one thousands of small structures run in waves of
+// nearly idle CTAs, about 3 us each.  Beyond eight waves more than the atoms fill
+// the general pipeline is faster.  Neighbour pipelines (GB300), one CTA a
+// structure / general: a box of 13,800 atoms and 300 molecules of 40 atoms 74 / 77 us,
+// 1,000 137 / 139, 3,000 219 / 172, 10,000 506 / 284; a box of 3,000 atoms and 3,000
+// molecules 149 / 152, 10,000 330 / 258; a box of 1,020 atoms (256 threads) and 10,000
+// molecules 185 / 267; 300 boxes of 13,824 atoms 3,377 / 3,480.
+bool prepared_by_cta(int n_structs, int n_atoms, int max_struct, int sms) {
+  if (max_struct > kSmallStruct) return false;
+  if (small_threads(max_struct) < kSmallThreads) return true;
+  const int resident = std::min(2048 / kSmallThreads, (227 << 10) / (small_smem_bytes(max_struct) + 1024));
+  return n_structs - n_atoms / max_struct <= 8 * resident * sms;
+}
+
 cudaError_t launch_neighbor_pipeline(const NbrArgs& a, bool build, cudaStream_t st) {
   const int S = a.n_structs, N = a.n_atoms;
   if (S <= 0) return cudaSuccess;
-  if (a.max_struct <= kSmallStruct) {
-    const int smem = (int)sizeof(int) * (4 * a.max_struct + 9);
+  if (a.by_cta) {
+    const int smem = small_smem_bytes(a.max_struct);
     const cudaError_t e = cudaFuncSetAttribute(k_prep_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)sizeof(int) * (4 * kSmallStruct + 9));
+                                               small_smem_bytes(kSmallStruct));
     if (e != cudaSuccess) return e;
     count_launches(1);
-    k_prep_small<<<S, a.max_struct <= 1024 ? 256 : kSmallThreads, smem, st>>>(a, a.atom_slot);
+    k_prep_small<<<S, small_threads(a.max_struct), smem, st>>>(a, a.atom_slot);
   } else {
     count_launches(6);
     k_plan<<<S, 256, 0, st>>>(a);

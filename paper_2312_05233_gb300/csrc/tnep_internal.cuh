@@ -50,14 +50,18 @@ __host__ __device__ __forceinline__ size_t nbr_index(int i, int k, int cap) {
   return ((size_t)(i >> 5) * cap + k) * 32 + (i & 31);
 }
 
-// Arguments of the neighbour-list pipeline.
-// Structures up to this size are prepared by one CTA each (nbr.cu): their cells
+// Structures up to this size may be prepared by one CTA each (nbr.cu): their cells
 // and atoms take 224 of the 227 KB of shared memory.
 constexpr int kSmallStruct = 14000;
+// Whether the structures of a batch (the largest of max_struct atoms) are.
+bool prepared_by_cta(int n_structs, int n_atoms, int max_struct, int sms);
+
+// Arguments of the neighbour-list pipeline.
 struct NbrArgs {
   int n_structs;
   int n_atoms;
   int max_struct;           // largest structure
+  bool by_cta;              // one CTA prepares each structure (prepared_by_cta)
   const int* offsets;       // [S+1] device
   const int* src_offsets;   // [S+1] pinned host copy (small structures: read by the device)
   int* offsets_out;         // device array the small-structure kernel copies them to

@@ -155,3 +155,26 @@ def test_lists_of_large_batches(tn, n_types):
     assert np.array_equal(n1[0], n2[0][:N]) and np.array_equal(n1[1], n2[1][:N])
     for a, b in zip(n1[2:], n2[2:]):
         assert np.array_equal(np.sort(a, 1), np.sort(b[:N], 1))
+
+
+def test_uneven_batches_are_not_prepared_at_the_largest_size(tn):
+    """Thousands of small structures beside a larger one leave the preparation by
+    one CTA each (six launches more), with the same bits as alone."""
+    rng = np.random.default_rng(37)
+    structs = [water(400, rng)]
+    for k in range(5000):
+        n = 1 + k % 3
+        p = 1.5 * np.arange(3 * n).reshape(n, 3) * rng.uniform(0.5, 1, (n, 3))
+        structs.append(synth.Structure(p.astype(np.float32), (np.arange(n) % 2).astype(np.int32),
+                                       np.zeros(3, np.float32)))
+    few, all_ = synth.concat_structures(structs[:50]), synth.concat_structures(structs)
+    with context(tn, 2, 0) as ctx:
+        launches, outs = [], []
+        for bt in (few, all_):
+            n0 = tn.tnep_get_option(ctx, tn.TNEP_OPT_KERNEL_LAUNCHES_TOTAL)
+            outs.append(tn.tnep_eval_batch(ctx, bt.offsets, bt.pos, bt.box, bt.types, per_atom=True))
+            launches.append(tn.tnep_get_option(ctx, tn.TNEP_OPT_KERNEL_LAUNCHES_TOTAL) - n0)
+    for m in range(2):
+        assert np.array_equal(outs[0][0][m], outs[1][0][m][:50])
+        assert np.array_equal(outs[0][1][m], outs[1][1][m][:few.offsets[-1]])
+    assert launches[1] == launches[0] + 5
