@@ -316,6 +316,7 @@ tnep_status build_lists(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, const
   a.n_structs = S;
   a.n_atoms = N;
   a.max_struct = w.max_atoms;
+  a.sms = c->sms;
   a.by_cta = by_cta;
   a.offsets = w.offsets.p;
   a.src_offsets = w.h_offsets.p;

@@ -232,14 +232,42 @@ __global__ void k_bin(NbrArgs a) {
   a.atom_slot[g] = atomicAdd(&a.cell_count[cell], 1);
 }
 
-// One CTA per structure: its cells hold its atoms, so their starts follow from
-// the structure's first atom (one CTA over all cells: 79 us for 50 frames of
+// Every structure's cells hold its atoms, so their starts follow from the
+// structure's first atom (one CTA over all cells: 79 us for 50 frames of
 // 41,472 atoms).  The entry after the last cell is the next structure's first,
-// which both CTAs write with the same value.
+// which both write with the same value.  A CTA takes every gridDim.x-th
+// structure: a warp scans each small one, then the whole CTA each of the others
+// (a CTA for every structure: 284 us instead of 246 for the neighbour pipeline of
+// a box of 13,800 atoms and 10,000 molecules).
+constexpr int kWarpCells = 512;
 __global__ void __launch_bounds__(1024) k_scan_cells(NbrArgs a) {
-  const int s = blockIdx.x;
-  const int c0 = min(a.struct_cells[s], a.cells_cap), c1 = min(a.struct_cells[s + 1], a.cells_cap);
-  block_exclusive_scan(a.cell_count + c0, a.cell_start + c0, c1 - c0, a.offsets[s]);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, step = gridDim.x;
+  auto cells = [&](int s, int& c0) {
+    c0 = min(a.struct_cells[s], a.cells_cap);
+    return min(a.struct_cells[s + 1], a.cells_cap) - c0;
+  };
+  for (long long s = blockIdx.x + (long long)warp * step; s < a.n_structs; s += (long long)(blockDim.x >> 5) * step) {
+    int c0;
+    const int n = cells((int)s, c0);
+    if (n > kWarpCells) continue;
+    int run = a.offsets[s];
+    for (int base = 0; base <= n; base += 32) {
+      const int c = base + lane, v = c < n ? a.cell_count[c0 + c] : 0;
+      int incl = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+      }
+      if (c <= n) a.cell_start[c0 + c] = run + incl - v;
+      run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+  }
+  for (long long s = blockIdx.x; s < a.n_structs; s += step) {
+    int c0;
+    const int n = cells((int)s, c0);
+    if (n > kWarpCells) block_exclusive_scan(a.cell_count + c0, a.cell_start + c0, n, a.offsets[s]);
+  }
 }
 
 __global__ void k_scatter(NbrArgs a) {
@@ -1016,10 +1044,10 @@ __global__ void k_export(int n, const int* sorted_orig, const int* nbr_R, const 
 // structure, so beside a large one thousands of small structures run in waves of
 // nearly idle CTAs, about 3 us each.  Beyond eight waves more than the atoms fill
 // the general pipeline is faster.  Neighbour pipelines (GB300), one CTA a
-// structure / general: a box of 13,800 atoms and 300 molecules of 40 atoms 74 / 77 us,
-// 1,000 137 / 139, 3,000 219 / 172, 10,000 506 / 284; a box of 3,000 atoms and 3,000
-// molecules 149 / 152, 10,000 330 / 258; a box of 1,020 atoms (256 threads) and 10,000
-// molecules 185 / 267; 300 boxes of 13,824 atoms 3,377 / 3,480.
+// structure / general: a box of 13,800 atoms and 300 molecules of 40 atoms 74 / 72 us,
+// 1,000 137 / 138, 3,000 219 / 164, 10,000 506 / 246; a box of 3,000 atoms and 1,000
+// molecules 100 / 119, 3,000 149 / 142, 10,000 330 / 223; a box of 1,020 atoms (256
+// threads) and 10,000 molecules 185 / 230; 300 boxes of 13,824 atoms 3,377 / 3,479.
 bool prepared_by_cta(int n_structs, int n_atoms, int max_struct, int sms) {
   if (max_struct > kSmallStruct) return false;
   if (small_threads(max_struct) < kSmallThreads) return true;
@@ -1044,7 +1072,7 @@ cudaError_t launch_neighbor_pipeline(const NbrArgs& a, bool build, cudaStream_t 
     // The number of cells in use is known only on the device; the cell scan
     // and the per-cell sort read it from struct_cells[S].
     k_bin<<<(N + 255) / 256, 256, 0, st>>>(a);
-    k_scan_cells<<<S, 1024, 0, st>>>(a);
+    k_scan_cells<<<std::min(S, 2 * a.sms), 1024, 0, st>>>(a);
     k_scatter<<<(N + 255) / 256, 256, 0, st>>>(a);
     // sorted_cell reuses atom_slot (dead after the scatter)
     k_cell_sort<<<1216, 256, 0, st>>>(a, a.atom_slot);

@@ -61,6 +61,7 @@ struct NbrArgs {
   int n_structs;
   int n_atoms;
   int max_struct;           // largest structure
+  int sms;                  // SMs of the device
   bool by_cta;              // one CTA prepares each structure (prepared_by_cta)
   const int* offsets;       // [S+1] device
   const int* src_offsets;   // [S+1] pinned host copy (small structures: read by the device)
