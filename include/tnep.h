@@ -430,7 +430,9 @@ enum {
   TNEP_OPT_LAST_KERNEL_MS = 3,      /* read-only: device time of the tensor kernels (radial moments + fused) of the last call (ms) */
   TNEP_OPT_CELL_DIV = 4,            /* cells of edge rc_R / k with a +-k stencil, k in {1, 2, 3}; stencil cells
                                        farther than the cutoff are skipped (default 1) */
-  TNEP_OPT_LAST_KERNEL_LAUNCHES = 5,/* read-only: fused-kernel launches in the last call */
+  TNEP_OPT_LAST_KERNEL_LAUNCHES = 5,/* read-only: launches of the kernels that evaluate models in the last call:
+                                       per pass one per model, or, for FP32-network models of a pass of at most
+                                       12,288 atoms, one per four models of the same descriptor sizes */
   TNEP_OPT_LAST_NBR_MS = 6,         /* read-only: device time of the cell/neighbour pipeline in the last call (ms) */
   TNEP_OPT_KERNEL_LAUNCHES_TOTAL = 7,/* read-only: kernels launched by this library in this process */
   TNEP_OPT_SKIN = 8,                /* Verlet skin (A) for tnep_eval, default 0.  With a skin s > 0 each pass of

@@ -511,7 +511,7 @@ tnep_status sum_pass_times(tnep_ctx* c, int n_pass) {
   }
   c->last_nbr_ms = nbr;
   c->last_kernel_ms = fused;
-  c->last_launches = n_pass * (int)c->models.size();
+  c->last_launches = c->ws.model_launches;
   return TNEP_OK;
 }
 
@@ -537,6 +537,7 @@ static tnep_status run_wide(tnep_ctx* c, Workspace& w, cudaStream_t st, const Im
     for (size_t k = 0; k <= c->models.size(); ++k) {
       if (a.n_models == kWideModels || (k == c->models.size() && a.n_models > 0)) {
         TNEP_CUDA(launch_wide(variant, true, a, st));
+        if (a.n_active > 0) ++w.model_launches;
         a.n_models = 0;
       }
       if (k == c->models.size()) break;
@@ -651,6 +652,7 @@ tnep_status run_models(tnep_ctx* c, Workspace& w, cudaStream_t st, int S, int N,
       f.pc_stride = stride_of(m);
       f.work_next += side;
       e = launch_fused(m.variant, m.d.rank, f, 1, c->block_atoms, m.d.mlp_precision, side ? w.side : st);
+      if (N > 0) ++w.model_launches;
     }
     if (fork) TNEP_TRY(join_side(w, st));  // also after a failed launch: nothing is left behind on the side stream
     TNEP_CUDA(e);
@@ -701,6 +703,7 @@ tnep_status check_status(tnep_ctx* c, const DevStatus& s, bool* regrow) {
 
 tnep_status reset_status(Workspace& w, cudaStream_t st) {
   TNEP_CUDA(cudaMemsetAsync(w.d_status, 0, sizeof(DevStatus), st));
+  w.model_launches = 0;
   return TNEP_OK;
 }
 

@@ -148,6 +148,7 @@ struct Workspace {
   int two_ended = 0;         // radial list layout of the last build (see NbrArgs)
   bool wide = false;         // the batch is prepared for one warp per atom (no lists built yet)
   NbrArgs prepared{};        // its arguments
+  int model_launches = 0;    // kernels that evaluated models since reset_status
   void release() {
     for (auto* b : {&offsets, &atom_struct, &atom_cell, &atom_slot, &cell_count, &cell_start, &cell_atoms,
                     &sorted_orig, &orig_sorted, &sorted_struct, &struct_cells, &cnt_R, &cnt_A, &nbr_R, &nbr_A,

@@ -178,3 +178,22 @@ def test_uneven_batches_are_not_prepared_at_the_largest_size(tn):
         assert np.array_equal(outs[0][0][m], outs[1][0][m][:50])
         assert np.array_equal(outs[0][1][m], outs[1][1][m][:few.offsets[-1]])
     assert launches[1] == launches[0] + 5
+
+
+@pytest.mark.parametrize("n_mol,precisions,frames,launches",
+                         [(64, (0, 0), 1, 1), (64, (0,) * 5, 1, 2), (64, (2, 2), 1, 2), (64, (0, 2), 1, 2),
+                          (4400, (0, 0), 1, 2), (64, (0, 0), 3, 3), (4400, (0, 2), 3, 6)])
+def test_model_launches_are_counted(tn, n_mol, precisions, frames, launches):
+    """TNEP_OPT_LAST_KERNEL_LAUNCHES: one launch takes up to four FP32 models of a
+    small batch, otherwise each model has its own; three passes of one frame."""
+    rng = np.random.default_rng(41)
+    s = water(n_mol, rng)
+    models = []
+    for k, precision in enumerate(precisions):
+        hp = synth.HyperParams(n_types=2, rank=1 + k % 2)
+        models.append(tn.Model.from_hyper(hp, synth.model_params(hp, rng), synth.default_q_scaler(hp),
+                                          mlp_precision=precision))
+    with tn.tnep_create(models, 2, (6.0, 4.0)) as ctx:
+        tn.tnep_set_option(ctx, tn.TNEP_OPT_FRAMES_PER_BATCH, 1)
+        tn.tnep_eval(ctx, np.repeat(s.pos[None], frames, 0), s.box, s.types)
+        assert tn.tnep_get_option(ctx, tn.TNEP_OPT_LAST_KERNEL_LAUNCHES) == launches
