@@ -89,6 +89,19 @@ __device__ __forceinline__ void image_range(double s, double delta, int& lo, int
   hi = (int)ceil(1.0 + delta - s) - 1;
 }
 
+// Images of an atom, itself left out, and no more than the host refuses (a
+// minute cell may have beyond 2^31); none where a coordinate is not finite.
+__device__ __forceinline__ int image_count(const double* sf, const double* delta) {
+  if (!isfinite(sf[0]) || !isfinite(sf[1]) || !isfinite(sf[2])) return 0;
+  long long all = 1;
+  for (int a = 0; a < 3; ++a) {
+    int lo, hi;
+    image_range(sf[a], delta[a], lo, hi);
+    all = min(all * max((long long)hi - lo + 1, 0ll), (long long)kMaxBatchAtoms + 1);
+  }
+  return (int)max(all - 1, 0ll);
+}
+
 // One CTA per structure: its plan, and per atom the first of its images among
 // the structure's (exclusive scan of the image counts in atom order);
 // n_ghost[s] is their sum.
@@ -98,7 +111,7 @@ __global__ void __launch_bounds__(kExpandThreads) k_cell_count(const int* __rest
                                                                CellInfo* __restrict__ info, int* __restrict__ first,
                                                                int* __restrict__ atom_struct,
                                                                int* __restrict__ n_ghost, DevStatus* status) {
-  __shared__ int warp_sums[kExpandThreads / 32];
+  __shared__ long long warp_sums[kExpandThreads / 32];
   __shared__ CellInfo ci_sh;
   const int s = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int a0 = off[s], a1 = off[s + 1], n = a1 - a0;
@@ -108,41 +121,35 @@ __global__ void __launch_bounds__(kExpandThreads) k_cell_count(const int* __rest
   }
   __syncthreads();
   const CellInfo ci = ci_sh;
-  int carry = 0;
+  long long carry = 0;
   for (int c0 = 0; c0 < n; c0 += kExpandThreads) {
     const int k = c0 + threadIdx.x;
     int cnt = 0;
     if (k < n && ci.periodic) {
       double sf[3];
       frac_of(ci, pos + 3 * (size_t)(a0 + k), sf);
-      cnt = 1;
-      for (int a = 0; a < 3; ++a) {
-        int lo, hi;
-        image_range(sf[a], ci.delta[a], lo, hi);
-        cnt *= hi - lo + 1;
-      }
-      --cnt;  // n = 0 is the atom itself
+      cnt = image_count(sf, ci.delta);
     }
-    int incl = cnt;
+    long long incl = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      const long long v = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += v;
     }
     if (lane == 31) warp_sums[w] = incl;
     __syncthreads();
-    int before = carry;
+    long long before = carry;
     for (int u = 0; u < kExpandThreads / 32; ++u) {
       if (u < w) before += warp_sums[u];
       carry += warp_sums[u];
     }
     if (k < n) {
-      first[a0 + k] = before + incl - cnt;
+      first[a0 + k] = (int)(before + incl - cnt);  // (not read where the batch is refused)
       atom_struct[a0 + k] = s;
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) n_ghost[s] = carry;
+  if (threadIdx.x == 0) n_ghost[s] = (int)min(carry, (long long)kMaxBatchAtoms);
 }
 
 // One warp per atom: the wrapped atom at its own place (the structure's atoms
@@ -179,10 +186,10 @@ __global__ void __launch_bounds__(128) k_cell_expand(int N, const int* __restric
   }
   int lo[3], hi[3];
   for (int d = 0; d < 3; ++d) image_range(sf[d], ci.delta[d], lo[d], hi[d]);
-  const int w1 = hi[1] - lo[1] + 1, w2 = hi[2] - lo[2] + 1, all = (hi[0] - lo[0] + 1) * w1 * w2;
+  const int w1 = hi[1] - lo[1] + 1, w2 = hi[2] - lo[2] + 1, count = image_count(sf, ci.delta);
   const int zero = (-lo[0] * w1 - lo[1]) * w2 - lo[2];  // the atom itself
   const int g0 = o0 + n + first[a];
-  for (int e = lane; e < all - 1; e += 32) {
+  for (int e = lane; e < count; e += 32) {
     const int x = e < zero ? e : e + 1;
     const int n0 = lo[0] + x / (w1 * w2), n1 = lo[1] + x / w2 % w1, n2 = lo[2] + x % w2;
     const double f0 = sf[0] + n0, f1 = sf[1] + n1, f2 = sf[2] + n2;

@@ -135,3 +135,32 @@ def test_rotated_periodic_cell_is_covariant(tn, setup):
     mu0, al0 = a[0][0], a[1][0].reshape(3, 3)
     np.testing.assert_allclose(b[0][0], R @ mu0, rtol=0, atol=1e-4 * np.abs(mu0).max())
     np.testing.assert_allclose(b[1][0].reshape(3, 3), R @ al0 @ R.T, rtol=0, atol=1e-4 * np.abs(al0).max())
+
+
+def test_minute_cells_are_refused(tn, setup):
+    """Cells whose image count per atom passes 2^31 (three axes of about 1,600
+    images and more) are refused like any expansion beyond 2^29 atoms."""
+    ctx, _ = setup
+    for edge in (0.0140, 0.0074, 0.00738, 0.0073, 0.004):
+        with pytest.raises(tn.TnepError) as e:
+            tn.tnep_eval_batch_cell(ctx, [0, 1], np.zeros((1, 3), np.float32),
+                                    (edge * np.eye(3)).reshape(1, 9).astype(np.float32), np.zeros(1, np.int32))
+        assert e.value.status == tn.TNEP_ERR_INVALID
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_a_coordinate_that_is_not_finite_leaves_the_other_cells_alone(tn, setup, bad):
+    """It has no images; the other structures of the batch keep their bits."""
+    ctx, _ = setup
+    structs = [s for s in _structures() if s[2] is not None][:2]
+    lone = (np.full((1, 3), bad), np.zeros(1, np.int32), 9.0 * np.eye(3))
+    order = [structs[0], lone, structs[1], lone]
+
+    def run(batch):
+        offsets = np.concatenate([[0], np.cumsum([len(s[1]) for s in batch])]).astype(np.int32)
+        return tn.tnep_eval_batch_cell(ctx, offsets, np.concatenate([s[0] for s in batch]).astype(np.float32),
+                                       np.stack([np.reshape(s[2], 9) for s in batch]).astype(np.float32),
+                                       np.concatenate([s[1] for s in batch]).astype(np.int32))
+    alone, mixed = run(structs), run(order)
+    for a, b in zip(alone, mixed):
+        assert np.array_equal(a, b[[0, 2]])
