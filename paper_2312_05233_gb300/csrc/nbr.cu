@@ -83,7 +83,7 @@ __device__ bool plan_structure(const NbrArgs& a, int s, int a0, int a1, StructGr
     const float em = d == 0 ? edge_min_x : edge_min;
     if (L[d] > 0.0f) {
       if (L[d] < 2.0f * a.rc_R) raise_error(a.status, TNEP_ERR_BOX_TOO_SMALL, s);
-      nc[d] = max(1, (int)floorf(L[d] / em));
+      nc[d] = max(1, min(1 << 20, (int)floorf(L[d] / em)));  // (the product below fits 64 bits)
       ext[d] = L[d];
     } else if (L[d] < 0.0f || isnan(L[d])) {
       raise_error(a.status, TNEP_ERR_INVALID, s);
@@ -333,13 +333,6 @@ __global__ void __launch_bounds__(kSmallThreads) k_prep_small(NbrArgs a, int* __
     StructBox B;
     if (plan_structure(a, s, a0, a1, G, B)) {
       G.cell_offset = 2 * a0 + 9 * s;
-      // the plan keeps to 2 n + 8 cells; an absurd box (infinite edges) may not
-      const int most = 2 * n + 8;
-      if (G.nc[0] < 1 || G.nc[1] < 1 || G.nc[2] < 1 || G.nc[0] > most || G.nc[1] > most || G.nc[2] > most ||
-          (long long)G.nc[0] * G.nc[1] * G.nc[2] > most) {
-        raise_error(a.status, TNEP_ERR_INVALID, s);
-        G.nc[0] = G.nc[1] = G.nc[2] = 1;
-      }
       Gs = G;
       a.grids[s] = G;
       a.boxes[s] = B;

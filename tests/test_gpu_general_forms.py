@@ -109,3 +109,23 @@ def test_pair_cache_and_cta_sizes_of_large_batches(tn, mode, n_mol, drop, small,
         for m in range(2):
             assert np.array_equal(tensors[m], outs[0][0][m]), (form, m)
             assert np.array_equal(atoms[m], outs[0][1][m]), (form, m)
+
+
+@pytest.mark.parametrize("edges", [(6e9, 6e9, 6e9), (3e9, 5e9, 7e10), (1e12, 20.0, 1e12), (1e30, 1e30, 1e30)])
+def test_huge_boxes_have_the_pairs_of_open_axes(tn, layouts, edges):
+    """More cells along an axis than an int holds: the plan keeps to 2 n + 8 cells
+    in both preparations."""
+    rng = np.random.default_rng(9)
+    pos = rng.uniform(0.0, 18.0, (300, 3)).astype(np.float32)
+    box = np.float32(edges)
+    short = np.where(box < 100.0, box, 0.0).astype(np.float32)  # the axis that does wrap
+    want = [oracle.neighbours_fp32(pos, short, rc) for rc in RC]
+    hp = synth.HyperParams(n_types=2, rank=1)
+    model = tn.Model.from_hyper(hp, synth.model_params(hp, rng), synth.default_q_scaler(hp))
+    for beside in ([], [layouts[2]]):
+        bt = synth.concat_structures([synth.Structure(pos, np.zeros(300, np.int32), box)] + beside)
+        with tn.tnep_create([model], 2, RC) as ctx:
+            cR, cA, lR, lA = tn.tnep_neighbors(ctx, bt.offsets, bt.pos, bt.box, cap_R=256, cap_A=128)
+        for a in range(300):
+            assert np.array_equal(np.sort(lR[a, :cR[a]]), want[0][a])
+            assert np.array_equal(np.sort(lA[a, :cA[a]]), want[1][a])
