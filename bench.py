@@ -410,19 +410,19 @@ def raman_bench(tn, synth, T=100_000, M=2000, n_theta=181):
     """Polarized Raman tail at the BaZrO3 production length: a synthetic
     susceptibility trajectory of 100,000 samples (500 ps at 5 fs), lineshape
     tensor up to 10 ps lag, then the Z(XX)Z-bar / Z(XY)Z-bar orientation map
-    for 181 crystal angles about z.  Wall time of the synchronous calls,
-    host series in, host spectra out."""
+    for 181 crystal angles about z.  Wall time of the synchronous calls, each
+    after one of the same size, host series in, host spectra out."""
     a = synth.tensor_series(T, np.random.default_rng(synth.seed_for(7, 5)))
-    tn.tnep_raman_tensor(a[:4000], 5.0, 100)  # warm-up
+    th = np.linspace(0.0, np.pi, n_theta)
+    tn.tnep_raman_porto_map(tn.tnep_raman_tensor(a, 5.0, M)[1], th, 2)  # warm-up
     t0 = time.perf_counter()
     _, L = tn.tnep_raman_tensor(a, 5.0, M)
     t1 = time.perf_counter()
-    th = np.linspace(0.0, np.pi, n_theta)
     tn.tnep_raman_porto_map(L, th, 2)
     t2 = time.perf_counter()
     return {"workload": f"susceptibility series T = {T} (500 ps at 5 fs), M = {M} lags, {n_theta} angles",
             "tensor_ms": (t1 - t0) * 1e3, "porto_map_ms": (t2 - t1) * 1e3,
-            "route": "fourier" if 81.0 * T * (M + 1) > 1.0e9 else "direct"}
+            "route": "fourier" if 81.0 * T * (M + 1) > (2.0e7 if M <= T // 2 else 1.0e9) else "direct"}
 
 
 def precision_report(tn, synth, device, pool, n_frames=500, oracle_frames=(0, 1)):

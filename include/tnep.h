@@ -315,9 +315,11 @@ enum {
  *   series   [T][C] (host or device), C = 3 (IR) or 9 (Raman)
  *   freq_cm1 [M+1] frequencies in cm^-1, spec [M+1] (host or device)
  *   acf_out  NULL or [M+1] the autocorrelation itself
- * Once channels x T x (M+1) exceeds 1e9 (channels: IR 3, iso 1, aniso 9) the
- * autocorrelation is taken through a float64 FFT of the zero-padded series
- * (length a power of two >= T + M); it equals the direct sums to rounding. */
+ * Once channels x T x (M+1) exceeds 2e7 and M <= T/2, or 1e9 otherwise (channels:
+ * IR 3, iso 1, aniso 9), the autocorrelation is taken through float64 FFTs of
+ * zero-padded segments of the series (length a power of two >= 2 M, at least
+ * 256), and for M above 4000 the cosine transform through FFTs as well; both
+ * equal the direct sums to rounding. */
 tnep_status tnep_spectrum(const double* series, int T, int C, double dt_fs, int kind,
                           int max_lag, int subtract_mean, double* freq_cm1, double* spec,
                           double* acf_out, void* stream);
@@ -377,7 +379,13 @@ void tnep_server_stop(tnep_server* server);
  * nu_k = k / (2 M dt), M = max_lag (<= 0: T/2), 0 < M < T.
  *   series   [T][9] float64 alpha(t) or chi(t), row-major 3x3 (host or device)
  *   freq_cm1 [M+1], L [M+1][9][9] (host or device).  Synchronous.
- * Cost: 81 T (M+1) float64 multiply-adds (direct time-origin sums). */
+ * Cost: 81 T (M+1) float64 multiply-adds (direct time-origin sums) up to 2e7 of
+ * them (1e9 where M > T/2); beyond, float64 FFTs of zero-padded segments, about
+ * 5 transforms forward per segment and 23 back.  The channels are scaled to like
+ * size (exactly, by powers of two) before they share a transform, so a component
+ * is as accurate relative to its own size on either route; where a component of
+ * the series holds a NaN or an infinity, its row and column of L are not finite
+ * and the others are as without it. */
 tnep_status tnep_raman_tensor(const double* series, int T, double dt_fs, int max_lag, int subtract_mean,
                               double* freq_cm1, double* L, void* stream);
 /* Eq. 7 for n_orient pairs of polarization vectors: n, eps [n_orient][3]
@@ -408,7 +416,7 @@ tnep_status tnep_raman_porto_map(const double* L, int max_lag, int n_theta, cons
  *   (or NULL) must be device memory; arguments and results are as in
  *   tnep_spectrum.  T <= TNEP_NOALLOC_MAX_T, else TNEP_ERR_INVALID.
  * Scratch lives in one file-scope device array of about 3 MB
- * ((12 * TNEP_NOALLOC_MAX_T) doubles) that every GPU which loads the library
+ * ((12 * TNEP_NOALLOC_MAX_T + 2048) doubles) that every GPU which loads the library
  * holds until the process exits.  The first call on a device looks up that
  * device's address of the array (once per device); make that first call
  * before any stream capture.  The call is asynchronous on `stream`: results
@@ -426,14 +434,19 @@ enum {
   TNEP_OPT_FRAMES_PER_BATCH = 0,    /* frames per device pass in tnep_eval (0 = automatic) */
   TNEP_OPT_MAX_NEIGHBORS = 1,       /* hard cap on neighbours per atom (default 1024); lists grow up to it */
   TNEP_OPT_BLOCK_ATOMS = 2,         /* atoms per CTA of the fused kernel: 64 or 128 (default 128); models whose
-                                       network runs on the tensor cores always take 128 (one per product row) */
-  TNEP_OPT_LAST_KERNEL_MS = 3,      /* read-only: device time of the tensor kernels (radial moments + fused) of the last call (ms) */
+                                       network runs on the tensor cores always take 128 (one per product row).
+                                       FP32-network models of passes of at most 12,288 atoms take one warp per
+                                       atom instead, whatever this and TNEP_OPT_PAIR_CACHE say */
+  TNEP_OPT_LAST_KERNEL_MS = 3,      /* read-only: device time of the tensor kernels (radial moments + fused) of the
+                                       last call (ms); passes of at most 12,288 atoms build their neighbour lists
+                                       in these kernels, so the time of the lists is here too */
   TNEP_OPT_CELL_DIV = 4,            /* cells of edge rc_R / k with a +-k stencil, k in {1, 2, 3}; stencil cells
                                        farther than the cutoff are skipped (default 1) */
   TNEP_OPT_LAST_KERNEL_LAUNCHES = 5,/* read-only: launches of the kernels that evaluate models in the last call:
                                        per pass one per model, or, for FP32-network models of a pass of at most
                                        12,288 atoms, one per four models of the same descriptor sizes */
-  TNEP_OPT_LAST_NBR_MS = 6,         /* read-only: device time of the cell/neighbour pipeline in the last call (ms) */
+  TNEP_OPT_LAST_NBR_MS = 6,         /* read-only: device time of the cell/neighbour pipeline in the last call (ms);
+                                       without the lists of passes of at most 12,288 atoms (see LAST_KERNEL_MS) */
   TNEP_OPT_KERNEL_LAUNCHES_TOTAL = 7,/* read-only: kernels launched by this library in this process */
   TNEP_OPT_SKIN = 8,                /* Verlet skin (A) for tnep_eval, default 0.  With a skin s > 0 each pass of
                                        frames builds lists with cutoffs + s for its first frame and re-tests those
@@ -457,7 +470,9 @@ enum {
                                        process so far.  Host-side fault injection: with the environment variable
                                        TNEP_FAULT=oom@N set before the library is loaded, allocation number N
                                        fails once (nothing is allocated, the device is untouched) and the call
-                                       making it returns TNEP_ERR_OOM; the context stays usable. */
+                                       making it returns TNEP_ERR_OOM; the context stays usable.  (Only the
+                                       second pair cache of a batch, see PAIR_CACHE, is optional: the call then
+                                       goes on without it.) */
   TNEP_OPT_WAIT_TRIES = 13,         /* try_wait limit of the device-side waits for the tensor-core network's
                                        products (default 4194304).  A CTA whose wait runs out stores nothing,
                                        waits (with the default limit) for its product to finish, frees its tensor
@@ -465,9 +480,13 @@ enum {
                                        wait give up at once (used to test that path).  The context stays usable. */
   TNEP_OPT_PAIR_CACHE = 14          /* 1 (default): the fused kernel's forward walk over the angular list stores
                                        each pair's r_ij, 1/|r_ij|, g_n and g_n' (64 bytes for the standard sizes)
-                                       in a device buffer of cap_A x 64 bytes per atom that its backward walk
-                                       reads back; 0: the backward walk recomputes them.  Results are the same
-                                       either way (bit for bit); skipped where the buffer would exceed 16 GB. */
+                                       in a device buffer of cap_A x 64 bytes per atom (with the tensor-core
+                                       network, per resident thread) that its backward walk reads back; 0: the
+                                       backward walk recomputes them.  Results are the same either way (bit for
+                                       bit); skipped where the buffer would exceed 16 GB.  Batches of up to
+                                       131,072 atoms with two such models or more (not those of one warp per
+                                       atom) take a second one and run their models on two streams, where both
+                                       fit in that bound and in memory; the batches of a server do not. */
 };
 tnep_status tnep_set_option(tnep_ctx* ctx, int option, double value);
 tnep_status tnep_get_option(const tnep_ctx* ctx, int option, double* value);

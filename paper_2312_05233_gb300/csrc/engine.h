@@ -35,7 +35,8 @@ tnep_status cuda_fail(cudaError_t e, const char* what);
 // with the environment variable TNEP_FAULT=oom@N set when the library loads,
 // the N-th allocation fails once with cudaErrorMemoryAllocation (nothing is
 // allocated and the device is not touched), so callers can check that every
-// entry point returns TNEP_ERR_OOM and that the context stays usable.
+// entry point returns TNEP_ERR_OOM and that the context stays usable (only
+// Workspace::pcache_side is optional: the call goes on without it).
 cudaError_t dev_malloc(void** p, size_t bytes);
 // Stream-ordered scratch of one call, from a pool of this library per device
 // that keeps up to kPoolKeepBytes between calls (the runtime's default pool

@@ -1,6 +1,7 @@
 // Polarized Raman tail in float64 (Sec. II.G, Eqs. 7-8).
 //
-//   sums   partial column sums of alpha(t) (or chi(t)), a fixed grid
+//   sums   partial column sums of alpha(t) (or chi(t)), a fixed grid; for the
+//          Fourier route also each channel's size
 //   direct route (short series):
 //     prep   x [9][T] channel-major, mean removed if asked
 //     corr   C_pq(tau) = sum_t x_p(t) x_q(t + tau), all 81 ordered pairs; one
@@ -8,14 +9,16 @@
 //     lags   S_pq(tau) = (C_pq + C_qp) / (2 (T - tau)), sequence-major
 //   Fourier route (rule at raman_uses_fft): segments of L = N/2 >= M samples,
 //   N a power of two, as in the spectrum tail (X_b, F_b defined there):
-//     prep   two channels per complex value, [5 packs][T], mean removed if asked
+//     prep   two channels per complex value, [5 packs][T], mean removed if asked,
+//            each divided by a power of two near its size
 //     fft    5 x (number of segments) transforms of length N
 //     (T = 1e5, M = 2000, tensor and 181-angle map: 6136 -> 644 us a call;
 //     before, one 2^17-point transform per channel and 23 back, and 4240 us of
 //     cosine sums that divided and took a 64-bit remainder in every term)
 //     cross  for the 45 pairs p <= q, sum over the segments b of
 //            conj(X_p) F_q + conj(X_q) F_p
-//     ifft   23 transforms, two pairs each; the real sequences are S_pq(tau)
+//     ifft   23 transforms, two pairs each; the real sequences are S_pq(tau),
+//            multiplied back by the pair's powers of two
 //   cos    L_pq(nu_k) = dt [S_pq(0) + 2 sum_tau S_pq(tau) cos(pi k tau / M)]
 //          (spectrum.cu)
 //   polar  spec_o(nu_k) = sum_pq w_p w_q L_pq(nu_k), w = vec(n_o eps_o^T) (Eq. 7)
