@@ -17,9 +17,9 @@
 //
 // Bound by latency for a few hundred atoms (one frame of 64 water molecules, two
 // models: the kernel 34 us, the call 284 -> 113 us) and by issue slots beyond: 6,660
-// warp instructions per atom (lists 1,330, radial 1,480, per model 1,930), against
-// about 625 for a thread per atom with all lanes busy, so it is taken up to
-// kWideAtoms (the rule is there).
+// warp instructions per atom in boxes of 192 atoms (lists 1,330, radial 1,480, per
+// model 1,930; 7,390 in one box of 10,137 atoms), against about 625 for a thread per
+// atom with all lanes busy, so it is taken up to kWideAtoms (the rule is there).
 //
 // FUSED = false writes the angular lists and the radial moments in the layouts
 // of the general path instead (tensor-core network: its products need 128 atoms
