@@ -415,6 +415,9 @@ __global__ void __launch_bounds__(kSmallThreads) k_prep_small(NbrArgs a, int* __
 // periodic axes list every cell once and leave the shift to rint (flagged by
 // the return value < 0).
 // `off` receives each stencil cell's offset from the centre cell before wrapping.
+// The same cells in the same order as Stencil (nbr_device.cuh), which computes
+// them instead of keeping arrays; with it k_build takes 72 registers instead of
+// 64 (lists of 2,073,600 water atoms 1,581 -> 1,639 us), so it has this form.
 __device__ __forceinline__ int axis_stencil(int c, int nc, float L, int k, int* cell, float* sh, int* unit,
                                             int* off) {
   int n = 0;

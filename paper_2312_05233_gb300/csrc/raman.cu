@@ -12,7 +12,7 @@
 //     prep   two channels per complex value, [5 packs][T], mean removed if asked,
 //            each divided by a power of two near its size
 //     fft    5 x (number of segments) transforms of length N
-//     (T = 1e5, M = 2000, tensor and 181-angle map: 6136 -> 644 us a call;
+//     (T = 1e5, M = 2000, tensor and 181-angle map: 6181 -> 659 us a call;
 //     before, one 2^17-point transform per channel and 23 back, and 4240 us of
 //     cosine sums that divided and took a 64-bit remainder in every term)
 //     cross  for the 45 pairs p <= q, sum over the segments b of
